@@ -68,6 +68,7 @@ qcad_status autotune(qcad_mesh_s* m, const qcad_bias* b, int precision, int* var
       cfg.by = r;
       cfg.kchunk = ch;
       cfg.variant = variant;
+      cfg.fit = false;
       auto run = [&]() {
         if (precision == 0) {
           ApplyArgs<double> a{};
@@ -138,6 +139,7 @@ static int tune_batch_kchunk(qcad_mesh_s* m) {
     cfg.by = 8;
     cfg.kchunk = ch;
     cfg.variant = 3;
+    cfg.fit = false;
     ApplyArgs<float> a{};
     a.v = v.as<float>();
     a.y = y.as<float>();

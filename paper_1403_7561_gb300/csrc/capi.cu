@@ -297,6 +297,7 @@ qcad_status qcad_set_launch(qcad_mesh_t m, int family, int variant, int tile_row
     c.by = tile_rows;
     c.kchunk = z_chunk;
     c.variant = (family == 1 && variant == 1) ? 0 : variant;
+    c.fit = false;
     if (family == 0)
       m->cfg_res = c;
     else if (family == 1)

@@ -31,10 +31,42 @@ static void lin_launch(const Grid<T>& g, const Op& op, int kchunk, cudaStream_t 
   note_launch(), lin_march_kernel<T, BY, R, Op><<<grid, dim3(32, BY), S::dyn_bytes, s>>>(g, op, kchunk);
 }
 
+// Default launch shapes fitted to the grid. A march block runs one node plane after the other, so
+// its time is its planes; a fixed chunk of 16 planes left most SMs idle on small grids (6 blocks of
+// 16 planes on 17 x 17 x 33 nodes: 223 us per FP64 apply) and half of the last wave on others.
+// FP32 is bound by the latency of a plane: slots are resident blocks, 2 per SM at 8 warps and two
+// rows. FP64 is bound by the SM's FP64 pipe, which all resident blocks share: one slot per SM, the
+// cost of a plane is its rows, and smaller tiles (more halo, but more SMs at work) compete.
+template <class T>
+static LaunchCfg fit_lin(int nxn, int nyn, int nzn, int nvec, LaunchCfg cfg) {
+  if (!cfg.fit || cfg.variant < 2) return cfg;
+  constexpr bool F32 = std::is_same<T, float>::value;
+  const long long tx = (long long)((nxn + 29) / 30) * nvec;
+  const long long slots = (F32 ? 2LL : 1LL) * sm_count();
+  const double over = F32 ? 3.0 : 2.0;
+  auto tiles = [&](int tr) { return tx * ((nyn + tr - 3) / (tr - 2)); };
+  static const int shape[3][2] = {{8, 2}, {4, 2}, {4, 1}};  // warps, rows per thread; FP32: the first
+  double best = FIT_GAIN * 16 * march_planes(tiles(16), nzn, slots, over, cfg.kchunk);
+  LaunchCfg out = cfg;
+  for (int h = 0; h < (F32 ? 1 : 3); ++h) {
+    const int tr = shape[h][0] * shape[h][1];
+    double cost;
+    const int kc = fit_chunk(tiles(tr), nzn, slots, over, 32, &cost);
+    if (cost * tr < best) {
+      best = cost * tr;
+      out.by = shape[h][0];
+      out.variant = shape[h][1] == 2 ? 3 : 2;
+      out.kchunk = kc;
+    }
+  }
+  return out;
+}
+
 // Supported (warps, rows per thread): FP32 4/8/16/32 x 1 and 4/8/16 x 2; FP64 4/8 x 1 and
 // 4/8 x 2 (shared memory). Other requests are clamped to the nearest supported shape.
 template <class T, class Op>
 static void run_lin(const Grid<T>& g, const Op& op, LaunchCfg cfg, cudaStream_t s) {
+  cfg = fit_lin<T>(g.nxn, g.nyn, g.nzn, 1, cfg);
   const int kc = cfg.kchunk > 0 ? (cfg.kchunk < 128 ? cfg.kchunk : 128) : 16;  // LinShape::ZMAX
   const bool two = cfg.variant == 3;
   if constexpr (std::is_same<T, float>::value) {
@@ -289,7 +321,13 @@ void launch_hm_apply_lin(const Grid<T>& g, const HmArgs<T>& args, LaunchCfg cfg,
   HmLinOp<T> op = {};
   op.a = args;
   op.mscale = (T)args.mscale;
+  cfg = fit_lin<T>(g.nxn, g.nyn, g.nzn, args.nvec, cfg);
   const int kc = cfg.kchunk > 0 ? (cfg.kchunk < 128 ? cfg.kchunk : 128) : 16;
+  if constexpr (std::is_same<T, double>::value) {
+    if (cfg.by == 4 && cfg.variant == 3)
+      return lin_launch_vec<T, 4, 2>(g, op, kc, args.nvec, s);
+    if (cfg.by == 4) return lin_launch_vec<T, 4, 1>(g, op, kc, args.nvec, s);
+  }
   if (cfg.variant == 3)
     lin_launch_vec<T, 8, 2>(g, op, kc, args.nvec, s);
   else
@@ -341,7 +379,8 @@ struct ChebHmOp {
 void launch_cheb_hm_step(const Grid<float>& g, const ChebHmArgs& args, cudaStream_t s) {
   ChebHmOp op = {};
   op.a = args;
-  lin_launch_vec<float, 8, 2>(g, op, 16, args.nvec, s);
+  lin_launch_vec<float, 8, 2>(g, op, fit_lin<float>(g.nxn, g.nyn, g.nzn, args.nvec, LaunchCfg()).kchunk, args.nvec,
+                              s);
 }
 
 void launch_hm_apply_df(const Grid<dfl>& g, const HmArgs<double>& args, cudaStream_t s) {
@@ -352,7 +391,7 @@ void launch_hm_apply_df(const Grid<dfl>& g, const HmArgs<double>& args, cudaStre
   op.cV = args.cV;
   op.ld = args.ld;
   op.mscale = dfl(args.mscale);
-  lin_launch_vec<dfl, 8, 2>(g, op, 16, args.nvec, s);
+  lin_launch_vec<dfl, 8, 2>(g, op, fit_lin<float>(g.nxn, g.nyn, g.nzn, args.nvec, LaunchCfg()).kchunk, args.nvec, s);
 }
 
 // Batched PCG apply: a work table maps each block to (instance, tile) of instances of different

@@ -130,6 +130,38 @@ struct ResidualOp {
 };
 
 
+int sm_count() {
+  static int n[64] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 152;
+  if (n[dev] == 0) {
+    int v = 0;
+    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v < 1) v = 152;
+    n[dev] = v;
+  }
+  return n[dev];
+}
+
+// Default shapes of the FP64 element-gather march fitted to the grid: its planes are bound by the
+// SM's FP64 pipe, so a block's time is its rows x planes, and small grids want smaller tiles and
+// chunks on all SMs (17 x 17 x 33 nodes: 6 blocks of 16 rows x 16 planes took 136 us).
+static LaunchCfg fit_march64(int nxn, int nyn, int nzn, LaunchCfg cfg) {
+  if (!cfg.fit) return cfg;
+  auto tiles = [&](int by) { return (long long)((nxn + 29) / 30) * ((nyn + by - 3) / (by - 2)); };
+  double best = FIT_GAIN * cfg.by * march_planes(tiles(cfg.by), nzn, sm_count(), 1.5, cfg.kchunk);
+  LaunchCfg out = cfg;
+  for (int by = 16; by >= 4; by /= 2) {
+    double cost;
+    const int kc = fit_chunk(tiles(by), nzn, sm_count(), 1.5, 32, &cost);
+    if (cost * by < best) {
+      best = cost * by;
+      out.by = by;
+      out.kchunk = kc;
+    }
+  }
+  return out;
+}
+
 template <class T, class Op>
 static void run_march(const Grid<T>& g, const Op& op, LaunchCfg cfg, cudaStream_t s, int nvec = 1) {
   switch (cfg.by) {
@@ -442,6 +474,7 @@ void launch_residual_2pass(const Grid<double>& g, const ResidualArgs& args, doub
   const ResidualGatherOp op = make_gather_op(args, elR, elD);
   LaunchCfg c = cfg;
   if (c.by == 32) c.by = 16;
+  if (face == nullptr) c = fit_march64(g.nxn, g.nyn, g.nzn, c);
   if (args.bsurf != nullptr) {
     SurfaceGatherOp sop;
     static_cast<ResidualGatherOp&>(sop) = op;

@@ -90,7 +90,45 @@ struct LaunchCfg {
   int by = 8;
   int kchunk = 16;
   int variant = 3;
+  bool fit = true;  // the shape is a default: the launch fits it to the grid (fit_march); a shape
+                    // set or autotuned for the mesh runs as given
 };
+
+// Planes that a march's SMs (or resident slots) run one after the other with z chunk c: a block takes
+// its planes + `over` (what it does before its first output plane), `tiles` blocks per chunk. The
+// blocks of full chunks come first, in waves of `slots`; those of the last, shorter chunk fill the
+// slots that the last wave leaves free.
+inline double march_planes(long long tiles, int nzn, long long slots, double over, int c) {
+  const long long full = tiles * (nzn / c);
+  const int r = nzn % c;
+  const double tf = c + over, tr = r + over;
+  const long long rest = full % slots;
+  double t = (double)(full / slots) * tf;
+  long long part = r ? tiles : 0;
+  if (rest > 0) {
+    t += tf;
+    if (part > 0) part = part > (slots - rest) * (long long)(tf / tr) ? part - (slots - rest) * (long long)(tf / tr) : 0;
+  }
+  return t + (double)((part + slots - 1) / slots) * tr;
+}
+// The z chunk (up to kmax) with the fewest; *cost receives the count.
+inline int fit_chunk(long long tiles, int nzn, long long slots, double over, int kmax, double* cost) {
+  int best = 1;
+  *cost = 1e300;
+  for (int c = 1; c <= kmax && c <= nzn; ++c) {
+    const double t = march_planes(tiles, nzn, slots, over, c);
+    if (t < *cost) {
+      *cost = t;
+      best = c;
+    }
+  }
+  return best;
+}
+// A fitted shape replaces the default only where the model promises this much: on grids of several
+// waves the model's differences are below what it resolves (fitted shapes without this margin were
+// 1 to 3 % slower there).
+constexpr double FIT_GAIN = 0.8;
+int sm_count();  // of the current device (cached)
 
 void launch_residual(const Grid<double>& g, const ResidualArgs& a, LaunchCfg cfg, cudaStream_t s);
 // Adds the electron count of the elements [box0, box1) x [box2, box3) x [box4, box5) to *out.
