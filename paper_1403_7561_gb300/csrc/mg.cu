@@ -25,7 +25,7 @@ struct MgLevel {
   long long n = 0, ne = 0;
   std::vector<double> xs[3];  // node coordinates along x, y, z
   DevBuf mask;
-  DevBuf A[2], dinv[2], b[2], x[2], w[2];
+  DevBuf A[2], S[2], dinv[2], b[2], x[2], w[2];
   DevBuf em[3], pr[3], rs[3], ch[3];  // transfers to the next coarser level
   MgLevelDev<double> d64{};
   MgLevelDev<float> d32{};
@@ -364,22 +364,6 @@ __global__ void __launch_bounds__(128) mg_galerkin_kernel(const MgLevelDev<T> F,
   mg_store_masked<T>(Cl, I, J, K, AE, Aout + 64 * E);
 }
 
-// For every element E of level L that contains node (i, j, k): f(row of the node in E's matrix,
-// E's first corner node, the node's corner in E).
-template <class T, class F>
-__device__ __forceinline__ void mg_for_adjacent(const MgLevelDev<T>& L, int i, int j, int k, F&& f) {
-#pragma unroll
-  for (int e = 0; e < 8; ++e) {
-    const int ex = e & 1, ey = (e >> 1) & 1, ez = e >> 2;
-    const int I = i - 1 + ex, J = j - 1 + ey, K = k - 1 + ez;
-    if (I < 0 || J < 0 || K < 0 || I >= L.nx || J >= L.ny || K >= L.nz) continue;
-    const int c = (1 - ex) + 2 * (1 - ey) + 4 * (1 - ez);  // this node's corner in E
-    const long long E = I + (long long)L.nx * (J + (long long)L.ny * K);
-    const long long n0 = I + (long long)L.nxn * (J + (long long)L.nyn * K);
-    f(L.A + 64 * E + 8 * c, n0, c);
-  }
-}
-
 __device__ __forceinline__ void load_row8(const float* row, float (&r)[8]) {
   const float4 r0 = __ldg(reinterpret_cast<const float4*>(row)), r1 = __ldg(reinterpret_cast<const float4*>(row) + 1);
   r[0] = r0.x, r[1] = r0.y, r[2] = r0.z, r[3] = r0.w, r[4] = r1.x, r[5] = r1.y, r[6] = r1.z, r[7] = r1.w;
@@ -390,15 +374,6 @@ __device__ __forceinline__ void load_row8(const double* row, double (&r)[8]) {
     const double2 v = __ldg(reinterpret_cast<const double2*>(row) + q);
     r[2 * q] = v.x, r[2 * q + 1] = v.y;
   }
-}
-
-template <class T>
-__device__ __forceinline__ T mg_row_dot(const MgLevelDev<T>& L, const T* row, long long n0, const T* x) {
-  T r[8];
-  load_row8(row, r);
-  const long long sy = L.nxn, sz = (long long)L.nxn * L.nyn;
-  return r[0] * x[n0] + r[1] * x[n0 + 1] + r[2] * x[n0 + sy] + r[3] * x[n0 + sy + 1] + r[4] * x[n0 + sz] +
-         r[5] * x[n0 + sz + 1] + r[6] * x[n0 + sz + sy] + r[7] * x[n0 + sz + sy + 1];
 }
 
 // Maximum over the block of non-negative values, folded into *dst by an integer atomicMax on the
@@ -422,26 +397,57 @@ __device__ __forceinline__ void mg_block_max(T v, T* dst) {
   }
 }
 
-// Diagonal, D^-1 and the Gershgorin bound max_i sum_j |J_ij| / J_ii of a coarse level.
+// Assembled stencil rows, D^-1 and the Gershgorin bound max_i sum_j |J_ij| / J_ii (over the element
+// rows) of a coarse level. The V-cycle's sweeps read 27 assembled coefficients per node, coalesced,
+// where the element rows took 64 values of A and 64 of x per node (FP32, 207k nodes of level 1 on the
+// 128 x 128 x 96 device: 20 us per sweep before).
 template <class T>
-__global__ void mg_diag_kernel(const MgLevelDev<T> L, T* dinv, T* par_l) {
-  const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  const long long nn = (long long)L.nxn * L.nyn * L.nzn;
+__global__ void __launch_bounds__(MG_THREADS) mg_diag_kernel(const MgLevelDev<T> L, T* dinv, T* par_l) {
+  const int n = blockIdx.x * MG_THREADS + threadIdx.x;
+  const int nn = L.nxn * L.nyn * L.nzn;
   T ratio = T(0);
   if (n < nn) {
     int i, j, k;
     node_ijk(L, n, i, j, k);
-    T dg = T(0), ra = T(0);
-    mg_for_adjacent(L, i, j, k, [&](const T* row, long long, int c) {
-      dg += row[c];
+    T ra = T(0);
+    T st[27];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) ra += fabs(row[q]);
-    });
+    for (int q = 0; q < 27; ++q) st[q] = T(0);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const int ex = e & 1, ey = (e >> 1) & 1, ez = e >> 2;
+      const int I = i - 1 + ex, J = j - 1 + ey, K = k - 1 + ez;
+      if (I < 0 || J < 0 || K < 0 || I >= L.nx || J >= L.ny || K >= L.nz) continue;
+      const int c = (1 - ex) + 2 * (1 - ey) + 4 * (1 - ez);  // this node's corner in the element
+      T r[8];
+      load_row8(L.A + 64 * (I + (long long)L.nx * (J + (long long)L.ny * K)) + 8 * c, r);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        ra += fabs(r[q]);
+        st[(ex + (q & 1)) + 3 * (ey + ((q >> 1) & 1)) + 9 * (ez + (q >> 2))] += r[q];
+      }
+    }
+    const T dg = st[13];
     const bool dir = L.mask[n] != 0 || !(dg > T(0));
     dinv[n] = dir ? T(0) : T(1) / dg;
     ratio = dir ? T(0) : ra / dg;
+#pragma unroll
+    for (int q = 0; q < 27; ++q) L.S[(size_t)q * nn + n] = st[q];
   }
   mg_block_max<T>(ratio, par_l);
+}
+
+// (A x)_n from the assembled stencil.
+template <class T>
+__device__ __forceinline__ T mg_stencil_dot(const MgLevelDev<T>& L, int nn, int n, const T* __restrict__ x) {
+  const T* S = L.S + n;
+  const T* xc = x + n;
+  const int sy = L.nxn, sz = L.nxn * L.nyn;
+  T y[3] = {T(0), T(0), T(0)};
+#pragma unroll
+  for (int q = 0; q < 27; ++q)
+    y[q % 3] += __ldg(S + (size_t)q * nn) * xc[(q % 3 - 1) + ((q / 3) % 3 - 1) * sy + (q / 9 - 1) * sz];
+  return y[0] + y[1] + y[2];
 }
 
 // Gershgorin bound of D^-1 J on the mesh (rows of the element matrices rebuilt from the
@@ -589,16 +595,12 @@ __global__ void mg_restrict_kernel(const MgLevelDev<T> F, const T* __restrict__ 
 
 // Residual after pre-smoothing on a coarse level: w = b - A x.
 template <class T>
-__global__ void mg_resid_kernel(const MgLevelDev<T> L, const PcgScalars* sc) {
+__global__ void __launch_bounds__(MG_THREADS) mg_resid_kernel(const MgLevelDev<T> L, const PcgScalars* sc) {
   if (sc->done) return;
-  const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  const long long nn = (long long)L.nxn * L.nyn * L.nzn;
+  const int n = blockIdx.x * MG_THREADS + threadIdx.x;
+  const int nn = L.nxn * L.nyn * L.nzn;
   if (n >= nn) return;
-  int i, j, k;
-  node_ijk(L, n, i, j, k);
-  T y = T(0);
-  mg_for_adjacent(L, i, j, k, [&](const T* row, long long n0, int) { y += mg_row_dot<T>(L, row, n0, L.x); });
-  L.w[n] = L.b[n] - y;
+  L.w[n] = L.b[n] - mg_stencil_dot<T>(L, nn, n, L.x);
 }
 
 // Coarse correction of level l from the solution ec of level l+1: out = base + P ec on free
@@ -629,89 +631,71 @@ __global__ void mg_prolong_kernel(const MgLevelDev<T> F, const T* __restrict__ e
 
 // Post-smoothing on a coarse level: w = x + omega D^-1 (b - A x) (the level's solution).
 template <class T>
-__global__ void mg_post_kernel(const MgLevelDev<T> L, const T* par, int l, const PcgScalars* sc) {
+__global__ void __launch_bounds__(MG_THREADS) mg_post_kernel(const MgLevelDev<T> L, const T* par, int l,
+                                                             const PcgScalars* sc) {
   if (sc->done) return;
-  const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  const long long nn = (long long)L.nxn * L.nyn * L.nzn;
+  const int n = blockIdx.x * MG_THREADS + threadIdx.x;
+  const int nn = L.nxn * L.nyn * L.nzn;
   if (n >= nn) return;
-  int i, j, k;
-  node_ijk(L, n, i, j, k);
-  T y = T(0);
-  mg_for_adjacent(L, i, j, k, [&](const T* row, long long n0, int) { y += mg_row_dot<T>(L, row, n0, L.x); });
-  L.w[n] = L.x[n] + mg_omega<T>(par, l) * L.dinv[n] * (L.b[n] - y);
+  L.w[n] = L.x[n] + mg_omega<T>(par, l) * L.dinv[n] * (L.b[n] - mg_stencil_dot<T>(L, nn, n, L.x));
 }
 
-// Coarsest level: Chebyshev iteration of degree MG_COARSE_DEGREE for A x = b on
-// [hi / 64, hi] inside one block of 1024 threads, with the element matrices and the vectors
-// in shared memory; the result goes to w.
+// Coarsest level: Chebyshev iteration of degree MG_COARSE_DEGREE for A x = b on [hi / 64, hi] in one
+// block, one thread per node (at most 512): the node's 27 stencil coefficients, its residual and its
+// solution live in registers, only the direction is exchanged, double-buffered in shared memory with
+// zeros around the mesh (one barrier per step). The result goes to w. A step was bound by the 128
+// shared-memory reads per node of the element matrices: 61 us per solve in FP32 on 8 x 8 x 5 elements.
 template <class T>
-__global__ void __launch_bounds__(1024) mg_coarse_kernel(const MgLevelDev<T> L, const T* par, int l,
-                                                         const PcgScalars* sc) {
+__global__ void __launch_bounds__(MG_COARSE_NODES) mg_coarse_kernel(const MgLevelDev<T> L, const T* par, int l,
+                                                                    const PcgScalars* sc) {
   if (sc->done) return;
   extern __shared__ __align__(16) unsigned char mg_coarse_sh[];
   T* sh = reinterpret_cast<T*>(mg_coarse_sh);
-  const int ne = L.nx * L.ny * L.nz;
-  const int nn = L.nxn * L.nyn * L.nzn;
-  T* sA = sh;               // 64 ne
-  T* sd = sA + 64 * ne;     // direction
-  T* sr = sd + nn;          // residual
-  T* sx = sr + nn;          // solution
-  for (int q = threadIdx.x; q < 64 * ne; q += blockDim.x) sA[q] = L.A[q];
-  const T hi = par[l];
-  const int n = threadIdx.x;  // one node per thread: the coarsest level has at most 512 nodes
+  const int sy = L.nxn, sz = L.nxn * L.nyn;
+  const int nn = sz * L.nzn;
+  const int pad = 1 + sy + sz, len = nn + 2 * pad;
+  const int n = threadIdx.x;
   const bool own = n < nn;
+  const T hi = par[l];
   if (!(hi > T(0))) {
     if (own) L.w[n] = T(0);
     return;
   }
+  T st[27];
+#pragma unroll
+  for (int q = 0; q < 27; ++q) st[q] = own ? __ldg(L.S + (size_t)q * nn + n) : T(0);
   const T lo = hi / T(64);
   const T theta = T(0.5) * (hi + lo), delta = T(0.5) * (hi - lo), sigma = theta / delta;
   const T dv = own ? L.dinv[n] : T(0);
-  if (own) {
-    const T r = L.b[n];
-    const T d = dv * r / theta;
-    sr[n] = r;
-    sd[n] = d;
-    sx[n] = d;
-  }
+  T r = own ? L.b[n] : T(0);
+  T d = dv * r / theta, x = d;
+  for (int q = threadIdx.x; q < 2 * len; q += blockDim.x) sh[q] = T(0);
   __syncthreads();
-  int i = 0, j = 0, k = 0;
-  const int sy = L.nxn, sz = L.nxn * L.nyn;
-  if (own) {
-    i = n % L.nxn;
-    j = (n / L.nxn) % L.nyn;
-    k = n / sz;
-  }
+  T* cur = sh + pad;
+  T* nxt = cur + len;
+  if (own) cur[n] = d;
+  __syncthreads();
   T rho = T(1) / sigma;
   for (int it = 1; it < MG_COARSE_DEGREE; ++it) {
     const T rho_new = T(1) / (T(2) * sigma - rho);
     const T c1 = rho_new * rho, c2 = T(2) * rho_new / delta;
-    T y = T(0);
     if (own) {
-      for (int e = 0; e < 8; ++e) {
-        const int ex = e & 1, ey = (e >> 1) & 1, ez = e >> 2;
-        const int I = i - 1 + ex, J = j - 1 + ey, K = k - 1 + ez;
-        if (I < 0 || J < 0 || K < 0 || I >= L.nx || J >= L.ny || K >= L.nz) continue;
-        const int c = (1 - ex) + 2 * (1 - ey) + 4 * (1 - ez);
-        const T* row = sA + 64 * (I + L.nx * (J + L.ny * K)) + 8 * c;
-        const int n0 = I + sy * (J + L.nyn * K);
-        y += row[0] * sd[n0] + row[1] * sd[n0 + 1] + row[2] * sd[n0 + sy] + row[3] * sd[n0 + sy + 1] +
-             row[4] * sd[n0 + sz] + row[5] * sd[n0 + sz + 1] + row[6] * sd[n0 + sz + sy] +
-             row[7] * sd[n0 + sz + sy + 1];
-      }
-    }
-    __syncthreads();
-    if (own) {
-      const T r = sr[n] - y;
-      const T d = c1 * sd[n] + c2 * dv * r;
-      sr[n] = r;
-      sd[n] = d;
-      sx[n] += d;
+      T y[3] = {T(0), T(0), T(0)};
+#pragma unroll
+      for (int q = 0; q < 27; ++q)
+        y[q % 3] += st[q] * cur[n + (q % 3 - 1) + ((q / 3) % 3 - 1) * sy + (q / 9 - 1) * sz];
+      r -= y[0] + y[1] + y[2];
+      d = c1 * d + c2 * dv * r;
+      x += d;
+      nxt[n] = d;
     }
     rho = rho_new;
     __syncthreads();
+    T* t = cur;
+    cur = nxt;
+    nxt = t;
   }
-  if (own) L.w[n] = sx[n];
+  if (own) L.w[n] = x;
 }
 
 // Prolongation into level 0: zq = zp + P e1 (d[1] from d[0]).
@@ -720,9 +704,12 @@ __global__ void __launch_bounds__(1024) mg_coarse_kernel(const MgLevelDev<T> L, 
 // ---------------------------------------------------------------------------
 // Host.
 
-// Shared memory of the coarsest solve in precision T.
-static size_t coarse_smem_bytes(const MgLevel& co, size_t elem) { return ((size_t)64 * co.ne + 3 * (size_t)co.n) * elem; }
-static constexpr size_t MG_COARSE_SMEM_MAX = 200 * 1024;
+// Nodes a stencil may reach off the mesh on either side of a level's vector.
+static size_t stencil_pad(const MgLevel& v) { return 1 + (size_t)(v.nx + 1) + (size_t)(v.nx + 1) * (v.ny + 1); }
+// Shared memory of the coarsest solve: two padded direction buffers. Every axis has at least two node
+// planes, so a pad is at most 1 + n/4 + n/2 nodes and 512 nodes stay below 21 KB in FP64.
+static size_t coarse_smem_bytes(const MgLevel& co, size_t elem) { return 2 * (co.n + 2 * stencil_pad(co)) * elem; }
+static constexpr size_t MG_COARSE_SMEM_MAX = 48 * 1024;
 
 bool mg_prepare(qcad_mesh_s* m) {
   // charged gates: the hierarchy's level-0 kernels carry no Robin face term (Jacobi instead)
@@ -795,11 +782,6 @@ bool mg_prepare(qcad_mesh_s* m) {
   for (size_t l = 0; l + 1 < L.size(); ++l)
     mg_mask_coarsen_kernel<<<blocks_for(L[l + 1].n), MG_THREADS, 0, s>>>(L[l].d32, L[l + 1].d32,
                                                                           L[l + 1].mask.as<unsigned char>());
-  // the largest coarsest level any mesh may have (checked above), so one setting serves all
-  CK(cudaFuncSetAttribute(mg_coarse_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                          (int)MG_COARSE_SMEM_MAX));
-  CK(cudaFuncSetAttribute(mg_coarse_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                          (int)MG_COARSE_SMEM_MAX));
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(s));
   return true;
@@ -808,7 +790,8 @@ bool mg_prepare(qcad_mesh_s* m) {
 // Operators and vectors of precision T on every coarse level (first use of that precision).
 // Kernel arguments carry these pointers by value, so this runs before any V-cycle is captured.
 template <class T>
-static void mg_alloc(MgHier* H) {
+static void mg_alloc(qcad_mesh_s* m) {
+  MgHier* H = hier(m);
   const int p = prec_index<T>();
   if (H->alloc[p]) return;
   std::deque<MgLevel>& L = H->L;
@@ -817,22 +800,27 @@ static void mg_alloc(MgHier* H) {
     v.A[p].ensure((size_t)64 * v.ne * sizeof(T) + 64);
     v.dinv[p].ensure((size_t)v.n * sizeof(T) + 64);
     v.b[p].ensure((size_t)v.n * sizeof(T) + 64);
-    v.x[p].ensure((size_t)v.n * sizeof(T) + 64);
+    const size_t pad = (stencil_pad(v) + 31) / 32 * 32, xlen = ((size_t)v.n + 2 * pad) * sizeof(T);
+    v.x[p].ensure(xlen);
+    CK(cudaMemsetAsync(v.x[p].p, 0, xlen, m->stream));
+    v.S[p].ensure((size_t)27 * v.n * sizeof(T) + 64);
     v.w[p].ensure((size_t)v.n * sizeof(T) + 64);
     MgLevelDev<T>& d = level_dev<T>(v);
     d.A = v.A[p].template as<T>();
     d.dinv = v.dinv[p].template as<T>();
     d.b = v.b[p].template as<T>();
-    d.x = v.x[p].template as<T>();
+    d.S = v.S[p].template as<T>();
+    d.x = v.x[p].template as<T>() + pad;
     d.w = v.w[p].template as<T>();
   }
   H->par[p].ensure(MG_MAX_LEVELS * sizeof(T) + 64);
+  CK(cudaStreamSynchronize(m->stream));  // the V-cycles may run on another stream
   H->alloc[p] = true;
 }
 
 template <class T>
 void mg_reserve(qcad_mesh_s* m) {
-  mg_alloc<T>(hier(m));
+  mg_alloc<T>(m);
 }
 template void mg_reserve<float>(qcad_mesh_s*);
 template void mg_reserve<double>(qcad_mesh_s*);
@@ -857,7 +845,7 @@ template <class T>
 void mg_setup(qcad_mesh_s* m, cudaStream_t s, bool force) {
   MgHier* H = hier(m);
   const int p = prec_index<T>();
-  mg_alloc<T>(H);
+  mg_alloc<T>(m);
   if (!force && H->lin_ver[p] == m->lin_ver[p]) return;
   std::deque<MgLevel>& L = H->L;
   const PcgBufs<T>& k = mesh_bufs<T>(m);
@@ -912,11 +900,11 @@ static void enqueue_vcycle(qcad_mesh_s* m, const PcgVecs<T>& v, PcgScalars* sc, 
   }
   const MgLevel& co = L[nl - 1];
   const int smem = (int)coarse_smem_bytes(co, sizeof(T));
-  note_launch(), mg_coarse_kernel<T><<<1, 1024, smem, s>>>(level_dev<T>(L[nl - 1]), par, nl - 1, sc);
+  note_launch(), mg_coarse_kernel<T><<<1, MG_COARSE_NODES, smem, s>>>(level_dev<T>(L[nl - 1]), par, nl - 1, sc);
   for (int l = nl - 2; l >= 1; --l) {
     note_launch(), mg_prolong_kernel<T><<<blocks_for(L[l].n), MG_THREADS, 0, s>>>(
                        level_dev<T>(L[l]), L[l + 1].w[p].template as<T>(), level_dev<T>(L[l + 1]),
-                       L[l].x[p].template as<T>(), L[l].x[p].template as<T>(), sc);
+                       level_dev<T>(L[l]).x, level_dev<T>(L[l]).x, sc);
     note_launch(), mg_post_kernel<T><<<blocks_for(L[l].n), MG_THREADS, 0, s>>>(level_dev<T>(L[l]), par, l, sc);
   }
   note_launch(), mg_prolong_kernel<T><<<blocks_for(L[0].n), MG_THREADS, 0, s>>>(

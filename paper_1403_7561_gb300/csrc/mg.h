@@ -50,10 +50,13 @@ struct MgChild {     // per coarse element: its first fine element and how many 
 template <class T>
 struct MgLevelDev {
   int nx, ny, nz, nxn, nyn, nzn;
-  const T* A;                 // 64 per element (levels >= 1)
+  const T* A;                 // 64 per element (levels >= 1): input of the next level's Galerkin product
+  T* S;                       // [27][nodes] assembled stencil rows (levels >= 1): offset (dx, dy, dz) at
+                              // (dx + 1) + 3 (dy + 1) + 9 (dz + 1); 0 off the mesh and on Dirichlet rows/columns
   T* dinv;                    // 0 on Dirichlet rows (levels >= 1)
   const unsigned char* mask;  // 1 on Dirichlet nodes
-  T *b, *x, *w;
+  T *b, *x, *w;               // x is padded by a plane, a row and a node of zeros on both sides, so that a
+                              // stencil may read (and multiply by 0) off the mesh
   // to the next coarser level (absent on the coarsest)
   const MgElemMap* em[3];
   const MgProl* pr[3];
