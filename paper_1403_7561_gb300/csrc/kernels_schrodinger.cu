@@ -70,7 +70,6 @@ void launch_hm_apply(const Grid<T>& g, const HmArgs<T>& args, LaunchCfg cfg, cud
   else
     note_launch(), march_kernel<T, 8, HmOp<T>><<<grid, dim3(QCAD_BX, 8), 0, s>>>(g, op, cfg.kchunk);
 }
-template void launch_hm_apply<float>(const Grid<float>&, const HmArgs<float>&, LaunchCfg, cudaStream_t);
 template void launch_hm_apply<double>(const Grid<double>&, const HmArgs<double>&, LaunchCfg, cudaStream_t);
 
 constexpr int DT = 256;

@@ -52,19 +52,67 @@ struct SubSetup {
   long long ns;     // subdomain nodes
   long long ndof;   // interior nodes
   GridDev<double> g64;
-  GridDev<float> g32;
-  GridDev<dfl> gdf;  // double-float tables: the FP64 phase's H and M applies
-  DevBuf cV64, cV32, dinv, interior;
+  DevBuf cV64, dinv, interior;
+  // the assembled operators: FP32, double-float (the FP64 phase's applies) and FP64
+  HmStencil<float> st32{};
+  HmStencil<float2> stdf{};
+  HmStencil<double> st64{};
+  DevBuf zt32, ztdf, zt64;
   double vmin;
   double inv_kx;    // 1 / kappa_x = 2 m_x / hbar^2 (scale of the separable mass stencil)
   double shift = 0.0;  // constant added to the potential (eV)
 };
 
+// rows: the precisions to assemble (ROWS_*; 0 none).
+enum { ROWS_32 = 1, ROWS_DF = 2, ROWS_64 = 4 };
+static void assemble_rows(qcad_mesh_s* m, const GridTables& t, double hx, double hy, int rows, SubSetup& S,
+                          cudaStream_t s) {
+  const int nxn = S.sm.nxs + 1, nyn = S.sm.nys + 1, nzn = S.sm.nzs + 1;
+  const long long nes = (long long)S.sm.nxs * S.sm.nys * S.sm.nzs;
+  m->s_mom.ensure((size_t)27 * nes * sizeof(double) + 64);
+  auto buf = [&](DevBuf& b, int bit, size_t e) -> void* {
+    if (!(rows & bit)) return nullptr;
+    b.ensure((size_t)27 * S.ns * e + 64);
+    return b.p;
+  };
+  float* s32 = static_cast<float*>(buf(m->s_S32, ROWS_32, sizeof(float)));
+  float2* sdf = static_cast<float2*>(buf(m->s_Sdf, ROWS_DF, sizeof(float2)));
+  double* s64 = static_cast<double*>(buf(m->s_S64, ROWS_64, sizeof(double)));
+  launch_hm_rows(S.cV64.as<double>(), nxn, nyn, nzn, m->s_mom.as<double>(), s32, sdf, s64, s);
+  // kinetic and mass coefficients of the planes, with the x and y step sizes of the a and b sums
+  std::vector<double> z((size_t)12 * nzn);
+  std::vector<float> zf(z.size());
+  std::vector<float2> zd(z.size());
+  const double mxy = hx * hy / 36.0;
+  for (int k = 0; k < nzn; ++k)
+    for (int q = 0; q < 3; ++q) {
+      z[12 * k + q] = t.mzx[3 * k + q] * (hy / (6.0 * hx));
+      z[12 * k + 3 + q] = t.mzy[3 * k + q] * (hx / (6.0 * hy));
+      z[12 * k + 6 + q] = t.kzz[3 * k + q] * mxy;
+      z[12 * k + 9 + q] = S.inv_kx * t.mzx[3 * k + q] * mxy;
+    }
+  for (size_t q = 0; q < z.size(); ++q) {
+    zf[q] = (float)z[q];
+    zd[q] = make_float2((float)z[q], (float)(z[q] - (double)(float)z[q]));
+  }
+  auto up = [&](DevBuf& b, const void* src, size_t bytes) {
+    b.ensure(bytes + 64);
+    CK(cudaMemcpyAsync(b.p, src, bytes, cudaMemcpyHostToDevice, s));
+  };
+  if (rows & ROWS_32) up(S.zt32, zf.data(), zf.size() * sizeof(float));
+  if (rows & ROWS_DF) up(S.ztdf, zd.data(), zd.size() * sizeof(float2));
+  if (rows & ROWS_64) up(S.zt64, z.data(), z.size() * sizeof(double));
+  CK(cudaStreamSynchronize(s));
+  S.st32 = {s32, S.zt32.as<float>(), nxn, nyn, nzn};
+  S.stdf = {sdf, S.ztdf.as<float2>(), nxn, nyn, nzn};
+  S.st64 = {s64, S.zt64.as<double>(), nxn, nyn, nzn};
+}
+
 // vxq: an extra potential energy at the subdomain's Gauss points (eV, [element][point]) or null;
 // shift_floor > 0: the whole potential is raised by the constant that brings its minimum to
 // shift_floor (returned in S.shift, subtracted from the eigenvalues), so that every eigenvalue
 // stays well away from zero for the relative residual test.
-static void setup_sub(qcad_mesh_s* m, const qcad_bias* b, const double* phi, const double* m_eff, int need32,
+static void setup_sub(qcad_mesh_s* m, const qcad_bias* b, const double* phi, const double* m_eff, int rows,
                       SubSetup& S, const EigIo& io, const double* vxq = nullptr, double shift_floor = 0.0) {
   if (!m->has_sub) throw Error(QCAD_ERR_INVALID_ARG, "mesh has no Schrodinger subdomain");
   for (int d = 0; d < 3; ++d)
@@ -96,16 +144,6 @@ static void setup_sub(qcad_mesh_s* m, const qcad_bias* b, const double* phi, con
   S.g64.g.dir_boundary = 1;
   S.g64.g.dir_bottom = 0;
   S.g64.g.dir_top = nullptr;
-  if (need32) {
-    build_grid<float>(S.g32, t, hx, hy, hz, s);
-    S.g32.g.dir_boundary = 1;
-    S.g32.g.dir_bottom = 0;
-    S.g32.g.dir_top = nullptr;
-    build_grid<dfl>(S.gdf, t, hx, hy, hz, s);
-    S.gdf.g.dir_boundary = 1;
-    S.gdf.g.dir_bottom = 0;
-    S.gdf.g.dir_top = nullptr;
-  }
   // potential energy at the qp: V = q phi_ref - chi - q phi (Eq. SchrodPotEnergy, no V_xc)
   const Phys P = make_phys(m, b);
   const long long nes = (long long)sm.nxs * sm.nys * sm.nzs;
@@ -117,11 +155,6 @@ static void setup_sub(qcad_mesh_s* m, const qcad_bias* b, const double* phi, con
     CK(cudaMemcpyAsync(vmin_d, &big, sizeof(double), cudaMemcpyHostToDevice, s));
     launch_potential<double>(sm, phi, V0, m->g64.g.hx, m->g64.g.hy, m->g64.g.hz, vxq, S.cV64.as<double>(), vmin_d,
                              s);
-    if (need32) {
-      S.cV32.ensure(nes * 8 * sizeof(float) + 64);
-      launch_potential<float>(sm, phi, V0, m->g64.g.hx, m->g64.g.hy, m->g64.g.hz, vxq, S.cV32.as<float>(), vmin_d,
-                              s);
-    }
     CK(cudaGetLastError());
     double vmin_shift = 0;
     CK(cudaMemcpyAsync(&vmin_shift, vmin_d, sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -134,6 +167,7 @@ static void setup_sub(qcad_mesh_s* m, const qcad_bias* b, const double* phi, con
     S.shift = shift_floor - S.vmin;
     potentials(P.phi_ref - P.chi + S.shift);
   }
+  if (rows) assemble_rows(m, t, hx[0], hy[0], rows, S, s);
   // Jacobi preconditioner from the kinetic diagonal, interior mask
   std::vector<double> dinv(S.ns, 0.0);
   std::vector<unsigned char> inter(S.ns, 0);
@@ -169,7 +203,10 @@ static void hm_apply(qcad_mesh_s* m, SubSetup& S, int prec, int nvec, const doub
     a.nvec = nvec;
     a.mscale = S.inv_kx;
     if (m->prof.on) m->prof.begin(PROF_HM, s, pp);
-    launch_hm_apply<double>(S.g64.g, a, LaunchCfg{8, 16}, s);
+    if (S.st64.S)
+      launch_hm_stencil(S.st64, a, s);
+    else
+      launch_hm_apply<double>(S.g64.g, a, LaunchCfg{8, 16}, s);
     if (m->prof.on) m->prof.end(pp, s);
   } else {
     const long long tot = S.ns * nvec;
@@ -182,12 +219,10 @@ static void hm_apply(qcad_mesh_s* m, SubSetup& S, int prec, int nvec, const doub
     a.x = x32;
     a.hx = HX ? h32 : nullptr;
     a.mx = MX ? m32 : nullptr;
-    a.cV = S.cV32.as<float>();
     a.ld = S.ns;
     a.nvec = nvec;
-    a.mscale = S.inv_kx;
     if (m->prof.on) m->prof.begin(PROF_HM, s, pp);
-    launch_hm_apply<float>(S.g32.g, a, LaunchCfg{8, 16}, s);
+    launch_hm_stencil(S.st32, a, s);
     if (m->prof.on) m->prof.end(pp, s);
     if (HX) launch_f2d(tot, h32, HX, s);
     if (MX) launch_f2d(tot, m32, MX, s);
@@ -200,7 +235,8 @@ qcad_status schrodinger_apply(qcad_mesh_s* m, const qcad_bias* b, const double* 
   if (!b || !phi || !m_eff || !X || nvec < 1) throw Error(QCAD_ERR_INVALID_ARG, "null pointer or nvec < 1");
   if (precision != 0 && precision != 1) throw Error(QCAD_ERR_INVALID_ARG, "precision must be 0 or 1");
   SubSetup S;
-  setup_sub(m, b, phi, m_eff, precision, S, mesh_io(m));
+  // FP64: assembling the rows costs about as much as applying the Gauss-point form to two vectors
+  setup_sub(m, b, phi, m_eff, precision ? ROWS_32 : nvec >= 3 ? ROWS_64 : 0, S, mesh_io(m));
   cudaStream_t s = m->stream;
   DevBuf full, tmp;
   full.ensure(3 * S.ns * nvec * sizeof(double) + 64);
@@ -241,11 +277,9 @@ struct ChebPre {
     a.x = X;
     a.hx = HX;
     a.mx = nullptr;
-    a.cV = S->cV32.as<float>();
     a.ld = ns;
     a.nvec = nvec;
-    a.mscale = S->inv_kx;
-    launch_hm_apply<float>(S->g32.g, a, LaunchCfg{8, 16}, io.s);
+    launch_hm_stencil(S->st32, a, io.s);
   }
   void init(qcad_mesh_s* m_, const EigIo& io_, SubSetup* S_, int nb_, int k_, const float* dinv32) {
     m = m_;
@@ -310,12 +344,11 @@ struct ChebPre {
       a.w = W;
       a.z = Z;
       a.dinv = dinv;
-      a.cV = S->cV32.as<float>();
       a.ld = ns;
       a.nvec = nvec;
       a.c1 = (float)(rho * rho_prev);
       a.c2 = (float)(2.0 * rho / delta);
-      launch_cheb_hm_step(S->g32.g, a, s);
+      launch_cheb_hm_step(S->st32, a, s);
       std::swap(dcur, dnext);
     }
   }
@@ -377,21 +410,19 @@ struct LobpcgRun {
     a.x = blk(Sx, b);
     a.hx = blk(HS, b);
     a.mx = blk(MS, b);
-    a.cV = cv();
     a.ld = ns;
     a.nvec = nvec;
-    a.mscale = S->inv_kx;
     Profiler::Pair pp;
     if (m->prof.on) m->prof.begin(PROF_HM, s, pp);
     if constexpr (sizeof(T) == 8) {
       // FP64 vectors: H and M in double-float arithmetic on the FP32 pipes while the residuals are
       // above DF_FLOOR, FP64 applies below it; QCAD_LOBPCG_NATIVE64 selects FP64 ones throughout
       if (df_ok && use_df_apply())
-        launch_hm_apply_df(S->gdf.g, a, s);
+        launch_hm_stencil(S->stdf, a, s);
       else
-        launch_hm_apply<T>(grid(), a, LaunchCfg{8, 16}, s);
+        launch_hm_stencil(S->st64, a, s);
     } else {
-      launch_hm_apply<T>(grid(), a, LaunchCfg{8, 16}, s);
+      launch_hm_stencil(S->st32, a, s);
     }
     if (m->prof.on) m->prof.end(pp, s);
     applies += nvec;
@@ -415,8 +446,6 @@ struct LobpcgRun {
   // locked columns are pulled back up by the rotations of the others and the iteration loses
   // stability, so that phase keeps every column active.
   bool soft_lock = false;
-  const T* cv();
-  const Grid<T>& grid();
 
   // Enqueues G1 = A^T B1 (and G2 = A^T B2) for p columns of A and q of B, with the copy of
   // both to hG (G1 at hG, G2 at hG + p*q); the caller synchronizes.
@@ -722,10 +751,6 @@ struct LobpcgRun {
   }
 };
 
-template <> const double* LobpcgRun<double>::cv() { return S->cV64.as<double>(); }
-template <> const float* LobpcgRun<float>::cv() { return S->cV32.as<float>(); }
-template <> const Grid<double>& LobpcgRun<double>::grid() { return S->g64.g; }
-template <> const Grid<float>& LobpcgRun<float>::grid() { return S->g32.g; }
 
 template <class T>
 static void init_run(LobpcgRun<T>& L, qcad_mesh_s* m, const EigIo& io, SubSetup* S, int nb, int nev, DevBuf& work,
@@ -762,7 +787,7 @@ qcad_status schrodinger_eigs_io(qcad_mesh_s* m, const EigIo& io, const qcad_bias
   if (nev < 1 || nev > 16) throw Error(QCAD_ERR_INVALID_ARG, "nev must be in [1, 16]");
   if (!(tol > 0)) throw Error(QCAD_ERR_INVALID_ARG, "tol must be > 0");
   SubSetup S;
-  setup_sub(m, b, phi, m_eff, 1, S, io, vxq, shift_floor);
+  setup_sub(m, b, phi, m_eff, ROWS_32 | ROWS_DF | ROWS_64, S, io, vxq, shift_floor);
   const double t_setup = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
   if (S.ndof < 3 * (nev + 4)) throw Error(QCAD_ERR_INVALID_ARG, "subdomain too small for nev");
   cudaStream_t s = io.s;

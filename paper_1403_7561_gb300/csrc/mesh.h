@@ -184,5 +184,6 @@ struct qcad_mesh_s {
   qcad::Profiler prof;                     // thread-safe: concurrent calls may record
   // Schrodinger workspace
   qcad::DevBuf s_mx, s_kx, s_my, s_ky, s_mzx, s_mzy, s_kzz, s_cV, s_dinv, s_interior, s_blocks, s_gram;
+  qcad::DevBuf s_mom, s_S32, s_Sdf, s_S64;  // the V rows of the subdomain and the scratch of their assembly
   ~qcad_mesh_s();
 };

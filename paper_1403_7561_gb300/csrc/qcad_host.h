@@ -212,8 +212,25 @@ template <class T>
 void launch_hm_apply(const Grid<T>& g, const HmArgs<T>& a, LaunchCfg cfg, cudaStream_t s);
 template <class T>
 void launch_hm_apply_lin(const Grid<T>& g, const HmArgs<T>& a, LaunchCfg cfg, cudaStream_t s);
-// One fused step of the LOBPCG Chebyshev-Jacobi block preconditioner (kernels_lin.cu): the H apply
-// of D_in (nvec columns at stride ld, coefficients cV) with the recurrence W -= H D_in,
+// H and M with the V term assembled into a 27-point row per node (kernels_hm.cu): S [27][nodes], zt
+// [planes][12] the kinetic coefficients of an output plane along x, y, z and its mass, each for the
+// input planes below, at and above it. C: float, double, or float2 for double-float arithmetic on
+// FP64 vectors (a.cV and a.mscale are not used).
+template <class C>
+struct HmStencil {
+  const C* S;
+  const C* zt;
+  int nxn, nyn, nzn;
+};
+void launch_hm_stencil(const HmStencil<float>& st, const HmArgs<float>& a, cudaStream_t s);
+void launch_hm_stencil(const HmStencil<double>& st, const HmArgs<double>& a, cudaStream_t s);
+void launch_hm_stencil(const HmStencil<float2>& st, const HmArgs<double>& a, cudaStream_t s);
+// The rows of the subdomain grid from its coefficients cV (8 per element), in the precisions whose
+// output is not null; mom: scratch of 27 doubles per element.
+void launch_hm_rows(const double* cV, int nxn, int nyn, int nzn, double* mom, float* S32, float2* Sdf, double* S64,
+                    cudaStream_t s);
+// One fused step of the LOBPCG Chebyshev-Jacobi block preconditioner (kernels_hm.cu): the H apply
+// of D_in (nvec columns at stride ld) with the recurrence W -= H D_in,
 // D_out = c1 D_in + c2 D^-1 W, Z += D_out in its epilogue.
 struct ChebHmArgs {
   const float* din;
@@ -221,16 +238,11 @@ struct ChebHmArgs {
   float* w;
   float* z;
   const float* dinv;
-  const float* cV;
   long long ld;
   int nvec;
   float c1, c2;
 };
-void launch_cheb_hm_step(const Grid<float>& g, const ChebHmArgs& args, cudaStream_t s);
-struct dfl;
-// The H and M applies of FP64 vectors in double-float arithmetic on the FP32 pipes (g: the
-// subdomain grid's tables as double-float pairs; a.cV the FP64 coefficients).
-void launch_hm_apply_df(const Grid<dfl>& g, const HmArgs<double>& a, cudaStream_t s);
+void launch_cheb_hm_step(const HmStencil<float>& st, const ChebHmArgs& args, cudaStream_t s);
 
 }  // namespace qcad
 
