@@ -120,8 +120,17 @@ void launch_batch_residual(const BatchResEntry* tab, int n_inst, int total_block
   note_launch(), batch_residual_kernel<8><<<total_blocks, dim3(QCAD_BX, 8), 0, s>>>(tab, n_inst);
 }
 
+// Clears the activity maps before the Gauss-point pass (one row of blocks per instance).
+__global__ void __launch_bounds__(256) batch_clear_act_kernel(const BatchResEntry* tab) {
+  const BatchResEntry& e = tab[blockIdx.y];
+  const int n = act_cells(e.g.nx, ACT_X) * act_cells(e.g.ny, ACT_Y) * act_cells(e.g.nz, ACT_Z);
+  if (e.a.act32 == nullptr) return;
+  for (int q = blockIdx.x * 256 + threadIdx.x; q < n; q += gridDim.x * 256) e.a.act32[q] = 0;
+}
+
 void launch_batch_residual_2pass(const BatchResEntry* tab, int n_inst, int qp_blocks, int node_blocks,
                                  cudaStream_t s) {
+  note_launch(), batch_clear_act_kernel<<<dim3(4, n_inst), 256, 0, s>>>(tab);
   note_launch(), batch_residual_qp_kernel<<<qp_blocks, 256, 0, s>>>(tab, n_inst);
   note_launch(), batch_residual_gather_kernel<8><<<node_blocks, dim3(QCAD_BX, 8), 0, s>>>(tab, n_inst);
 }

@@ -142,6 +142,7 @@ struct MgResid0Op {
   __device__ bool skip() const { return sc->done != 0; }
   __device__ void set_vec(int) {}
   __device__ const T* coeffs() const { return v.c; }
+  __device__ const unsigned char* act() const { return v.act; }
   __device__ const T* lin_src(int) const { return v.d[0]; }
   __device__ T lin_mix(T x0, T) const { return x0; }
   __device__ T lin_in(int n) const { return v.d[0][n]; }
@@ -171,6 +172,7 @@ struct MgPost0Op {
     om = mg_omega<T>(par, 0);
   }
   __device__ const T* coeffs() const { return v.c; }
+  __device__ const unsigned char* act() const { return v.act; }
   __device__ const T* lin_src(int) const { return v.d[1]; }
   __device__ T lin_mix(T x0, T) const { return x0; }
   __device__ T lin_in(int n) const { return v.d[1][n]; }
@@ -232,6 +234,7 @@ struct HmLinOp {
     mv = a.mx ? a.mx + o : nullptr;
   }
   __device__ const T* coeffs() const { return a.cV; }
+  __device__ const unsigned char* act() const { return nullptr; }
   __device__ const T* lin_src(int) const { return xv; }
   __device__ T lin_mix(T x0, T) const { return x0; }
   __device__ T lin_in(int n) const { return xv[n]; }

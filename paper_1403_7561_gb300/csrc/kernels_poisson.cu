@@ -316,6 +316,13 @@ __device__ __forceinline__ void residual_qp_body(const Grid<double>& g, const Re
     if (a.c64) a.c64[t] = c;
     if (a.c32) a.c32[t] = (float)c;
   }
+  // an element with a nonzero coefficient marks its cell of the activity map
+  const unsigned nz = __ballot_sync(FULL_MASK, c != 0.0);
+  if (l == 0 && ((nz >> (threadIdx.x & 24)) & 0xffu) != 0) {
+    const size_t cell = i / ACT_X + (size_t)act_cells(g.nx, ACT_X) * (j / ACT_Y + act_cells(g.ny, ACT_Y) * (k / ACT_Z));
+    if (a.act64) a.act64[cell] = 1;
+    if (a.act32) a.act32[cell] = 1;
+  }
   const double A2 = A * A, B2 = B * B;
   // the transposed interpolation of each field, skipped where the whole warp holds zeros (the
   // neutral bulk, where every density is below resolution, and the fully ionized depletion

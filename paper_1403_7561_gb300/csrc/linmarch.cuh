@@ -108,6 +108,139 @@ inline dim3 lin_grid(int nxn, int nyn, int nzn, int by, int r, int kchunk, int n
   return dim3((nxn + 29) / 30, (nyn + tr - 3) / (tr - 2), ((nzn + kchunk - 1) / kchunk) * nvec);
 }
 
+// True when some cell of the activity map that the tile's output nodes touch is active (all threads).
+template <class T, int BY, int R>
+__device__ __forceinline__ bool tile_active(const Grid<T>& g, const unsigned char* act, int bx, int by, int k0,
+                                            int k1) {
+  constexpr int TR = BY * R;
+  const int nax = act_cells(g.nx, ACT_X), nay = act_cells(g.ny, ACT_Y);
+  const int i0 = max(bx * 30 - 1, 0) / ACT_X, i1 = min(bx * 30 + 29, g.nx - 1) / ACT_X;
+  const int j0 = max(by * (TR - 2) - 1, 0) / ACT_Y, j1 = min(by * (TR - 2) + TR - 3, g.ny - 1) / ACT_Y;
+  const int l0 = max(k0 - 1, 0) / ACT_Z, l1 = min(k1 - 1, g.nz - 1) / ACT_Z;
+  const int ni = i1 - i0 + 1, nj = j1 - j0 + 1, nc = ni * nj * (l1 - l0 + 1);
+  int any = 0;
+  for (int q = threadIdx.x + 32 * threadIdx.y; q < nc; q += 32 * BY) {
+    const int i = i0 + q % ni, r = q / ni;
+    any |= act[i + nax * (j0 + r % nj + (long long)nay * (l0 + r / nj))];
+  }
+  return __syncthreads_or(any) != 0;
+}
+
+// The march of a tile without charge response (every coefficient zero): y = K v alone, the separable
+// stiffness on the mesh's uniform x and y spacings, in difference form. With, on each plane, c the node,
+// dy its second difference along y and X the second difference along x of a sum, the row of plane o is
+//   sum over the planes k = o-1, o, o+1 of  a1 dy + X(a2 c + a3 dy),  plus the fluxes w (c_o - c_k),
+// 17 operations per node (a1, a2, a3 and w per plane pair in g.zs) against about 95 with the Gauss-point
+// mass term, which dominates the FP64 form (2 FP64 lanes per SM). A constant field gives exactly zero,
+// as it does with the three-stage stencil of lin_body. The natural boundary in x and y is the mirrored
+// neighbour with half the row. Warps are independent (a warp holds two rows and reloads its neighbours'
+// from L1), so there is no barrier, and the next plane is in flight while one is summed.
+template <class T, int BY, int R, class Op>
+__device__ __forceinline__ void stiff_body(const Grid<T>& g, Op& op, int bx, int by, int k0, int k1) {
+  constexpr int TR = BY * R;
+  const int lane = threadIdx.x, ty = threadIdx.y;
+  if (ty >= (TR - 2) / 2) return;
+  const int i = bx * 30 - 1 + lane;
+  const int jb = by * (TR - 2) + 2 * ty;
+  if (jb >= g.nyn) return;
+  const int plane = (int)g.plane;
+  auto mirror = [](int q, int n) { return min(max(q < 0 ? -q : (q >= n ? 2 * (n - 1) - q : q), 0), n - 1); };
+  const int im = mirror(i, g.nxn);
+  int nrow[4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r) nrow[r] = im + g.nxn * mirror(jb - 1 + r, g.nyn);
+  const bool dov = op.lin_dir();
+  bool wr[2], top[2], bnd[2];
+  T f[2];
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    const int j = jb + r;
+    const bool nin = i >= 0 && i < g.nxn && j < g.nyn;
+    wr[r] = nin && lane >= 1 && lane <= 30;
+    top[r] = dov && nin && g.dir_top != nullptr && g.dir_top[nrow[r + 1]] != 0;
+    bnd[r] = dov && g.dir_boundary && (i == 0 || j == 0 || i == g.nx || j == g.ny);
+    f[r] = (i == 0 || i == g.nx ? T(0.5) : T(1)) * (j == 0 || j == g.ny ? T(0.5) : T(1));
+  }
+  const int kb = max(k0 - 1, 0), ke = min(k1, g.nzn - 1);
+  const T* s0 = op.lin_src(0);
+  const T* s1 = Op::NIN > 1 ? op.lin_src(1) : s0;
+  T raw[Op::NIN][4];
+  auto fetch = [&](int k) {
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      raw[0][r] = s0[nrow[r] + k * plane];
+      if (Op::NIN > 1) raw[Op::NIN - 1][r] = s1[nrow[r] + k * plane];
+    }
+  };
+  fetch(kb);
+  T c1[3][2], c2[3][2], cold[2];
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+#pragma unroll
+    for (int o = 0; o < 3; ++o) c1[o][r] = c2[o][r] = T(0);
+    cold[r] = T(0);
+  }
+  auto put = [&](int k, const typename Op::Pre* pre) {  // output plane k from the oldest sums
+    const bool pdir = dov && ((g.dir_bottom && k == 0) || (g.dir_boundary && (k == 0 || k == g.nz)));
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      const T up = __shfl_up_sync(FULL_MASK, c2[0][r], 1), dn = __shfl_down_sync(FULL_MASK, c2[0][r], 1);
+      const T y = f[r] * (c1[0][r] + ((up + dn) - T(2) * c2[0][r]));
+      const bool isdir = pdir || bnd[r] || (k == g.nz && top[r]);
+      if (wr[r]) op.lin_out(nrow[r + 1] + k * plane, pre[r], cold[r], isdir ? cold[r] : y);
+    }
+  };
+  for (int k = kb; k <= ke; ++k) {
+    T v[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) v[r] = op.lin_mix(raw[0][r], raw[Op::NIN - 1][r]);
+    if (k < ke) fetch(k + 1);
+    typename Op::Pre pre[2];
+    if (k - 1 >= k0) {
+#pragma unroll
+      for (int r = 0; r < 2; ++r)
+        if (wr[r]) pre[r] = op.lin_pre(nrow[r + 1] + (k - 1) * plane);
+    }
+    // a1, a2, a3 towards the output planes k-1, k, k+1, then the flux weight of the layer below plane k
+    T z[10];
+#pragma unroll
+    for (int q = 0; q < 10; ++q) z[q] = __ldg(g.zs + 12 * k + q);
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      const T c = v[r + 1];
+      const T dy = (v[r] + v[r + 2]) - T(2) * c;
+#pragma unroll
+      for (int o = 0; o < 3; ++o) {
+        c1[o][r] += z[3 * o] * dy;
+        c2[o][r] += z[3 * o + 1] * c;
+        c2[o][r] += z[3 * o + 2] * dy;
+      }
+      const T d = k > kb ? c - cold[r] : T(0);
+      c1[0][r] -= z[9] * d;
+      c1[1][r] += z[9] * d;
+    }
+    if (k - 1 >= k0) put(k - 1, pre);
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      cold[r] = v[r + 1];
+#pragma unroll
+      for (int o = 0; o < 2; ++o) {
+        c1[o][r] = c1[o + 1][r];
+        c2[o][r] = c2[o + 1][r];
+      }
+      c1[2][r] = c2[2][r] = T(0);
+    }
+  }
+  if (k1 == g.nzn) {
+    // the top plane has no plane above it
+    typename Op::Pre pre[2];
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+      if (wr[r]) pre[r] = op.lin_pre(nrow[r + 1] + (k1 - 1) * plane);
+    put(k1 - 1, pre);
+  }
+}
+
 // Op: the linear ops of pcg_ops.cuh (lin_in, lin_out, lin_dir, skip, set_vec, finish, coeffs),
 // or an op with SEPM = true (m_scale, lin_out2), which writes the operator with zero Dirichlet
 // rows and, as a second output, the separable consistent mass (Schrodinger H and M).
@@ -123,6 +256,16 @@ __device__ __forceinline__ void lin_body(const Grid<T>& g, const Op& op_in, int 
   const int nch = (g.nzn + kchunk - 1) / kchunk;
   Op op = op_in;
   op.set_vec(bz / nch);
+  if constexpr (!Op::SEPM) {
+    if (g.zs != nullptr && op.act() != nullptr) {
+      const int c0 = (bz % nch) * kchunk, c1 = min(c0 + kchunk, g.nzn);
+      if (!tile_active<T, BY, R>(g, op.act(), bx, by, c0, c1)) {
+        stiff_body<T, BY, R, Op>(g, op, bx, by, c0, c1);
+        op.finish();
+        return;
+      }
+    }
+  }
   // [relative plane parity][...][BY][32]: X (qx = 0, 1) of each warp's first row; upper-row
   // gather (qx = 0, 1) of each warp's last row; stiffness z stage (3 fields + pad) of the first
   // and of the last row

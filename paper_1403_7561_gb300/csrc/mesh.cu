@@ -6,7 +6,6 @@
 #include <cstring>
 #include <string>
 
-#include "dfloat.cuh"
 #include "mesh.h"
 #include "physics.cuh"
 
@@ -275,6 +274,26 @@ void build_grid(GridDev<T>& gd, const GridTables& t, const std::vector<double>& 
       zt[12 * k + 6 + q] = t.kzz[3 * k + q];
     }
   upload<T>(gd.zt, zt, s);
+  // the stiffness of uniform x and y spacings by input plane k, in difference form (stiff_body): a1, a2
+  // and a3 towards the output planes k - 1, k and k + 1, then the flux weight of the layer below plane k
+  const int nzn = (int)(t.kzz.size() / 3);
+  double Lx = 0.0, Ly = 0.0;
+  for (double h : hx) Lx += h;
+  for (double h : hy) Ly += h;
+  const double dx = Lx / hx.size(), dy = Ly / hy.size();
+  std::vector<double> zs(12 * (size_t)nzn, 0.0);
+  for (int k = 0; k < nzn; ++k) {
+    for (int o = 0; o < 3; ++o) {
+      const int out = k + o - 1;
+      if (out < 0 || out >= nzn) continue;
+      const double zx = t.mzx[3 * out + 2 - o], zy = t.mzy[3 * out + 2 - o], zz = t.kzz[3 * out + 2 - o];
+      zs[12 * k + 3 * o] = -(dx / dy) * zy + (dx * dy / 6.0) * zz;
+      zs[12 * k + 3 * o + 1] = -(dy / dx) * zx + (dx * dy / 6.0) * zz;
+      zs[12 * k + 3 * o + 2] = -(dy / (6.0 * dx)) * zx - (dx / (6.0 * dy)) * zy + (dx * dy / 36.0) * zz;
+    }
+    if (k > 0) zs[12 * k + 9] = -t.kzz[3 * (k - 1) + 2] * dx * dy;
+  }
+  upload<T>(gd.zs, zs, s);
   upload<T>(gd.hx, hx, s);
   upload<T>(gd.hy, hy, s);
   upload<T>(gd.hz, hz, s);
@@ -294,6 +313,7 @@ void build_grid(GridDev<T>& gd, const GridTables& t, const std::vector<double>& 
   g.mzy = gd.mzy.template as<T>();
   g.kzz = gd.kzz.template as<T>();
   g.zt = gd.zt.template as<T>();
+  g.zs = gd.zs.template as<T>();
   g.hx = gd.hx.template as<T>();
   g.hy = gd.hy.template as<T>();
   g.hz = gd.hz.template as<T>();
@@ -302,8 +322,6 @@ template void build_grid<float>(GridDev<float>&, const GridTables&, const std::v
                                 const std::vector<double>&, const std::vector<double>&, cudaStream_t);
 template void build_grid<double>(GridDev<double>&, const GridTables&, const std::vector<double>&,
                                  const std::vector<double>&, const std::vector<double>&, cudaStream_t);
-template void build_grid<dfl>(GridDev<dfl>&, const GridTables&, const std::vector<double>&,
-                              const std::vector<double>&, const std::vector<double>&, cudaStream_t);
 
 // Faces (fi, fj) of a node plane whose four corners lie in the closed rectangle: fi in [i0, i1),
 // fj in [j0, j1) (empty ranges when none).

@@ -67,7 +67,7 @@ struct GridTables {
 // Per-precision device copy of a grid's tables.
 template <class T>
 struct GridDev {
-  DevBuf mx, kx, my, ky, mzx, mzy, kzz, zt, hx, hy, hz;
+  DevBuf mx, kx, my, ky, mzx, mzy, kzz, zt, zs, hx, hy, hz;
   Grid<T> g{};
 };
 
@@ -97,6 +97,7 @@ struct Profiler {
 template <class T>
 struct PcgBufs {
   DevBuf x, r, z, p, Ap, b, dinv, c, w, d;
+  DevBuf act;  // activity map of c (qcad_internal.cuh)
 };
 
 struct PcgGraph {

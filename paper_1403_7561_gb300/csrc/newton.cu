@@ -55,6 +55,11 @@ template <> struct Prec<float> {
   static const int prof_apply = PROF_APPLY32, prof_update = PROF_UPDATE32;
 };
 
+// Size of a linearization's activity map.
+static size_t act_bytes(const qcad_mesh_s* m) {
+  return (size_t)act_cells(m->nx, ACT_X) * act_cells(m->ny, ACT_Y) * act_cells(m->nz, ACT_Z);
+}
+
 template <class T>
 static PcgVecs<T> ensure_pcg(qcad_mesh_s* m) {
   PcgBufs<T>& b = Prec<T>::bufs(m);
@@ -67,6 +72,7 @@ static PcgVecs<T> ensure_pcg(qcad_mesh_s* m) {
   b.b.ensure(nb);
   b.dinv.ensure(nb);
   b.c.ensure((size_t)m->n_elems * 8 * sizeof(T) + 64);
+  b.act.ensure(act_bytes(m));
   b.w.ensure(nb);
   b.d.ensure(2 * nb);
   PcgVecs<T> v;
@@ -79,6 +85,7 @@ static PcgVecs<T> ensure_pcg(qcad_mesh_s* m) {
   v.b = b.b.template as<T>();
   v.dinv = b.dinv.template as<T>();
   v.c = b.c.template as<T>();
+  v.act = b.act.template as<unsigned char>();
   v.w = b.w.template as<T>();
   v.d[0] = b.d.template as<T>();
   v.d[1] = v.d[0] + (nb / sizeof(T));
@@ -195,6 +202,7 @@ static double lambda_max(qcad_mesh_s* m, int steps) {
     a.v = x;
     a.y = y;
     a.c = v.c;
+    a.act = v.act;
     launch_apply<T>(Prec<T>::grid(m), a, Prec<T>::cfg(m), s, Prec<T>::face(m));
     CK(cudaMemsetAsync(acc, 0, 3 * sizeof(double), s));
     launch_power_step<T>(n, x, y, v.dinv, xn, acc, s);
@@ -371,12 +379,16 @@ static ResStats eval_residual(qcad_mesh_s* m, const Phys& P, const double* phi, 
   if (prec == 0 || prec == 2) {
     PcgVecs<double> v = ensure_pcg<double>(m);
     a.c64 = const_cast<double*>(v.c);
+    a.act64 = const_cast<unsigned char*>(v.act);
+    CK(cudaMemsetAsync(a.act64, 0, act_bytes(m), s));
     a.dinv64 = const_cast<double*>(v.dinv);
     a.b64 = const_cast<double*>(v.b);
   }
   if (prec == 1 || prec == 2) {
     PcgVecs<float> v = ensure_pcg<float>(m);
     a.c32 = const_cast<float*>(v.c);
+    a.act32 = const_cast<unsigned char*>(v.act);
+    CK(cudaMemsetAsync(a.act32, 0, act_bytes(m), s));
     a.dinv32 = const_cast<float*>(v.dinv);
     a.b32 = const_cast<float*>(v.b);
   }
@@ -630,6 +642,7 @@ qcad_status poisson_jv(qcad_mesh_s* m, const qcad_bias* b, const double* phi, co
     a.v = vin;
     a.y = y;
     a.c = v.c;
+    a.act = v.act;
     launch_apply<double>(m->g64.g, a, m->cfg64, s, Prec<double>::face(m));
   } else {
     PcgVecs<float> v = ensure_pcg<float>(m);
@@ -638,6 +651,7 @@ qcad_status poisson_jv(qcad_mesh_s* m, const qcad_bias* b, const double* phi, co
     a.v = v.r;
     a.y = v.Ap;
     a.c = v.c;
+    a.act = v.act;
     launch_apply<float>(m->g32.g, a, m->cfg32, s, Prec<float>::face(m));
     launch_f2d(m->n_nodes, v.Ap, y, s);
   }
@@ -852,6 +866,7 @@ static void batch_residual(BatchCtx& B, const std::vector<int>& idx, const std::
     a.phi = phi[i];
     a.R = m->R.as<double>();
     a.c32 = const_cast<float*>(v.c);
+    a.act32 = const_cast<unsigned char*>(v.act);  // cleared by the launch
     a.dinv32 = const_cast<float*>(v.dinv);
     a.b32 = const_cast<float*>(v.b);
     a.layer_semi = m->d_layer_semi.as<unsigned char>();
@@ -1052,6 +1067,7 @@ static void adjoint_solve_mixed_mg(qcad_mesh_s* m, const double* g, double* lam,
     a.v = lam;
     a.y = y;
     a.c = v.c;
+    a.act = v.act;
     launch_apply<double>(m->g64.g, a, m->cfg64, s, Prec<double>::face(m));
     launch_sub(n, g, y, r, const_cast<float*>(w.b), s);
     CK(cudaMemsetAsync(d2, 0, sizeof(double), s));
@@ -1157,6 +1173,7 @@ static void adjoint_solve_mixed(qcad_mesh_s* m, int nd, const double* G, double*
       a.v = lam;
       a.y = y;
       a.c = v64.c;
+      a.act = v64.act;
       launch_apply<double>(m->g64.g, a, m->cfg64, s, Prec<double>::face(m));
       launch_sub(n, G + (size_t)d * n, y, r, const_cast<float*>(B.vecs[d].b), s);
       launch_dot<double>(n, r, r, d2 + d, s);
@@ -1437,6 +1454,7 @@ qcad_status adjoint_batch(int n, const qcad_mesh_t* ms, const qcad_bias* bs, con
         a.v = lam(q);
         a.y = ybuf(q);
         a.c = ensure_pcg<double>(m).c;
+        a.act = ensure_pcg<double>(m).act;
         launch_apply<double>(m->g64.g, a, m->cfg64, s, nullptr);
         launch_sub(nn, rhs(q), ybuf(q), rbuf(q), const_cast<float*>(B.vecs[q].b), s);
         launch_dot<double>(nn, rbuf(q), rbuf(q), d2 + q, s);

@@ -37,6 +37,7 @@ struct ApplyOp {
   __device__ T load(const Grid<T>&, int n, bool in, int, int, int) const { return in ? a.v[n] : T(0); }
   __device__ ED edata(const Grid<T>& g, int i, int j, int k) const { return load_coeffs<T>(a.c, elem_index(g, i, j, k)); }
   __device__ const T* coeffs() const { return a.c; }
+  __device__ const unsigned char* act() const { return a.act; }
   // plane-factorized kernels: unpredicated input (n always in range), Dirichlet override
   // flag (the kernel substitutes the input on Dirichlet rows) and the store
   struct Pre {};
@@ -118,6 +119,7 @@ struct PcgApplyOp {
   }
   __device__ ED edata(const Grid<T>& g, int i, int j, int k) const { return load_coeffs<T>(v.c, elem_index(g, i, j, k)); }
   __device__ const T* coeffs() const { return v.c; }
+  __device__ const unsigned char* act() const { return v.act; }
   __device__ void elem(const Grid<T>&, int, int, int, const T* x, const ED& ed, T (*out)[8], bool) const {
     qp_mass<T>(x, ed.c, out[0]);
   }
@@ -250,6 +252,7 @@ struct ChebStepOp {
   __device__ T load(const Grid<T>&, int n, bool in, int, int, int) const { return in ? dprev[n] : T(0); }
   __device__ ED edata(const Grid<T>& g, int i, int j, int k) const { return load_coeffs<T>(v.c, elem_index(g, i, j, k)); }
   __device__ const T* coeffs() const { return v.c; }
+  __device__ const unsigned char* act() const { return v.act; }
   __device__ void elem(const Grid<T>&, int, int, int, const T* x, const ED& ed, T (*out)[8], bool) const {
     qp_mass<T>(x, ed.c, out[0]);
   }

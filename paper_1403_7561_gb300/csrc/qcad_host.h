@@ -43,6 +43,7 @@ struct PcgVecs {
   const T* b;
   const T* dinv;
   const T* c;   // element quadrature coefficients of the operator (8 per element)
+  const unsigned char* act;  // activity map of c (qcad_internal.cuh) or null (all cells active)
   T* w;         // Chebyshev inner residual
   T* d[2];      // Chebyshev correction, ping-ponged by step parity
 };
@@ -54,6 +55,8 @@ struct ResidualArgs {
   double* diag;              // or null
   double* c64;               // or null
   float* c32;                // or null
+  unsigned char* act64;      // activity map of c64, cleared by the caller, or null
+  unsigned char* act32;      // of c32
   double* dinv64;            // or null
   float* dinv32;             // or null
   double* b64;               // -R or null
@@ -78,6 +81,7 @@ struct ApplyArgs {
   const T* v;
   T* y;
   const T* c;
+  const unsigned char* act;  // activity map of c or null
   double* dot;   // accumulate v.y (writer nodes) or null
   int raw;       // 1: no identity override on Dirichlet rows (adjoint column sums)
 };

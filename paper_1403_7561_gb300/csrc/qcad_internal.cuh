@@ -39,6 +39,7 @@ struct Grid {
   const T* mzy;          // [nzn*3] kappa_y-weighted 1D mass along z
   const T* kzz;          // [nzn*3] kappa_z-weighted 1D stiffness along z
   const T* zt;           // [nzn*12] mzx, mzy, kzz rows of each plane packed (3 zeros pad), or null
+  const T* zs;           // [nzn*12] stiffness of uniform x and y spacings by input plane (stiff_body), or null
   const T* hx;           // [nx] element sizes
   const T* hy;           // [ny]
   const T* hz;           // [nz]
@@ -85,6 +86,11 @@ __device__ __forceinline__ T face_diag(const Grid<T>& g, const T* alpha, int i, 
     }
   return d;
 }
+
+// Cells of 8 x 8 x 4 elements of the activity map: a byte per cell, nonzero where some quadrature
+// coefficient of the linearization is nonzero (the cell's elements respond to the potential).
+constexpr int ACT_X = 8, ACT_Y = 8, ACT_Z = 4;
+__host__ __device__ __forceinline__ int act_cells(int n, int c) { return (n + c - 1) / c; }
 
 template <class T>
 __device__ __forceinline__ bool grid_is_dir(const Grid<T>& g, int i, int j, int k) {
