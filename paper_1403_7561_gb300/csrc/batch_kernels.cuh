@@ -53,20 +53,7 @@ __global__ void batch_status_kernel(const BatchVecEntry* tab, int n_inst, int* s
   }
 }
 
-template <int BY>
-__global__ void __launch_bounds__(QCAD_BX * BY) batch_residual_kernel(const BatchResEntry* tab, int n_inst) {
-  const int b = blockIdx.x;
-  const BatchResEntry& e = tab[batch_find(tab, n_inst, b)];
-  const int local = b - e.begin;
-  const int bx = local % e.tiles_x;
-  const int by = (local / e.tiles_x) % e.tiles_y;
-  const int bz = local / (e.tiles_x * e.tiles_y);
-  ResidualOp op = {};
-  op.a = e.a;
-  march_body<double, BY, ResidualOp>(e.g, op, e.kchunk, bx, by, bz);
-}
-
-// Entry of block b for the Gauss-point pass (entries sorted by qbegin).
+// Entry of block b for the classification pass (entries sorted by qbegin).
 __device__ __forceinline__ int batch_find_q(const BatchResEntry* tab, int n, int b) {
   int lo = 0, hi = n - 1;
   while (lo < hi) {
@@ -79,25 +66,36 @@ __device__ __forceinline__ int batch_find_q(const BatchResEntry* tab, int n, int
   return lo;
 }
 
-// Two-pass residual over the instances: Gauss-point pass, then the node gather.
-__global__ void __launch_bounds__(256) batch_residual_qp_kernel(const BatchResEntry* tab, int n_inst) {
+// The residual's passes over the instances (resnode.cuh).
+__global__ void __launch_bounds__(256) batch_residual_classify_kernel(const BatchResEntry* tab, int n_inst) {
   const int b = blockIdx.x;
   const BatchResEntry& e = tab[batch_find_q(tab, n_inst, b)];
   const long long ne = (long long)e.g.nx * e.g.ny * e.g.nz;
-  residual_qp_body(e.g, e.a, e.el, e.el + 8 * ne, (long long)(b - e.qbegin) * 256 + threadIdx.x);
+  const int local = b - e.qbegin, k0 = (local / e.qtiles) * RES_CHUNK;
+  residual_classify_body(e.g, e.a, e.el, e.el + 8 * ne, (local % e.qtiles) * 256 + threadIdx.x, k0,
+                         min(k0 + RES_CHUNK, e.g.nz));
 }
 
-template <int BY>
-__global__ void __launch_bounds__(QCAD_BX * BY) batch_residual_gather_kernel(const BatchResEntry* tab, int n_inst) {
+__global__ void __launch_bounds__(256) batch_residual_density_kernel(const BatchResEntry* tab) {
+  const BatchResEntry& e = tab[blockIdx.y];
+  const long long ne = (long long)e.g.nx * e.g.ny * e.g.nz;
+  residual_density_body(e.g, e.a, e.el, e.el + 8 * ne, blockIdx.x, gridDim.x);
+}
+
+__global__ void __launch_bounds__(32 * NODE_WARPS) batch_residual_node_kernel(const BatchResEntry* tab, int n_inst) {
   const int b = blockIdx.x;
   const BatchResEntry& e = tab[batch_find(tab, n_inst, b)];
   const int local = b - e.begin;
   const int bx = local % e.tiles_x;
   const int by = (local / e.tiles_x) % e.tiles_y;
-  const int bz = local / (e.tiles_x * e.tiles_y);
+  const int k0 = (local / (e.tiles_x * e.tiles_y)) * e.kchunk;
+  const int jb = 2 * (by * NODE_WARPS + (threadIdx.x >> 5));
   const long long ne = (long long)e.g.nx * e.g.ny * e.g.nz;
-  const ResidualGatherOp op = make_gather_op(e.a, e.el, e.el + 8 * ne);
-  march_body<double, BY, ResidualGatherOp>(e.g, op, e.kchunk, bx, by, bz);
+  double r2 = 0.0;
+  unsigned long long rmax = 0;
+  if (jb < e.g.nyn)
+    residual_node_body(e.g, e.a, e.el, e.el + 8 * ne, bx, jb, k0, min(k0 + e.kchunk, e.g.nzn), r2, rmax);
+  residual_node_finish(e.a, r2, rmax);
 }
 
 __global__ void batch_stats_kernel(const BatchResEntry* tab, int n_inst, int mode, double* out) {
@@ -106,6 +104,7 @@ __global__ void batch_stats_kernel(const BatchResEntry* tab, int n_inst, int mod
     if (mode == 0) {
       st[0] = 0.0;
       st[1] = 0.0;
+      *tab[i].a.list_n = 0;
     } else if (mode == 1) {
       st[8] = 0.0;
     } else {
@@ -116,11 +115,7 @@ __global__ void batch_stats_kernel(const BatchResEntry* tab, int n_inst, int mod
   }
 }
 
-void launch_batch_residual(const BatchResEntry* tab, int n_inst, int total_blocks, cudaStream_t s) {
-  note_launch(), batch_residual_kernel<8><<<total_blocks, dim3(QCAD_BX, 8), 0, s>>>(tab, n_inst);
-}
-
-// Clears the activity maps before the Gauss-point pass (one row of blocks per instance).
+// Clears the activity maps before the residual (one row of blocks per instance).
 __global__ void __launch_bounds__(256) batch_clear_act_kernel(const BatchResEntry* tab) {
   const BatchResEntry& e = tab[blockIdx.y];
   const int n = act_cells(e.g.nx, ACT_X) * act_cells(e.g.ny, ACT_Y) * act_cells(e.g.nz, ACT_Z);
@@ -131,8 +126,23 @@ __global__ void __launch_bounds__(256) batch_clear_act_kernel(const BatchResEntr
 void launch_batch_residual_2pass(const BatchResEntry* tab, int n_inst, int qp_blocks, int node_blocks,
                                  cudaStream_t s) {
   note_launch(), batch_clear_act_kernel<<<dim3(4, n_inst), 256, 0, s>>>(tab);
-  note_launch(), batch_residual_qp_kernel<<<qp_blocks, 256, 0, s>>>(tab, n_inst);
-  note_launch(), batch_residual_gather_kernel<8><<<node_blocks, dim3(QCAD_BX, 8), 0, s>>>(tab, n_inst);
+  note_launch(3);
+  batch_residual_classify_kernel<<<qp_blocks, 256, 0, s>>>(tab, n_inst);
+  const int db = n_inst < 8 ? sm_count() : 2 * sm_count() * 8 / n_inst;  // density blocks per instance
+  batch_residual_density_kernel<<<dim3(db > 16 ? db : 16, n_inst), 256, 0, s>>>(tab);
+  batch_residual_node_kernel<<<node_blocks, 32 * NODE_WARPS, 0, s>>>(tab, n_inst);
+}
+
+// Tiles of an instance's residual passes; total and total_q are the table's block counts so far.
+void batch_residual_shape(BatchResEntry& e, const LaunchCfg& cfg, int& total, int& total_q) {
+  e.kchunk = cfg.kchunk < 2 ? 2 : cfg.kchunk;
+  e.tiles_x = (e.g.nxn + 29) / 30;
+  e.tiles_y = (e.g.nyn + 2 * NODE_WARPS - 1) / (2 * NODE_WARPS);
+  e.begin = total;
+  total += e.tiles_x * e.tiles_y * ((e.g.nzn + e.kchunk - 1) / e.kchunk);
+  e.qbegin = total_q;
+  e.qtiles = (e.g.nx * e.g.ny + 255) / 256;
+  total_q += e.qtiles * ((e.g.nz + RES_CHUNK - 1) / RES_CHUNK);
 }
 
 void launch_batch_stats(const BatchResEntry* tab, int n_inst, int mode, double* out, cudaStream_t s) {

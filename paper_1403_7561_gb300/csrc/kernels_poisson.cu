@@ -471,11 +471,25 @@ __host__ __device__ inline ResidualGatherOp make_gather_op(const ResidualArgs& a
   return op;
 }
 
+}  // namespace qcad
+#include "resnode.cuh"
+namespace qcad {
+
 void launch_residual_2pass(const Grid<double>& g, const ResidualArgs& args, double* el, LaunchCfg cfg,
                            cudaStream_t s, const double* face) {
   const long long ne = (long long)g.nx * g.ny * g.nz;
   double* elR = el;
   double* elD = el + 8 * ne;
+  if (args.list != nullptr && args.counts == nullptr && args.qd.w == nullptr && args.bsurf == nullptr) {
+    const dim3 gc((g.nx * g.ny + 255) / 256, (g.nz + RES_CHUNK - 1) / RES_CHUNK);
+    note_launch(3);
+    residual_classify_kernel<<<gc, 256, 0, s>>>(g, args, elR, elD);
+    residual_density_kernel<<<density_blocks(ne), 256, 0, s>>>(g, args, elR, elD);
+    const int kc = node_chunk(g.nxn, g.nyn, g.nzn, cfg);
+    const dim3 gn((g.nxn + 29) / 30, (g.nyn + 2 * NODE_WARPS - 1) / (2 * NODE_WARPS), (g.nzn + kc - 1) / kc);
+    residual_node_kernel<<<gn, 32 * NODE_WARPS, 0, s>>>(g, args, elR, elD, kc);
+    return;
+  }
   const int blocks = (int)((8 * ne + 255) / 256);
   note_launch(), residual_qp_kernel<<<blocks, 256, 0, s>>>(g, args, elR, elD);
   const ResidualGatherOp op = make_gather_op(args, elR, elD);

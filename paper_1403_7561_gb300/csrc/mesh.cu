@@ -292,6 +292,10 @@ void build_grid(GridDev<T>& gd, const GridTables& t, const std::vector<double>& 
       zs[12 * k + 3 * o + 2] = -(dy / (6.0 * dx)) * zx - (dx / (6.0 * dy)) * zy + (dx * dy / 36.0) * zz;
     }
     if (k > 0) zs[12 * k + 9] = -t.kzz[3 * (k - 1) + 2] * dx * dy;
+    // diagonal of an interior node and its reciprocal
+    zs[12 * k + 10] = (4.0 / 3.0) * (dy / dx * t.mzx[3 * k + 1] + dx / dy * t.mzy[3 * k + 1]) +
+                      (4.0 / 9.0) * dx * dy * t.kzz[3 * k + 1];
+    zs[12 * k + 11] = 1.0 / zs[12 * k + 10];
   }
   upload<T>(gd.zs, zs, s);
   upload<T>(gd.hx, hx, s);

@@ -164,6 +164,7 @@ struct qcad_mesh_s {
   bool qd_active = false;
   qcad::DevBuf sp_w, sp_phiq, sp_vxq, sp_evecs, sp_prev;
   qcad::DevBuf phi_a, phi_b, R, diag, stats, counts, scal, scratch;
+  qcad::DevBuf el_list;                    // elements whose density the residual evaluates
   qcad::DevBuf el_res;                     // residual corner contributions, 16 doubles per element
   qcad::PcgScalars* h_scal = nullptr;      // pinned host mirror
   double* h_small = nullptr;               // pinned host scratch (64 doubles)

@@ -405,7 +405,10 @@ static ResStats eval_residual(qcad_mesh_s* m, const Phys& P, const double* phi, 
   a.wq = m->d_wq.as<double>();
   a.ecode = m->d_ecode.as<unsigned char>();
   if (m->has_surface) a.bsurf = m->d_bsurf.as<double>();  // charged gates, surface charges
-  CK(cudaMemsetAsync(a.stats, 0, 2 * sizeof(double), s));
+  CK(cudaMemsetAsync(a.stats, 0, 3 * sizeof(double), s));
+  m->el_list.ensure((size_t)m->n_elems * sizeof(int) + 64);
+  a.list = m->el_list.as<int>();
+  a.list_n = reinterpret_cast<int*>(a.stats + 2);
   if (counts_out) {
     a.counts = m->counts.as<double>();
     CK(cudaMemsetAsync(a.counts, 0, QCAD_MAX_DOTS_K * sizeof(double), s));
@@ -879,15 +882,12 @@ static void batch_residual(BatchCtx& B, const std::vector<int>& idx, const std::
     a.stats = m->stats.as<double>();
     a.wq = m->d_wq.as<double>();
     a.ecode = m->d_ecode.as<unsigned char>();
-    e.kchunk = std::max(2, m->cfg_res.kchunk);
-    e.tiles_x = (e.g.nxn + QCAD_BX - 3) / (QCAD_BX - 2);
-    e.tiles_y = (e.g.nyn + 8 - 3) / (8 - 2);
-    e.begin = total;
-    total += e.tiles_x * e.tiles_y * ((e.g.nzn + e.kchunk - 1) / e.kchunk);
+    m->el_list.ensure((size_t)m->n_elems * sizeof(int) + 64);
+    a.list = m->el_list.as<int>();
+    a.list_n = reinterpret_cast<int*>(m->stats.as<double>() + 2);  // zeroed with the norms
+    batch_residual_shape(e, m->cfg_res, total, total_q);
     m->el_res.ensure((size_t)16 * m->n_elems * sizeof(double) + 64);
     e.el = m->el_res.as<double>();
-    e.qbegin = total_q;
-    total_q += (int)((8 * m->n_elems + 255) / 256);
     m->lin_ver[1] += 1;  // the FP32 linearization of this mesh is rewritten
   }
   const int nq = (int)idx.size();

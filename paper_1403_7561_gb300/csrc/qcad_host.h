@@ -74,6 +74,8 @@ struct ResidualArgs {
   const double* bsurf;       // [n_nodes] constant surface load b (R -= b; two-pass residual) or null
   const double* wq;          // [nz][8] per-layer load table of constant-charge elements (physics.cuh) or null
   unsigned char* ecode;      // [n_elems] per-element load code between the two residual passes, or null
+  int* list;                 // [n_elems] elements whose density is evaluated, and their number (zeroed by
+  int* list_n;               // the caller), or null: without counts and quantum density (resnode.cuh)
 };
 
 template <class T>
@@ -300,15 +302,16 @@ struct BatchResEntry {
   ResidualArgs a;
   int kchunk;
   int tiles_x, tiles_y;
-  int begin;       // first block of the node pass (z-march tiles)
-  int qbegin;      // first block of the Gauss-point pass (256 threads each)
+  int begin;       // first block of the node pass (z-march tiles of 30 columns and 2 NODE_WARPS rows)
+  int qbegin;      // first block of the classification pass
+  int qtiles;      // its blocks per z chunk
   double* el;      // the instance's corner-contribution scratch, 16 doubles per element
 };
 void launch_batch_pcg_apply(const BatchApplyEntry* tab, int n_inst, int total_blocks, int by, cudaStream_t s);
 // Plane-factorized batched PCG apply (8 warps, two rows per thread: tiles of 30 x 14 interior nodes).
 void launch_batch_lin_apply(const BatchApplyEntry* tab, int n_inst, int total_blocks, cudaStream_t s);
-void launch_batch_residual(const BatchResEntry* tab, int n_inst, int total_blocks, cudaStream_t s);
-// Two-pass batched residual: Gauss-point pass over qp_blocks blocks, then the node pass.
+// Two-pass batched residual (resnode.cuh): classification over qp_blocks blocks, density, node pass.
+void batch_residual_shape(BatchResEntry& e, const LaunchCfg& cfg, int& total, int& total_q);
 void launch_batch_residual_2pass(const BatchResEntry* tab, int n_inst, int qp_blocks, int node_blocks,
                                  cudaStream_t s);
 // Per-instance stats slots: mode 0 zeroes the residual slots (stats[0] max |R| as ordered bits,
