@@ -66,14 +66,16 @@ __device__ __forceinline__ int batch_find_q(const BatchResEntry* tab, int n, int
   return lo;
 }
 
+constexpr int BATCH_RES_CHUNK = 4;  // element layers per block of the classification pass
+
 // The residual's passes over the instances (resnode.cuh).
 __global__ void __launch_bounds__(256) batch_residual_classify_kernel(const BatchResEntry* tab, int n_inst) {
   const int b = blockIdx.x;
   const BatchResEntry& e = tab[batch_find_q(tab, n_inst, b)];
   const long long ne = (long long)e.g.nx * e.g.ny * e.g.nz;
-  const int local = b - e.qbegin, k0 = (local / e.qtiles) * RES_CHUNK;
+  const int local = b - e.qbegin, k0 = (local / e.qtiles) * BATCH_RES_CHUNK;
   residual_classify_body(e.g, e.a, e.el, e.el + 8 * ne, (local % e.qtiles) * 256 + threadIdx.x, k0,
-                         min(k0 + RES_CHUNK, e.g.nz));
+                         min(k0 + BATCH_RES_CHUNK, e.g.nz));
 }
 
 __global__ void __launch_bounds__(256) batch_residual_density_kernel(const BatchResEntry* tab) {
@@ -142,7 +144,7 @@ void batch_residual_shape(BatchResEntry& e, const LaunchCfg& cfg, int& total, in
   total += e.tiles_x * e.tiles_y * ((e.g.nzn + e.kchunk - 1) / e.kchunk);
   e.qbegin = total_q;
   e.qtiles = (e.g.nx * e.g.ny + 255) / 256;
-  total_q += e.qtiles * ((e.g.nz + RES_CHUNK - 1) / RES_CHUNK);
+  total_q += e.qtiles * ((e.g.nz + BATCH_RES_CHUNK - 1) / BATCH_RES_CHUNK);
 }
 
 void launch_batch_stats(const BatchResEntry* tab, int n_inst, int mode, double* out, cudaStream_t s) {

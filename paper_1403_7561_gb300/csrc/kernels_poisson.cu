@@ -481,9 +481,9 @@ void launch_residual_2pass(const Grid<double>& g, const ResidualArgs& args, doub
   double* elR = el;
   double* elD = el + 8 * ne;
   if (args.list != nullptr && args.counts == nullptr && args.qd.w == nullptr && args.bsurf == nullptr) {
-    const dim3 gc((g.nx * g.ny + 255) / 256, (g.nz + RES_CHUNK - 1) / RES_CHUNK);
+    const int tiles = (g.nx * g.ny + 255) / 256, cc = classify_chunk(tiles, g.nz);
     note_launch(3);
-    residual_classify_kernel<<<gc, 256, 0, s>>>(g, args, elR, elD);
+    residual_classify_kernel<<<dim3(tiles, (g.nz + cc - 1) / cc), 256, 0, s>>>(g, args, elR, elD, cc);
     residual_density_kernel<<<density_blocks(ne), 256, 0, s>>>(g, args, elR, elD);
     const int kc = node_chunk(g.nxn, g.nyn, g.nzn, cfg);
     const dim3 gn((g.nxn + 29) / 30, (g.nyn + 2 * NODE_WARPS - 1) / (2 * NODE_WARPS), (g.nzn + kc - 1) / kc);

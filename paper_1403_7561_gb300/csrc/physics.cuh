@@ -25,23 +25,38 @@ __device__ __forceinline__ void fd_half_d(double x, double& F, double& dF, doubl
     dF = 0.0;
     return;
   }
-  if (x < -50.0) {
+  // F = e^x below -50; from -50 to -40, 1 / (e^-x + C v^(-3/8)) rounds to it (C v^(-3/8) e^x < 1e-19)
+  if (x < -40.0) {
     F = exp(x);
     dF = F;
     return;
   }
   const double xp1 = x + 1.0;
-  const double g = exp(-0.17 * xp1 * xp1);
+  const double t2 = xp1 * xp1;
+  // exp(-0.17 (x + 1)^2) below 1e-19 changes neither v nor dv by half an ulp
+  const double g = t2 > 260.0 ? 0.0 : exp(-0.17 * t2);
   const double x2 = x * x;
-  const double v = x2 * x2 + 50.0 + 33.6 * x * (1.0 - 0.68 * g);
-  const double dv = 4.0 * x2 * x + 33.6 * (1.0 - 0.68 * g) + 33.6 * 0.68 * 0.34 * x * xp1 * g;
+  const double h = 33.6 - 22.848 * g;  // 33.6 (1 - 0.68 g)
+  const double v = fma(x2, x2, fma(x, h, 50.0));
+  const double dv = fma(4.0 * x2, x, fma(7.76832 * g, x * xp1, h));
   const double emx = exp(-x);
   const double C = 1.32934038817913702047;  // 3 sqrt(pi) / 4
-  const double vp = pow(v, -0.375);
-  const double D = emx + C * vp;
-  F = 1.0 / D;
-  const double dD = -emx - 0.375 * C * vp / v * dv;
-  dF = -dD * F * F;
+  // y = v^(-1/8) from an FP32 estimate by Newton's iteration for v y^8 = 1, y <- y + y (1 - v y^8) / 8
+  // (quadratic: 3e-7, 4e-13, below an ulp), where pow and the division by v took about 120 FP64
+  // operations; v >= 40, and beyond the FP32 range the estimate comes from pow
+  double y = (double)rsqrtf(sqrtf(sqrtf((float)v)));
+  if (y == 0.0) y = pow(v, -0.125);
+  double y8 = 0.0;
+#pragma unroll
+  for (int it = 0; it < 2; ++it) {
+    const double y2 = y * y, y4 = y2 * y2;
+    y8 = y4 * y4;
+    y = fma(0.125 * y, fma(-v, y8, 1.0), y);
+  }
+  const double y2 = y * y;
+  const double cvp = C * (y2 * y);  // C v^(-3/8)
+  F = 1.0 / (emx + cvp);
+  dF = fma(0.375 * cvp * (y2 * y2) * (y2 * y2), dv, emx) * F * F;  // v^(-11/8) = v^(-3/8) y^8
 }
 
 // s = 1/(1 + g e^z) and 1 - s without overflow. Beyond z = zmax, e^{-z} is taken as zero (746:

@@ -17,10 +17,24 @@
 
 namespace qcad {
 
-constexpr int RES_CHUNK = 8;   // element layers per block of the classification pass
 constexpr int NODE_WARPS = 4;  // warps of the node pass, two node rows each
 
-// Pass 1a for the column block starting at t0 (nx * ny columns) and layers [k0, k1).
+// A double rounded to float (to nearest) on the integer pipes: the conversion instruction runs on the
+// FP64 pipe.
+__device__ __forceinline__ float d2f_bits(double a) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(a);
+  const unsigned e = (unsigned)(u >> 52) & 0x7FFu;
+  if (e < 897u || e > 1149u) return __double2float_rn(a);
+  const unsigned long long m = (u & 0x7FFFFFFFFFFFFFFFull) - (896ull << 52);
+  return __uint_as_float((unsigned)((m + 0x0FFFFFFFull + ((m >> 29) & 1)) >> 29) | ((unsigned)(u >> 32) & 0x80000000u));
+}
+// 4 a by the exponent.
+__device__ __forceinline__ double times4(double a) {
+  const long long u = __double_as_longlong(a);
+  return (u << 1) == 0 ? a : __longlong_as_double(u + (2ll << 52));
+}
+
+// Pass 1a for one element column (lanes hold consecutive columns) and layers [k0, k1).
 __device__ __forceinline__ void residual_classify_body(const Grid<double>& g, const ResidualArgs& a, double* elR,
                                                        double* elD, int col, int k0, int k1) {
   const int lane = threadIdx.x & 31;
@@ -86,14 +100,21 @@ __device__ __forceinline__ void residual_classify_body(const Grid<double>& g, co
         }
         a.ecode[e] = 0;
       }
-      if (a.c32) {
-        float4* c = reinterpret_cast<float4*>(a.c32 + 8LL * e);
-        c[0] = c[1] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-      }
-      if (a.c64) {
-        double2* c = reinterpret_cast<double2*>(a.c64 + 8LL * e);
-        c[0] = c[1] = c[2] = c[3] = make_double2(0.0, 0.0);
-      }
+    }
+    // the flat elements' zero coefficients, a warp's 32 elements as one contiguous run
+    const unsigned fl = __ballot_sync(FULL_MASK, valid && flat);
+    const long long e0 = (long long)(col - lane) + (long long)ncol * k;
+    if (a.c32) {
+      float4* c = reinterpret_cast<float4*>(a.c32 + 8 * e0);
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+        if ((fl >> ((lane + 32 * h) >> 1)) & 1) c[lane + 32 * h] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    }
+    if (a.c64) {
+      double2* c = reinterpret_cast<double2*>(a.c64 + 8 * e0);
+#pragma unroll
+      for (int h = 0; h < 4; ++h)
+        if ((fl >> ((lane + 32 * h) >> 2)) & 1) c[lane + 32 * h] = make_double2(0.0, 0.0);
     }
   }
 }
@@ -160,14 +181,13 @@ __device__ __forceinline__ void residual_node_body(const Grid<double>& g, const 
 #pragma unroll
   for (int r = 0; r < 4; ++r) nrow[r] = im + g.nxn * mirror(jb - 1 + r, g.nyn);
   bool wr[2], top[2];
-  double f[2], finv[2];
+  int half[2];  // halvings of a boundary node's row
 #pragma unroll
   for (int r = 0; r < 2; ++r) {
     const int j = jb + r;
     wr[r] = i >= 0 && i < g.nxn && j < g.nyn && lane >= 1 && lane <= 30;
     top[r] = wr[r] && g.dir_top != nullptr && g.dir_top[nrow[r + 1]] != 0;
-    f[r] = (i == 0 || i == g.nx ? 0.5 : 1.0) * (j == 0 || j == g.ny ? 0.5 : 1.0);
-    finv[r] = (i == 0 || i == g.nx ? 2.0 : 1.0) * (j == 0 || j == g.ny ? 2.0 : 1.0);
+    half[r] = (i == 0 || i == g.nx) + (j == 0 || j == g.ny);
   }
   // load codes of the elements (i, jb-1 .. jb+1) of a layer, a byte each; 255: no element
   const int eplane = g.nx * g.ny;
@@ -187,41 +207,45 @@ __device__ __forceinline__ void residual_node_body(const Grid<double>& g, const 
   for (int r = 0; r < 4; ++r) vn[r] = __ldg(a.phi + nrow[r] + kb * plane);
   int cn = kb < ke ? codes(kb) : 0;  // of the layer above plane k, read one plane ahead
   double c1[3][2], c2[3][2], cold[2], up[2] = {0.0, 0.0}, dup[2] = {0.0, 0.0};
+  bool dresp[2] = {false, false};
 #pragma unroll
   for (int r = 0; r < 2; ++r) {
 #pragma unroll
     for (int o = 0; o < 3; ++o) c1[o][r] = c2[o][r] = 0.0;
     cold[r] = 0.0;
   }
-  // output plane k from the oldest sums, the loads of layer k - 1 (up, dup) and of layer k (lo, dlo)
-  auto put = [&](int k, const double* lo, const double* dlo) {
+  // output plane k from the oldest sums, the loads of layer k - 1 (up, dup) and of layer k (lo, dlo);
+  // resp: some adjacent element adds to the diagonal
+  auto put = [&](int k, const double* lo, const double* dlo, const bool* resp) {
     const bool pdir = (g.dir_bottom && k == 0) || (g.dir_boundary && (k == 0 || k == g.nz));
+    // interior stiffness diagonal of the plane; a boundary node has half or a quarter of it
+    const double kd = __ldg(g.zs + 12 * k + 10);
+    const float kf = d2f_bits(kd);
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
       const double xs = __shfl_up_sync(FULL_MASK, c2[0][r], 1) + __shfl_down_sync(FULL_MASK, c2[0][r], 1);
       if (!wr[r]) continue;
       const int n = nrow[r + 1] + k * plane;
-      double R = f[r] * (c1[0][r] + (xs - 2.0 * c2[0][r])) + (up[r] + lo[r]);
+      double R = c1[0][r] + (xs - 2.0 * c2[0][r]);
+      if (half[r] != 0) R *= half[r] == 1 ? 0.5 : 0.25;
+      R += up[r] + lo[r];
       const bool dir = pdir || (k == g.nz && top[r]);
       if (dir) R = 0.0;
-      const double dm = dup[r] + dlo[r];
       a.R[n] = R;
       if (a.b64) a.b64[n] = -R;
-      if (a.b32) a.b32[n] = (float)(-R);
-      // interior stiffness diagonal of the plane and its reciprocal: a boundary node has half or a quarter
-      double dg, di;
-      if (dm == 0.0) {
-        dg = f[r] * __ldg(g.zs + 12 * k + 10);
-        di = finv[r] * __ldg(g.zs + 12 * k + 11);
-      } else {
-        dg = f[r] * __ldg(g.zs + 12 * k + 10) + dm;
-        di = a.dinv64 ? 1.0 / dg : 0.0;
+      if (a.b32) a.b32[n] = d2f_bits(-R);
+      const float ff = half[r] == 0 ? 1.0f : half[r] == 1 ? 0.5f : 0.25f;
+      const bool rs = resp[r] || dresp[r];
+      if (a.dinv32 && !rs)  // the FP32 Jacobi scale as an FP32 reciprocal (within an ulp of the rounded inverse)
+        a.dinv32[n] = dir ? 1.0f : __frcp_rn(ff * kf);
+      if (rs || a.diag || a.dinv64) {
+        double dg = (double)ff * kd;
+        if (rs) dg += dup[r] + dlo[r];
+        if (dir) dg = 1.0;
+        if (a.diag) a.diag[n] = dg;
+        if (a.dinv64) a.dinv64[n] = dir ? 1.0 : rs ? 1.0 / dg : __ldg(g.zs + 12 * k + 11) * (double)(1 << half[r]);
+        if (a.dinv32 && rs) a.dinv32[n] = __frcp_rn(__double2float_rn(dg));
       }
-      if (dir) dg = di = 1.0;
-      if (a.diag) a.diag[n] = dg;
-      if (a.dinv64) a.dinv64[n] = di;
-      // the FP32 Jacobi scale as an FP32 reciprocal (within an FP32 ulp of the rounded inverse)
-      if (a.dinv32) a.dinv32[n] = __frcp_rn(__double2float_rn(dg));
       acc_r2 += R * R;
       // max |R| by bit pattern (NaN left out, as fmax does)
       const unsigned long long b = (unsigned long long)__double_as_longlong(R) & 0x7fffffffffffffffull;
@@ -258,13 +282,14 @@ __device__ __forceinline__ void residual_node_body(const Grid<double>& g, const 
       if (k < ke) cn = codes(k);
       // loads of layer k - 1: to its lower plane k - 1 (lo) and its upper plane k (hi)
       double lo[2], hi[2], dlo[2] = {0.0, 0.0}, dhi[2] = {0.0, 0.0};
+      bool resp[2] = {false, false};
       const int left = __shfl_up_sync(FULL_MASK, code, 1);
       const double* wq = a.wq + 8 * (k - 1);
 #pragma unroll
       for (int r = 0; r < 2; ++r) {
         const int pr = (code >> (8 * r)) & 0xffff, pl = (left >> (8 * r)) & 0xffff, c = pr & 255;
         if (pr == pl && c == (pr >> 8) && c != 0) {
-          lo[r] = hi[r] = c == 255 ? 0.0 : 4.0 * __ldg(wq + c - 1);
+          lo[r] = hi[r] = c == 255 ? 0.0 : times4(__ldg(wq + c - 1));
         } else {
           lo[r] = hi[r] = 0.0;
           if (!wr[r]) continue;
@@ -278,6 +303,7 @@ __device__ __forceinline__ void residual_node_body(const Grid<double>& g, const 
               lo[r] += t;
               hi[r] += t;
             } else {
+              resp[r] = true;
               const long long at = 8LL * (i - 1 + ex + g.nx * (jb + r - 1 + ey) + (long long)eplane * (k - 1)) +
                                    (1 - ex) + 2 * (1 - ey);
               lo[r] += elR[at];
@@ -288,11 +314,12 @@ __device__ __forceinline__ void residual_node_body(const Grid<double>& g, const 
           }
         }
       }
-      if (k - 1 >= k0) put(k - 1, lo, dlo);
+      if (k - 1 >= k0) put(k - 1, lo, dlo, resp);
 #pragma unroll
       for (int r = 0; r < 2; ++r) {
         up[r] = hi[r];
         dup[r] = dhi[r];
+        dresp[r] = resp[r];
       }
     }
 #pragma unroll
@@ -308,7 +335,8 @@ __device__ __forceinline__ void residual_node_body(const Grid<double>& g, const 
   }
   if (k1 == g.nzn) {
     const double zero[2] = {0.0, 0.0};
-    put(k1 - 1, zero, zero);
+    const bool none[2] = {false, false};
+    put(k1 - 1, zero, zero, none);
   }
 }
 
@@ -321,9 +349,9 @@ __device__ __forceinline__ void residual_node_finish(const ResidualArgs& a, doub
 
 __global__ void __launch_bounds__(256) residual_classify_kernel(const __grid_constant__ Grid<double> g,
                                                                 const __grid_constant__ ResidualArgs a, double* elR,
-                                                                double* elD) {
-  const int k0 = blockIdx.y * RES_CHUNK;
-  residual_classify_body(g, a, elR, elD, blockIdx.x * 256 + threadIdx.x, k0, min(k0 + RES_CHUNK, g.nz));
+                                                                double* elD, int chunk) {
+  const int k0 = blockIdx.y * chunk;
+  residual_classify_body(g, a, elR, elD, blockIdx.x * 256 + threadIdx.x, k0, min(k0 + chunk, g.nz));
 }
 __global__ void __launch_bounds__(256) residual_density_kernel(const __grid_constant__ Grid<double> g,
                                                                const __grid_constant__ ResidualArgs a, double* elR,
@@ -346,6 +374,13 @@ __global__ void __launch_bounds__(32 * NODE_WARPS) residual_node_kernel(const __
 inline int density_blocks(long long ne) {
   const long long b = (ne + 31) / 32, cap = 8LL * sm_count();
   return (int)(b < cap ? b : cap);
+}
+// Layers per block of the classification pass: a block rereads one plane's zones; four where that fills
+// the SMs (8 blocks each), fewer on small grids.
+inline int classify_chunk(int tiles, int nz) {
+  int c = 4;
+  while (c > 1 && (long long)tiles * ((nz + c - 1) / c) < 8LL * sm_count()) c /= 2;
+  return c;
 }
 // z chunk of the node pass: bound by the SM's FP64 pipe, so an SM's time is its warps' planes.
 inline int node_chunk(int nxn, int nyn, int nzn, const LaunchCfg& cfg) {
