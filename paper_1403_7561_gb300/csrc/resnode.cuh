@@ -239,11 +239,11 @@ __device__ __forceinline__ void residual_node_body(const Grid<double>& g, const 
       if (a.dinv32 && !rs)  // the FP32 Jacobi scale as an FP32 reciprocal (within an ulp of the rounded inverse)
         a.dinv32[n] = dir ? 1.0f : __frcp_rn(ff * kf);
       if (rs || a.diag || a.dinv64) {
-        double dg = (double)ff * kd;
+        double dg = kd * (half[r] == 0 ? 1.0 : half[r] == 1 ? 0.5 : 0.25);
         if (rs) dg += dup[r] + dlo[r];
         if (dir) dg = 1.0;
         if (a.diag) a.diag[n] = dg;
-        if (a.dinv64) a.dinv64[n] = dir ? 1.0 : rs ? 1.0 / dg : __ldg(g.zs + 12 * k + 11) * (double)(1 << half[r]);
+        if (a.dinv64) a.dinv64[n] = dir ? 1.0 : rs ? 1.0 / dg : __ldg(g.zs + 12 * k + 11) * (half[r] == 0 ? 1.0 : half[r] == 1 ? 2.0 : 4.0);
         if (a.dinv32 && rs) a.dinv32[n] = __frcp_rn(__double2float_rn(dg));
       }
       acc_r2 += R * R;
