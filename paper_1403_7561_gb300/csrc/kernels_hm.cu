@@ -29,7 +29,7 @@ template <class T> struct HmT;
 template <> struct HmT<float> {
   using X = float;
   using C = float;
-  static constexpr int NV = 4, MINB = 3;
+  static constexpr int NV = 4, MINB = 2;
   static __device__ __forceinline__ float ld(float x) { return x; }
   static __device__ __forceinline__ float co(float c) { return c; }
   static __device__ __forceinline__ float st(float x) { return x; }

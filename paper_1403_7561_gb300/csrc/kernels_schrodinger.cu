@@ -177,6 +177,50 @@ __device__ __forceinline__ void df_mac(float& sh, float& sl, float ah, float al,
   sl += e + pl;
 }
 
+// Packed pairs (f32x2): one instruction for two independent lanes of arithmetic. The double-float
+// products are bound by issue slots and instruction fetch rather than by the FP32 lanes, so the two
+// accumulators of a pair advance together.
+__device__ __forceinline__ unsigned long long f2_pack(float a, float b) {
+  return (unsigned long long)__float_as_uint(a) | ((unsigned long long)__float_as_uint(b) << 32);
+}
+__device__ __forceinline__ float f2_lo(unsigned long long a) { return __uint_as_float((unsigned)a); }
+__device__ __forceinline__ float f2_hi(unsigned long long a) { return __uint_as_float((unsigned)(a >> 32)); }
+__device__ __forceinline__ unsigned long long f2_fma(unsigned long long a, unsigned long long b, unsigned long long c) {
+  unsigned long long d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ unsigned long long f2_mul(unsigned long long a, unsigned long long b) {
+  unsigned long long d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ unsigned long long f2_add(unsigned long long a, unsigned long long b) {
+  unsigned long long d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ unsigned long long f2_sub(unsigned long long a, unsigned long long b) {
+  unsigned long long d;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+// df_mac for a pair of accumulators with a common factor a: A = (ah, ah), N = (-ah, -ah), L = (al, al).
+// The negated product stands in for the product, so that its error needs no sign change.
+__device__ __forceinline__ void df_mac2(unsigned long long& sh, unsigned long long& sl, unsigned long long A,
+                                        unsigned long long N, unsigned long long L, unsigned long long bh,
+                                        unsigned long long bl) {
+  const unsigned long long np = f2_mul(N, bh);
+  unsigned long long pl = f2_fma(A, bh, np);
+  pl = f2_fma(A, bl, pl);
+  pl = f2_fma(L, bh, pl);
+  const unsigned long long t = f2_sub(sh, np);
+  const unsigned long long bp = f2_sub(t, sh);
+  const unsigned long long e = f2_sub(f2_sub(sh, f2_sub(t, bp)), f2_add(np, bp));
+  sh = t;
+  sl = f2_add(sl, f2_add(e, pl));
+}
+
 // Splits and joins of FP64 values go through the bit patterns (dfloat.cuh): the FP32<->FP64
 // conversion instructions run on the FP64 pipe of this part (2 lanes per SM per clock), so
 // converting in float arithmetic would cost more than the products themselves.
@@ -378,7 +422,14 @@ size_t gram_part_doubles(int p, int q) { return (size_t)GRAM_MAX_BLOCKS * p * 2 
 // double-float before it is added to the FP64 accumulators.
 // upper: only the output tiles on or above the diagonal of each product (p == q, q a multiple of
 // 4); the entries below are left unwritten.
-__global__ void __launch_bounds__(512) gram_df_kernel(long long n, int p, int nb2, const double* A, long long lda,
+// A block of at most 256 threads, two on an SM: while one waits at its barriers or copies the other
+// computes (one block of 480 threads per SM and scalar products took 1.01 ms for 36 columns and
+// 735k rows, 58 % of the issue slots).
+// Products with more than 256 output tiles (14 or more columns per block without the triangle) take one
+// block of 512 threads.
+constexpr int DGR = 32;
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS, 512 / THREADS) gram_df_kernel(long long n, int p, int nb2, const double* A, long long lda,
                                                       const double* B1, const double* B2, long long ldb,
                                                       double* part, int G, int upper) {
   extern __shared__ __align__(16) unsigned char sh_raw[];
@@ -387,11 +438,11 @@ __global__ void __launch_bounds__(512) gram_df_kernel(long long n, int p, int nb
   const int ta_n = (p + 3) / 4, tb_n = (qt + 3) / 4;
   const int pp = 4 * ta_n, qp = 4 * tb_n;
   const int W = pp + qp + 4;
-  double* sh = reinterpret_cast<double*>(sh_raw);                 // two stages of GR x W doubles
-  float* fh = reinterpret_cast<float*>(sh + (size_t)2 * GR * W);  // GR x W hi words
-  float* fl = fh + (size_t)GR * W;                                // GR x W lo words
+  double* sh = reinterpret_cast<double*>(sh_raw);                 // two stages of DGR x W doubles
+  float* fh = reinterpret_cast<float*>(sh + (size_t)2 * DGR * W);  // DGR x W hi words
+  float* fl = fh + (size_t)DGR * W;                                // DGR x W lo words
   const int tid = threadIdx.x, nth = blockDim.x;
-  for (int t = tid; t < 2 * GR * W; t += nth) sh[t] = 0.0;
+  for (int t = tid; t < 2 * DGR * W; t += nth) sh[t] = 0.0;
   __syncthreads();
   // G row groups of nt output tiles, as in gram_kernel
   const int tq = ta_n, tri = tq * (tq + 1) / 2;  // upper: tiles per product on or above its diagonal
@@ -418,13 +469,13 @@ __global__ void __launch_bounds__(512) gram_df_kernel(long long n, int p, int nb
     acch[s] = 0.0f;
     accl[s] = 0.0f;
   }
-  const long long ntiles = (n + GR - 1) / GR;
+  const long long ntiles = (n + DGR - 1) / DGR;
   auto issue = [&](long long tile, int stage) {
     if (tile < ntiles) {
-      const long long r0 = tile * GR;
-      double* st = sh + (size_t)stage * GR * W;
-      for (int t = tid; t < (p + qt) * GR; t += nth) {
-        const int col = t / GR, rr = t % GR;
+      const long long r0 = tile * DGR;
+      double* st = sh + (size_t)stage * DGR * W;
+      for (int t = tid; t < (p + qt) * DGR; t += nth) {
+        const int col = t / DGR, rr = t % DGR;
         const long long row = r0 + rr;
         const bool ok = row < n;
         const double* src;
@@ -449,31 +500,33 @@ __global__ void __launch_bounds__(512) gram_df_kernel(long long n, int p, int nb
     asm volatile("cp.async.wait_group 1;\n" ::: "memory");
     __syncthreads();
     {
-      const double* st = sh + (size_t)stage * GR * W;
-      for (int t = tid; t < GR * W; t += nth) df_split_i(st[t], fh[t], fl[t]);
+      const double* st = sh + (size_t)stage * DGR * W;
+      for (int t = tid; t < DGR * W; t += nth) df_split_i(st[t], fh[t], fl[t]);
     }
     __syncthreads();
     if (active) {
-      float sh16[16], sl16[16];
+      unsigned long long th[8], tl[8];  // the row tile's sums, columns (2 w, 2 w + 1) of row u at 2 u + w
 #pragma unroll
-      for (int s = 0; s < 16; ++s) {
-        sh16[s] = 0.0f;
-        sl16[s] = 0.0f;
-      }
+      for (int s = 0; s < 8; ++s) th[s] = tl[s] = 0ull;
 #pragma unroll 2
-      for (int rr = grp; rr < GR; rr += G) {
-        float ah[4], al[4], bh[4], bl[4];
+      for (int rr = grp; rr < DGR; rr += G) {
+        float ah[4], al[4];
         gram_ld4(fh + rr * W + 4 * ta, ah);
         gram_ld4(fl + rr * W + 4 * ta, al);
-        gram_ld4(fh + rr * W + pp + 4 * tb, bh);
-        gram_ld4(fl + rr * W + pp + 4 * tb, bl);
+        const ulonglong2 bh = *reinterpret_cast<const ulonglong2*>(fh + rr * W + pp + 4 * tb);
+        const ulonglong2 bl = *reinterpret_cast<const ulonglong2*>(fl + rr * W + pp + 4 * tb);
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-          for (int v = 0; v < 4; ++v) df_mac(sh16[4 * u + v], sl16[4 * u + v], ah[u], al[u], bh[v], bl[v]);
+        for (int u = 0; u < 4; ++u) {
+          const unsigned long long A2 = f2_pack(ah[u], ah[u]), N2 = f2_pack(-ah[u], -ah[u]), L2 = f2_pack(al[u], al[u]);
+          df_mac2(th[2 * u], tl[2 * u], A2, N2, L2, bh.x, bl.x);
+          df_mac2(th[2 * u + 1], tl[2 * u + 1], A2, N2, L2, bh.y, bl.y);
+        }
       }
 #pragma unroll
-      for (int s = 0; s < 16; ++s) df_acc(acch[s], accl[s], sh16[s], sl16[s]);
+      for (int s = 0; s < 8; ++s) {
+        df_acc(acch[2 * s], accl[2 * s], f2_lo(th[s]), f2_lo(tl[s]));
+        df_acc(acch[2 * s + 1], accl[2 * s + 1], f2_hi(th[s]), f2_hi(tl[s]));
+      }
     }
     __syncthreads();
     stage ^= 1;
@@ -542,17 +595,23 @@ void launch_gram(long long n, int p, int q, const T* A, long long lda, const T* 
       // the upper triangles only (the caller mirrors them), where the tiles align with the products
       const int up = (upper && p == q && p % 4 == 0) ? 1 : 0;
       const int nt_df = up ? nb2 * (ta_n * (ta_n + 1) / 2) : nt;
-      const int G_df = std::max(1, std::min(8, 512 / nt_df));
-      const int nth_df = std::min(512, std::max(256, ((G_df * nt_df + 31) / 32) * 32));
+      const int cap = nt_df <= 256 ? 256 : 512;
+      const int G_df = std::max(1, std::min(8, cap / nt_df));
+      const int nth_df = std::min(cap, std::max(128, ((G_df * nt_df + 31) / 32) * 32));
       const size_t red_df = (size_t)G_df * nt_df * 16 * sizeof(double);
       // two double stages plus the hi and lo float tiles
       const size_t shm_df =
-          std::max(red_df, (size_t)2 * GR * (4 * ta_n + 4 * tb_n + 4) * (sizeof(double) + sizeof(float)));
+          std::max(red_df, (size_t)2 * DGR * (4 * ta_n + 4 * tb_n + 4) * (sizeof(double) + sizeof(float)));
       static bool attr_df = false;
       if (!attr_df)
-        attr_df = cudaFuncSetAttribute(gram_df_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) ==
-                  cudaSuccess;
-      note_launch(), gram_df_kernel<<<nblk, nth_df, shm_df, s>>>(n, p, nb2, A, lda, B1, B2, ldb, part, G_df, up);
+        attr_df = cudaFuncSetAttribute(gram_df_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) ==
+                      cudaSuccess &&
+                  cudaFuncSetAttribute(gram_df_kernel<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) ==
+                      cudaSuccess;
+      if (cap == 256)
+        note_launch(), gram_df_kernel<256><<<nblk, nth_df, shm_df, s>>>(n, p, nb2, A, lda, B1, B2, ldb, part, G_df, up);
+      else
+        note_launch(), gram_df_kernel<512><<<nblk, nth_df, shm_df, s>>>(n, p, nb2, A, lda, B1, B2, ldb, part, G_df, up);
       const int tot = p * p * nb2;
       note_launch(), gram_reduce_kernel<<<(tot + 31) / 32, dim3(32, 8), 0, s>>>(nblk, tot, p * p, part, G1, G2);
       return;
@@ -768,97 +827,75 @@ __global__ void __launch_bounds__(256) lobpcg_update_kernel(long long n, int nb,
   }
 }
 
-// lobpcg_update_kernel for FP64 blocks in double-float arithmetic (C split into hi and lo float
-// tables, each row split once; X' continues P's unrounded double-float sums).
-template <int NBX, int NZX>
-__global__ void __launch_bounds__(256, (NBX <= 12 ? 2 : 1)) lobpcg_update_df_kernel(long long n, int nb, int nz, double* S,
-                                                                long long ld, const double* C, long long bstride) {
+// lobpcg_update_kernel for FP64 blocks in double-float arithmetic: a thread holds the NB outputs of its
+// row as packed double-float pairs and walks the columns of [W P] and X, each value loaded and split
+// once; C's rows are read as broadcasts from shared memory (hi and lo tables, [W P] rows first). The
+// loop body is one column, so it stays in the instruction cache: holding the row in registers and
+// looping over groups of four outputs unrolled to some 3000 instructions, whose fetch was the largest
+// stall (830 us for 12 + 24 columns and 735k rows in three block sets).
+// Every output of a row is written after all its inputs of that block have been read; X' continues
+// P's unrounded sums.
+template <int NB>
+__global__ void __launch_bounds__(256, (NB <= 12 ? 3 : 2)) lobpcg_update_df_kernel(long long n, int nb, int nz,
+                                                                                 double* S, long long ld,
+                                                                                 const double* C, long long bstride) {
   extern __shared__ __align__(16) unsigned char su_raw[];
   S += blockIdx.y * bstride;
-  const int px = (nb + 3) & ~3, pz = (nz + 3) & ~3, nq = (nb + 3) & ~3, nuse = nb + nz;
-  float* sCxh = reinterpret_cast<float*>(su_raw);  // [nq][px]
-  float* sCxl = sCxh + (size_t)nq * px;
-  float* sCzh = sCxl + (size_t)nq * px;            // [nq][pz]
-  float* sCzl = sCzh + (size_t)nq * pz;
-  // the next row of each thread, staged by cp.async while the current one is combined:
-  // [NBX + NZX][blockDim.x] doubles (column-major over the threads: conflict-free accesses)
-  double* stg = reinterpret_cast<double*>(su_raw + (((size_t)nq * (px + pz) * 2 * sizeof(float) + 15) & ~(size_t)15));
-  for (int t = threadIdx.x; t < nq * px; t += blockDim.x) {
-    const int j = t / px, i = t % px;
-    df_split((i < nb && j < nb) ? C[j * nuse + i] : 0.0, sCxh[t], sCxl[t]);
-  }
-  for (int t = threadIdx.x; t < nq * pz; t += blockDim.x) {
-    const int j = t / pz, i = t % pz;
-    df_split((i < nz && j < nb) ? C[j * nuse + nb + i] : 0.0, sCzh[t], sCzl[t]);
+  const int nuse = nb + nz;
+  float* sh = reinterpret_cast<float*>(su_raw);  // [nuse][NB] hi words, then lo words
+  float* sl = sh + (size_t)nuse * NB;
+  for (int t = threadIdx.x; t < nuse * NB; t += blockDim.x) {
+    const int i = t / NB, j = t % NB;  // row i of [Cz; Cx]
+    df_split(j < nb ? C[j * nuse + (i < nz ? nb + i : i - nz)] : 0.0, sh[t], sl[t]);
   }
   __syncthreads();
-  double* X = S;
-  double* P = S + 2 * (long long)nb * ld;
-  const int tid = threadIdx.x, bd = blockDim.x;
-  const long long stride = (long long)gridDim.x * bd;
-  auto prefetch = [&](long long row) {
-    if (row < n) {
-      for (int i = 0; i < nb; ++i) gram_cp<double>(stg + (size_t)i * bd + tid, X + i * ld + row, true);
-      for (int i = 0; i < nz; ++i) gram_cp<double>(stg + (size_t)(NBX + i) * bd + tid, S + (nb + i) * ld + row, true);
-    }
-    asm volatile("cp.async.commit_group;\n" ::: "memory");
-  };
-  long long r = blockIdx.x * (long long)bd + tid;
-  prefetch(r);
-  for (; r < n; r += stride) {
-    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-    // this thread's staged row into registers (padding columns are zeros without a split: a zero
-    // would take the FP64 conversion), then the next row's copies into the freed stage (issue is
-    // in order, so they start after these reads have completed)
-    float axh[NBX], axl[NBX], azh[NZX], azl[NZX];
+  constexpr int Q = 4;  // columns in flight
+  for (long long r = blockIdx.x * 256LL + threadIdx.x; r < n; r += gridDim.x * 256LL) {
+    unsigned long long ah[NB / 2], al[NB / 2];
 #pragma unroll
-    for (int i = 0; i < NBX; ++i) {
-      axh[i] = axl[i] = 0.0f;
-      if (i < nb) df_split_i(stg[(size_t)i * bd + tid], axh[i], axl[i]);
-    }
+    for (int j = 0; j < NB / 2; ++j) ah[j] = al[j] = 0ull;
+    // acc += sum over the columns src .. src + m - 1 of value x row i0 + i of the tables
+    auto sweep = [&](const double* src, int m, int i0) {
+      double nx[Q];
 #pragma unroll
-    for (int i = 0; i < NZX; ++i) {
-      azh[i] = azl[i] = 0.0f;
-      if (i < nz) df_split_i(stg[(size_t)(NBX + i) * bd + tid], azh[i], azl[i]);
-    }
-    prefetch(r + stride);
-    for (int j0 = 0; j0 < nb; j0 += 4) {
-      float sh[4] = {0.0f, 0.0f, 0.0f, 0.0f}, sl[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+      for (int q = 0; q < Q; ++q) nx[q] = q < m ? src[q * ld] : 0.0;
+#pragma unroll 1
+      for (int i = 0; i < m; i += Q) {
+        double cu[Q];
 #pragma unroll
-      for (int i = 0; i < NZX; i += 4) {
-        if (i < pz) {
+        for (int q = 0; q < Q; ++q) {
+          cu[q] = nx[q];
+          nx[q] = i + Q + q < m ? src[(i + Q + q) * ld] : 0.0;
+        }
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            float ch[4], cl[4];
-            gram_ld4(sCzh + (j0 + u) * pz + i, ch);
-            gram_ld4(sCzl + (j0 + u) * pz + i, cl);
+        for (int q = 0; q < Q; ++q) {
+          if (i + q >= m) break;
+          float vh, vl;
+          df_split_i(cu[q], vh, vl);
+          const unsigned long long A = f2_pack(vh, vh), N = f2_pack(-vh, -vh), L = f2_pack(vl, vl);
+          const ulonglong2* ch = reinterpret_cast<const ulonglong2*>(sh + (size_t)(i0 + i + q) * NB);
+          const ulonglong2* cl = reinterpret_cast<const ulonglong2*>(sl + (size_t)(i0 + i + q) * NB);
 #pragma unroll
-            for (int w = 0; w < 4; ++w) df_mac(sh[u], sl[u], azh[i + w], azl[i + w], ch[w], cl[w]);
+          for (int j = 0; j < NB / 4; ++j) {
+            const ulonglong2 bh = ch[j], bl = cl[j];
+            df_mac2(ah[2 * j], al[2 * j], A, N, L, bh.x, bl.x);
+            df_mac2(ah[2 * j + 1], al[2 * j + 1], A, N, L, bh.y, bl.y);
           }
         }
       }
+    };
+    auto store = [&](double* dst) {
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (j0 + u < nb) P[(j0 + u) * ld + r] = df_join(sh[u], sl[u]);
-#pragma unroll
-      for (int i = 0; i < NBX; i += 4) {
-        if (i < px) {
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            float ch[4], cl[4];
-            gram_ld4(sCxh + (j0 + u) * px + i, ch);
-            gram_ld4(sCxl + (j0 + u) * px + i, cl);
-#pragma unroll
-            for (int w = 0; w < 4; ++w) df_mac(sh[u], sl[u], axh[i + w], axl[i + w], ch[w], cl[w]);
-          }
-        }
+      for (int j = 0; j < NB / 2; ++j) {
+        if (2 * j < nb) dst[2 * j * ld] = df_join(f2_lo(ah[j]), f2_lo(al[j]));
+        if (2 * j + 1 < nb) dst[(2 * j + 1) * ld] = df_join(f2_hi(ah[j]), f2_hi(al[j]));
       }
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (j0 + u < nb) X[(j0 + u) * ld + r] = df_join(sh[u], sl[u]);
-    }
+    };
+    sweep(S + nb * ld + r, nz, 0);
+    store(S + 2LL * nb * ld + r);
+    sweep(S + r, nb, nz);
+    store(S + r);
   }
-  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
 }
 
 template <class T>
@@ -869,24 +906,21 @@ void launch_lobpcg_update(long long n, int nb, int nz, T* S, long long ld, const
   const bool small = nb <= 12 && nz <= 24;
   if constexpr (std::is_same<T, double>::value) {
     if (dense_df()) {
-      // persistent: one wave of resident blocks over the nbase block sets, each thread walking
-      // rows with the next one staged in shared memory
-      const size_t tab = (((size_t)nq * (px + pz) * 2 * sizeof(float) + 15) & ~(size_t)15);
-      const size_t shm = tab + (size_t)(small ? 36 : 60) * 256 * sizeof(double);
-      static bool attr = false;
-      if (!attr)  // a failure shows as the launch's error, which the callers check
-        attr = cudaFuncSetAttribute(lobpcg_update_df_kernel<12, 24>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    100 * 1024) == cudaSuccess &&
-               cudaFuncSetAttribute(lobpcg_update_df_kernel<20, 40>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    150 * 1024) == cudaSuccess;
+      // one wave of resident blocks over the nbase block sets
       const long long rows = (n + 255) / 256;
-      const int per_sm = small ? 2 : 1;
-      const int gx = (int)std::max<long long>(1, std::min<long long>(rows, (long long)152 * per_sm / std::max(1, nbase)));
-      const dim3 pgrid(gx, std::max(1, nbase));
-      if (small)
-        note_launch(), lobpcg_update_df_kernel<12, 24><<<pgrid, 256, shm, s>>>(n, nb, nz, S, ld, C, bstride);
+      auto run = [&](auto kern, int NB, int per_sm) {
+        const size_t tab = (size_t)(nb + nz) * NB * 2 * sizeof(float);
+        const int gx = (int)std::max<long long>(1, std::min<long long>(rows, (long long)sm_count() * per_sm / std::max(1, nbase)));
+        note_launch(), kern<<<dim3(gx, std::max(1, nbase)), 256, tab, s>>>(n, nb, nz, S, ld, C, bstride);
+      };
+      if (nb <= 8)
+        run(lobpcg_update_df_kernel<8>, 8, 3);
+      else if (nb <= 12)
+        run(lobpcg_update_df_kernel<12>, 12, 3);
+      else if (nb <= 16)
+        run(lobpcg_update_df_kernel<16>, 16, 2);
       else
-        note_launch(), lobpcg_update_df_kernel<20, 40><<<pgrid, 256, shm, s>>>(n, nb, nz, S, ld, C, bstride);
+        run(lobpcg_update_df_kernel<20>, 20, 2);
       return;
     }
   }
