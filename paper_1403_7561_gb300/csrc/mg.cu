@@ -47,7 +47,8 @@ struct MgHier {
   // and the level-0 Gershgorin row sums sum_j |K_ij| (per node). Where every coefficient c of the
   // elements involved is zero (no charge response) the operator is the stiffness alone, and the
   // setup copies these instead of rebuilding them.
-  DevBuf S1[2], ra0[2];
+  // Levels 2 and up keep theirs too, and per element whether it responded at the last setup.
+  DevBuf Sl[2][MG_MAX_LEVELS], resp[2][MG_MAX_LEVELS], ra0[2];
   bool stiff_ok[2] = {false, false};
 };
 
@@ -161,14 +162,20 @@ __global__ void mg_mask_coarsen_kernel(const MgLevelDev<float> F, const MgLevelD
   cmask[n] = F.mask[f];
 }
 
-// Row `a` of a fine element matrix P-transformed from the right, accumulated into the coarse
-// element matrix: AE[R][C] += P[a][R] (row_a P)[C], with P = px (x) py (x) pz (2 x 2 factors,
-// [fine corner][coarse corner]).
+// Galerkin products with eight lanes per coarse element (lane R of the group: row R of its matrix), so
+// that the small levels use the chip and a lane's chain is an eighth of the element's: with one thread
+// per element even the coarsest levels took 47 us in FP32 and 300 us in FP64.
+//
+// One child: lane a holds row a of the child's matrix. The row is multiplied by P from the right, one
+// axis at a time, and P^T from the left is a butterfly over the lanes per axis: lane R adds its own
+// row's part P[R][R] u and its partner's P[1-R][R] u (P = px (x) py (x) pz, 2 x 2 factors [fine][coarse]).
 template <class T>
-__device__ __forceinline__ void mg_accum_row(T (&AE)[64], const T (&row)[8], int a, const T (&px)[4],
-                                             const T (&py)[4], const T (&pz)[4]) {
+__device__ __forceinline__ void mg_accum_child(T (&acc)[8], const T (&row)[8], const MgElemMap& ex,
+                                               const MgElemMap& ey, const MgElemMap& ez, int R) {
+  const T px[4] = {(T)ex.p00, (T)ex.p01, (T)ex.p10, (T)ex.p11};
+  const T py[4] = {(T)ey.p00, (T)ey.p01, (T)ey.p10, (T)ey.p11};
+  const T pz[4] = {(T)ez.p00, (T)ez.p01, (T)ez.p10, (T)ez.p11};
   T u[8], t[8];
-  // right multiplication by P, one axis at a time: t[C] = sum_b row[b] P[b][C]
 #pragma unroll
   for (int yz = 0; yz < 4; ++yz) {
     const T r0 = row[2 * yz], r1 = row[2 * yz + 1];
@@ -189,46 +196,49 @@ __device__ __forceinline__ void mg_accum_row(T (&AE)[64], const T (&row)[8], int
     u[xy] = r0 * pz[0] + r1 * pz[2];
     u[xy + 4] = r0 * pz[1] + r1 * pz[3];
   }
-  // P[a][R] factors by selection (a is a runtime index; indexing the arrays with it would
-  // move them to local memory)
-  const bool ax = a & 1, ay = (a >> 1) & 1, az = a >> 2;
-  const T qx[2] = {ax ? px[2] : px[0], ax ? px[3] : px[1]};
-  const T qy[2] = {ay ? py[2] : py[0], ay ? py[3] : py[1]};
-  const T qz[2] = {az ? pz[2] : pz[0], az ? pz[3] : pz[1]};
+  const T* const p[3] = {px, py, pz};
 #pragma unroll
-  for (int R = 0; R < 8; ++R) {
-    const T pa = qx[R & 1] * qy[(R >> 1) & 1] * qz[R >> 2];
+  for (int ax = 0; ax < 3; ++ax) {
+    const bool hi = (R >> ax) & 1;
+    const T own = hi ? p[ax][3] : p[ax][0], oth = hi ? p[ax][1] : p[ax][2];
 #pragma unroll
-    for (int C = 0; C < 8; ++C) AE[8 * R + C] += pa * u[C];
+    for (int c = 0; c < 8; ++c) u[c] = own * u[c] + oth * __shfl_xor_sync(FULL_MASK, u[c], 1 << ax);
+  }
+#pragma unroll
+  for (int c = 0; c < 8; ++c) acc[c] += u[c];
+}
+
+__device__ __forceinline__ void load_row8(const float* row, float (&r)[8]) {
+  const float4 r0 = __ldg(reinterpret_cast<const float4*>(row)), r1 = __ldg(reinterpret_cast<const float4*>(row) + 1);
+  r[0] = r0.x, r[1] = r0.y, r[2] = r0.z, r[3] = r0.w, r[4] = r1.x, r[5] = r1.y, r[6] = r1.z, r[7] = r1.w;
+}
+__device__ __forceinline__ void load_row8(const double* row, double (&r)[8]) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const double2 v = __ldg(reinterpret_cast<const double2*>(row) + q);
+    r[2 * q] = v.x, r[2 * q + 1] = v.y;
   }
 }
 
-__device__ __forceinline__ void store4(float* o, const float (&v)[4]) {
-  *reinterpret_cast<float4*>(o) = make_float4(v[0], v[1], v[2], v[3]);
+__device__ __forceinline__ void store_row8(float* o, const float (&v)[8]) {
+  reinterpret_cast<float4*>(o)[0] = make_float4(v[0], v[1], v[2], v[3]);
+  reinterpret_cast<float4*>(o)[1] = make_float4(v[4], v[5], v[6], v[7]);
 }
-__device__ __forceinline__ void store4(double* o, const double (&v)[4]) {
-  reinterpret_cast<double2*>(o)[0] = make_double2(v[0], v[1]);
-  reinterpret_cast<double2*>(o)[1] = make_double2(v[2], v[3]);
+__device__ __forceinline__ void store_row8(double* o, const double (&v)[8]) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q) reinterpret_cast<double2*>(o)[q] = make_double2(v[2 * q], v[2 * q + 1]);
 }
 
+// Row R of the coarse matrix with the rows and columns of Dirichlet corners zeroed. All lanes call it.
 template <class T>
-__device__ __forceinline__ void mg_store_masked(const MgLevelDev<T>& Cl, int I, int J, int K, T (&AE)[64], T* out) {
-  bool dm[8];
+__device__ __forceinline__ void mg_store_masked(const MgLevelDev<T>& Cl, int I, int J, int K, T (&acc)[8], int R,
+                                                bool write, T* out) {
+  const long long nd = (I + (R & 1)) + (long long)Cl.nxn * ((J + ((R >> 1) & 1)) + (long long)Cl.nyn * (K + (R >> 2)));
+  const unsigned dm = __ballot_sync(FULL_MASK, Cl.mask[nd] != 0) >> (threadIdx.x & 24);
 #pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    const long long nd = (I + (c & 1)) + (long long)Cl.nxn * ((J + ((c >> 1) & 1)) + (long long)Cl.nyn * (K + (c >> 2)));
-    dm[c] = Cl.mask[nd] != 0;
-  }
-#pragma unroll
-  for (int q = 0; q < 16; ++q) {
-    T v[4];
-#pragma unroll
-    for (int s = 0; s < 4; ++s) {
-      const int R = (4 * q + s) >> 3, C = (4 * q + s) & 7;
-      v[s] = (dm[R] || dm[C]) ? T(0) : AE[4 * q + s];
-    }
-    store4(out + 4 * q, v);
-  }
+  for (int c = 0; c < 8; ++c)
+    if (((dm >> R) | (dm >> c)) & 1) acc[c] = T(0);
+  if (write) store_row8(out + 8 * R, acc);
 }
 
 // Row a of the fine-mesh element matrix of element (i, j, k) (stiffness from the 1D element
@@ -273,107 +283,127 @@ __device__ __forceinline__ bool mg_coef_zero(const T* __restrict__ coef, long lo
   return z;
 }
 
+// The element that a group of eight lanes works on, clamped into the level (`valid`: it exists).
+template <class T>
+__device__ __forceinline__ long long mg_group_elem(const MgLevelDev<T>& Cl, int& I, int& J, int& K, bool& valid) {
+  const long long ne = (long long)Cl.nx * Cl.ny * Cl.nz;
+  long long E = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 3;
+  valid = E < ne;
+  if (!valid) E = ne - 1;
+  I = (int)(E % Cl.nx);
+  const long long r = E / Cl.nx;
+  J = (int)(r % Cl.ny);
+  K = (int)(r / Cl.ny);
+  return E;
+}
+
+// An element without charge response has the stiffness-only matrix S_l. resp[E] is its state of the
+// last setup (1 before the first): where it is 0 then and now, the level's matrix already is that one.
+// Returns whether the group has to rebuild the matrix; copies row R of S_l where that is needed.
+template <class T>
+__device__ __forceinline__ bool mg_response(bool zero, bool valid, long long E, int R, const T* __restrict__ S,
+                                            unsigned char* resp, T* Aout) {
+  const unsigned char was = resp[E];
+  __syncwarp();
+  if (valid && R == 0 && was != (zero ? 0 : 1)) resp[E] = zero ? 0 : 1;
+  if (valid && zero && was != 0) {
+    T row[8];
+    load_row8(S + 64 * E + 8 * R, row);
+    store_row8(Aout + 64 * E + 8 * R, row);
+  }
+  return valid && !zero;
+}
+
 // Level-1 element matrices from the mesh operator (coefficients c, 8 per element). STIFF: the
-// stiffness-only matrices (c taken as zero, coef unused), stored once as S1. Otherwise a coarse
-// element whose children all have zero coefficients copies its S1 matrix (the same values the
-// rebuild would give), and the others are rebuilt.
+// stiffness-only matrices (c taken as zero, coef unused), stored once as S1. act: the activity map of
+// c (a coarse element's children lie in one of its cells) or null.
 template <class T, bool STIFF>
 __global__ void __launch_bounds__(128) mg_galerkin0_kernel(const Grid<T> g, const T* __restrict__ coef,
-                                                           const T* __restrict__ S1, const MgLevelDev<T> F,
-                                                           const MgLevelDev<T> Cl, T* Aout) {
-  const long long E = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  const long long ne = (long long)Cl.nx * Cl.ny * Cl.nz;
-  if (E >= ne) return;
-  const int I = (int)(E % Cl.nx);
-  const long long r = E / Cl.nx;
-  const int J = (int)(r % Cl.ny), K = (int)(r / Cl.ny);
+                                                           const unsigned char* __restrict__ act,
+                                                           const T* __restrict__ S1, unsigned char* resp,
+                                                           const MgLevelDev<T> F, const MgLevelDev<T> Cl, T* Aout) {
+  int I, J, K;
+  bool valid;
+  const long long E = mg_group_elem(Cl, I, J, K, valid);
+  const int R = threadIdx.x & 7;
   const MgChild cx = F.ch[0][I], cy = F.ch[1][J], cz = F.ch[2][K];
+  // child q of the group's eight: lane R looks at child R's coefficients
+  const int ci = cx.first + min(R & 1, cx.count - 1), cj = cy.first + min((R >> 1) & 1, cy.count - 1),
+            ck = cz.first + min(R >> 2, cz.count - 1);
+  bool build = valid;
   if (!STIFF) {
-    bool zero = true;
-    for (int k = cz.first; k < cz.first + cz.count; ++k)
-      for (int j = cy.first; j < cy.first + cy.count; ++j)
-        for (int i = cx.first; i < cx.first + cx.count; ++i)
-          zero = zero && mg_coef_zero<T>(coef, i + (long long)g.nx * (j + (long long)g.ny * k));
-    if (zero) {
-      const uint4* src = reinterpret_cast<const uint4*>(S1 + 64 * E);
-      uint4* dst = reinterpret_cast<uint4*>(Aout + 64 * E);
+    const bool cell = act == nullptr || act[cx.first / ACT_X + (size_t)act_cells(g.nx, ACT_X) *
+                                                                   (cy.first / ACT_Y + act_cells(g.ny, ACT_Y) * (cz.first / ACT_Z))] != 0;
+    const bool nz = cell && !mg_coef_zero<T>(coef, ci + (long long)g.nx * (cj + (long long)g.ny * ck));
+    const bool zero = ((__ballot_sync(FULL_MASK, nz) >> (threadIdx.x & 24)) & 0xffu) == 0;
+    build = mg_response<T>(zero, valid, E, R, S1, resp, Aout);
+  }
+  if (!__any_sync(FULL_MASK, build)) return;
+  T acc[8];
 #pragma unroll
-      for (int q = 0; q < (int)(64 * sizeof(T) / 16); ++q) dst[q] = __ldg(src + q);
-      return;
+  for (int q = 0; q < 8; ++q) acc[q] = T(0);
+  for (int q = 0; q < 8; ++q) {
+    const int i = cx.first + (q & 1), j = cy.first + ((q >> 1) & 1), k = cz.first + (q >> 2);
+    const bool in = build && (q & 1) < cx.count && ((q >> 1) & 1) < cy.count && (q >> 2) < cz.count;
+    T row[8];
+#pragma unroll
+    for (int b = 0; b < 8; ++b) row[b] = T(0);
+    const int ic = min(i, g.nx - 1), jc = min(j, g.ny - 1), kc = min(k, g.nz - 1);
+    if (in) {
+      T c[8];
+      if (STIFF) {
+#pragma unroll
+        for (int b = 0; b < 8; ++b) c[b] = T(0);
+      } else {
+        load_c8<T>(coef, i + (long long)g.nx * (j + (long long)g.ny * k), c);
+      }
+      bool dm[8];
+#pragma unroll
+      for (int b = 0; b < 8; ++b)
+        dm[b] = F.mask[(i + (b & 1)) + (long long)F.nxn * ((j + ((b >> 1) & 1)) + (long long)F.nyn * (k + (b >> 2)))] != 0;
+      const bool dR = F.mask[(i + (R & 1)) + (long long)F.nxn * ((j + ((R >> 1) & 1)) + (long long)F.nyn * (k + (R >> 2)))] != 0;
+      if (!dR) mg_fine_row<T>(g, i, j, k, c, dm, R, row);
     }
+    mg_accum_child<T>(acc, row, F.em[0][ic], F.em[1][jc], F.em[2][kc], R);
   }
-  T AE[64];
-#pragma unroll
-  for (int q = 0; q < 64; ++q) AE[q] = T(0);
-  for (int k = cz.first; k < cz.first + cz.count; ++k)
-    for (int j = cy.first; j < cy.first + cy.count; ++j)
-      for (int i = cx.first; i < cx.first + cx.count; ++i) {
-        const MgElemMap ex = F.em[0][i], ey = F.em[1][j], ez = F.em[2][k];
-        const T px[4] = {(T)ex.p00, (T)ex.p01, (T)ex.p10, (T)ex.p11};
-        const T py[4] = {(T)ey.p00, (T)ey.p01, (T)ey.p10, (T)ey.p11};
-        const T pz[4] = {(T)ez.p00, (T)ez.p01, (T)ez.p10, (T)ez.p11};
-        T c[8];
-        if (STIFF) {
-#pragma unroll
-          for (int q = 0; q < 8; ++q) c[q] = T(0);
-        } else {
-          load_c8<T>(coef, i + (long long)g.nx * (j + (long long)g.ny * k), c);
-        }
-        bool dm[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q)
-          dm[q] = F.mask[(i + (q & 1)) + (long long)F.nxn * ((j + ((q >> 1) & 1)) + (long long)F.nyn * (k + (q >> 2)))] != 0;
-        for (int a = 0; a < 8; ++a) {
-          if (dm[a]) continue;
-          T row[8];
-          mg_fine_row<T>(g, i, j, k, c, dm, a, row);
-          mg_accum_row<T>(AE, row, a, px, py, pz);
-        }
-      }
-  mg_store_masked<T>(Cl, I, J, K, AE, Aout + 64 * E);
+  mg_store_masked<T>(Cl, I, J, K, acc, R, build, Aout + 64 * E);
 }
 
-// Level l+1 element matrices from the stored level-l ones.
-template <class T>
-__global__ void __launch_bounds__(128) mg_galerkin_kernel(const MgLevelDev<T> F, const MgLevelDev<T> Cl, T* Aout) {
-  const long long E = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  const long long ne = (long long)Cl.nx * Cl.ny * Cl.nz;
-  if (E >= ne) return;
-  const int I = (int)(E % Cl.nx);
-  const long long r = E / Cl.nx;
-  const int J = (int)(r % Cl.ny), K = (int)(r / Cl.ny);
-  T AE[64];
-#pragma unroll
-  for (int q = 0; q < 64; ++q) AE[q] = T(0);
+// Level l+1 element matrices from the stored level-l ones (child_resp: their response states; STIFF as
+// above, from the stiffness-only matrices in F.A).
+template <class T, bool STIFF>
+__global__ void __launch_bounds__(128) mg_galerkin_kernel(const MgLevelDev<T> F, const T* __restrict__ Af,
+                                                          const unsigned char* __restrict__ child_resp,
+                                                          const T* __restrict__ S, unsigned char* resp,
+                                                          const MgLevelDev<T> Cl, T* Aout) {
+  int I, J, K;
+  bool valid;
+  const long long E = mg_group_elem(Cl, I, J, K, valid);
+  const int R = threadIdx.x & 7;
   const MgChild cx = F.ch[0][I], cy = F.ch[1][J], cz = F.ch[2][K];
-  for (int k = cz.first; k < cz.first + cz.count; ++k)
-    for (int j = cy.first; j < cy.first + cy.count; ++j)
-      for (int i = cx.first; i < cx.first + cx.count; ++i) {
-        const MgElemMap ex = F.em[0][i], ey = F.em[1][j], ez = F.em[2][k];
-        const T px[4] = {(T)ex.p00, (T)ex.p01, (T)ex.p10, (T)ex.p11};
-        const T py[4] = {(T)ey.p00, (T)ey.p01, (T)ey.p10, (T)ey.p11};
-        const T pz[4] = {(T)ez.p00, (T)ez.p01, (T)ez.p10, (T)ez.p11};
-        const T* Ae = F.A + 64 * (i + (long long)F.nx * (j + (long long)F.ny * k));
-        for (int a = 0; a < 8; ++a) {
-          T row[8];
-#pragma unroll
-          for (int b = 0; b < 8; ++b) row[b] = __ldg(Ae + 8 * a + b);
-          mg_accum_row<T>(AE, row, a, px, py, pz);
-        }
-      }
-  mg_store_masked<T>(Cl, I, J, K, AE, Aout + 64 * E);
-}
-
-__device__ __forceinline__ void load_row8(const float* row, float (&r)[8]) {
-  const float4 r0 = __ldg(reinterpret_cast<const float4*>(row)), r1 = __ldg(reinterpret_cast<const float4*>(row) + 1);
-  r[0] = r0.x, r[1] = r0.y, r[2] = r0.z, r[3] = r0.w, r[4] = r1.x, r[5] = r1.y, r[6] = r1.z, r[7] = r1.w;
-}
-__device__ __forceinline__ void load_row8(const double* row, double (&r)[8]) {
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const double2 v = __ldg(reinterpret_cast<const double2*>(row) + q);
-    r[2 * q] = v.x, r[2 * q + 1] = v.y;
+  bool build = valid;
+  if (!STIFF) {
+    const int ci = cx.first + min(R & 1, cx.count - 1), cj = cy.first + min((R >> 1) & 1, cy.count - 1),
+              ck = cz.first + min(R >> 2, cz.count - 1);
+    const bool nz = child_resp[ci + (long long)F.nx * (cj + (long long)F.ny * ck)] != 0;
+    const bool zero = ((__ballot_sync(FULL_MASK, nz) >> (threadIdx.x & 24)) & 0xffu) == 0;
+    build = mg_response<T>(zero, valid, E, R, S, resp, Aout);
   }
+  if (!__any_sync(FULL_MASK, build)) return;
+  T acc[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) acc[q] = T(0);
+#pragma unroll 2
+  for (int q = 0; q < 8; ++q) {
+    const int i = cx.first + (q & 1), j = cy.first + ((q >> 1) & 1), k = cz.first + (q >> 2);
+    const bool in = build && (q & 1) < cx.count && ((q >> 1) & 1) < cy.count && (q >> 2) < cz.count;
+    T row[8];
+#pragma unroll
+    for (int b = 0; b < 8; ++b) row[b] = T(0);
+    if (in) load_row8(Af + 64 * (i + (long long)F.nx * (j + (long long)F.ny * k)) + 8 * R, row);
+    mg_accum_child<T>(acc, row, F.em[0][min(i, F.nx - 1)], F.em[1][min(j, F.ny - 1)], F.em[2][min(k, F.nz - 1)], R);
+  }
+  mg_store_masked<T>(Cl, I, J, K, acc, R, build, Aout + 64 * E);
 }
 
 // Maximum over the block of non-negative values, folded into *dst by an integer atomicMax on the
@@ -455,14 +485,14 @@ __device__ __forceinline__ T mg_stencil_dot(const MgLevelDev<T>& L, int nn, int 
 // sums sum_j |K_ij| into ra0 (c taken as zero). Otherwise a node whose adjacent elements all have
 // zero coefficients takes its row sum from ra0 (the value the rebuild would give).
 template <class T, bool STIFF>
-__global__ void mg_gersh0_kernel(const Grid<T> g, const T* __restrict__ coef, const MgLevelDev<T> F,
-                                 const T* dinv0, T* ra0, T* par0) {
-  const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  const long long nn = (long long)F.nxn * F.nyn * F.nzn;
+__global__ void mg_gersh0_kernel(const Grid<T> g, const T* __restrict__ coef,
+                                 const unsigned char* __restrict__ act, const MgLevelDev<T> F, const T* dinv0, T* ra0,
+                                 T* par0) {
+  const int n = blockIdx.x * blockDim.x + threadIdx.x;
+  const int nn = F.nxn * F.nyn * F.nzn;
   T ratio = T(0);
   if (n < nn) {
-    int i, j, k;
-    node_ijk(F, n, i, j, k);
+    const int k = n / (F.nxn * F.nyn), r2 = n - k * (F.nxn * F.nyn), j = r2 / F.nxn, i = r2 - j * F.nxn;
     if (F.mask[n]) {
       ratio = T(1);
       if (STIFF) ra0[n] = T(0);
@@ -472,7 +502,8 @@ __global__ void mg_gersh0_kernel(const Grid<T> g, const T* __restrict__ coef, co
         for (int e = 0; e < 8; ++e) {
           const int I = i - 1 + (e & 1), J = j - 1 + ((e >> 1) & 1), K = k - 1 + (e >> 2);
           if (I < 0 || J < 0 || K < 0 || I >= F.nx || J >= F.ny || K >= F.nz) continue;
-          zero = zero && mg_coef_zero<T>(coef, I + (long long)g.nx * (J + (long long)g.ny * K));
+          const int cell = I / ACT_X + act_cells(g.nx, ACT_X) * (J / ACT_Y + act_cells(g.ny, ACT_Y) * (K / ACT_Z));
+          zero = zero && (act[cell] == 0 || mg_coef_zero<T>(coef, I + (long long)g.nx * (J + (long long)g.ny * K)));
         }
       }
       T ra = T(0);
@@ -514,13 +545,44 @@ __global__ void mg_gersh0_kernel(const Grid<T> g, const T* __restrict__ coef, co
 // V-cycle kernels. Every kernel returns at once when the PCG has finished (sc->done), so the
 // iterations captured after convergence cost a launch each and nothing more.
 
+// 16 bytes of values of type T.
+template <class T>
+struct alignas(16) MgPack {
+  static constexpr int N = 16 / (int)sizeof(T);
+  T v[N];
+};
+template <class T>
+__device__ __forceinline__ MgPack<T> mg_ldp(const T* p, int i) {
+  return reinterpret_cast<const MgPack<T>*>(p)[i];
+}
+template <class T>
+__device__ __forceinline__ void mg_stp(T* p, int i, const MgPack<T>& q) {
+  reinterpret_cast<MgPack<T>*>(p)[i] = q;
+}
+
 // PCG start with the multigrid preconditioner: x = 0, r = b, ||r||^2, and the level-0
 // pre-smoothing zp = omega D^-1 r (into d[0]).
 template <class T>
-__global__ void mg_pcg_init_kernel(int n, PcgVecs<T> v, PcgScalars* sc, const T* par) {
+__global__ void __launch_bounds__(256) mg_pcg_init_kernel(int n, PcgVecs<T> v, PcgScalars* sc, const T* par) {
+  constexpr int N = MgPack<T>::N;
   const T om = mg_omega<T>(par, 0);
   T rr = T(0);
-  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < n; idx += gridDim.x * blockDim.x) {
+  const int np = n / N;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < np; i += gridDim.x * blockDim.x) {
+    const MgPack<T> r = mg_ldp(v.b, i), di = mg_ldp(v.dinv, i);
+    MgPack<T> z, d;
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+      z.v[q] = T(0);
+      d.v[q] = om * di.v[q] * r.v[q];
+      rr += r.v[q] * r.v[q];
+    }
+    mg_stp(v.x, i, z);
+    mg_stp(v.r, i, r);
+    mg_stp(v.d[0], i, d);
+  }
+  const int idx = N * np + blockIdx.x * blockDim.x + threadIdx.x;  // the last n % N values
+  if (idx < n) {
     const T r = v.b[idx];
     v.x[idx] = T(0);
     v.r[idx] = r;
@@ -531,10 +593,13 @@ __global__ void mg_pcg_init_kernel(int n, PcgVecs<T> v, PcgScalars* sc, const T*
   block_sum_atomic<1>(s1, &sc->rr[0]);
 }
 
-// PCG update (alpha = rz / pAp): x += alpha p, r -= alpha Ap, ||r||^2, then zp = omega D^-1 r.
+// PCG update (alpha = rz / pAp): x += alpha p, r -= alpha Ap, ||r||^2, then zp = omega D^-1 r. Bound by
+// memory (32 bytes per node in FP32): with one value per load the five streams kept too few bytes in
+// flight (95 us for 8.5M nodes, 42 % of the copy rate).
 template <class T>
-__global__ void mg_pcg_update_kernel(int n, PcgVecs<T> v, PcgScalars* sc, const T* par) {
+__global__ void __launch_bounds__(256) mg_pcg_update_kernel(int n, PcgVecs<T> v, PcgScalars* sc, const T* par) {
   if (sc->done) return;
+  constexpr int N = MgPack<T>::N;
   const int t = sc->t;
   const double alpha_d = sc->rz[t & 3] / sc->pAp[t & 3];
   if (!(alpha_d == alpha_d) || alpha_d <= 0.0 || fabs(alpha_d) > 1e300) {
@@ -549,7 +614,23 @@ __global__ void mg_pcg_update_kernel(int n, PcgVecs<T> v, PcgScalars* sc, const 
   const T om = mg_omega<T>(par, 0);
   const T* __restrict__ p = (t & 1) ? v.p[1] : v.p[0];
   T rr = T(0);
-  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < n; idx += gridDim.x * blockDim.x) {
+  const int np = n / N;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < np; i += gridDim.x * blockDim.x) {
+    MgPack<T> x = mg_ldp(v.x, i), r = mg_ldp(v.r, i), d;
+    const MgPack<T> pp = mg_ldp(p, i), ap = mg_ldp(v.Ap, i), di = mg_ldp(v.dinv, i);
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+      x.v[q] += alpha * pp.v[q];
+      r.v[q] -= alpha * ap.v[q];
+      d.v[q] = om * di.v[q] * r.v[q];
+      rr += r.v[q] * r.v[q];
+    }
+    mg_stp(v.x, i, x);
+    mg_stp(v.r, i, r);
+    mg_stp(v.d[0], i, d);
+  }
+  const int idx = N * np + blockIdx.x * blockDim.x + threadIdx.x;  // the last n % N values
+  if (idx < n) {
     v.x[idx] += alpha * p[idx];
     const T r = v.r[idx] - alpha * v.Ap[idx];
     v.r[idx] = r;
@@ -561,20 +642,22 @@ __global__ void mg_pcg_update_kernel(int n, PcgVecs<T> v, PcgScalars* sc, const 
 }
 
 // Restriction to level l+1 of the fine residual wf: b = P^T wf on the coarse free nodes, and
-// the coarse pre-smoothing x = omega D^-1 b.
+// the coarse pre-smoothing x = omega D^-1 b. One plane per blockIdx.y (the z weights are uniform).
 template <class T>
-__global__ void mg_restrict_kernel(const MgLevelDev<T> F, const T* __restrict__ wf, const MgLevelDev<T> C,
-                                   const T* par, int lc, const PcgScalars* sc) {
+__global__ void __launch_bounds__(MG_THREADS) mg_restrict_kernel(const MgLevelDev<T> F, const T* __restrict__ wf,
+                                                                 const MgLevelDev<T> C, const T* par, int lc,
+                                                                 const PcgScalars* sc) {
   if (sc->done) return;
-  const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  const long long nn = (long long)C.nxn * C.nyn * C.nzn;
-  if (n >= nn) return;
-  int I, J, K;
-  node_ijk(C, n, I, J, K);
+  const int plane = C.nxn * C.nyn;
+  const int q = blockIdx.x * MG_THREADS + threadIdx.x;
+  if (q >= plane) return;
+  const int J = q / C.nxn, I = q - J * C.nxn, K = blockIdx.y;
+  const int n = q + plane * K;
+  const MgRestr rx = F.rs[0][I], ry = F.rs[1][J], rz = F.rs[2][K];
+  const T dv = C.dinv[n];
   T b = T(0);
   if (!C.mask[n]) {
-    const MgRestr rx = F.rs[0][I], ry = F.rs[1][J], rz = F.rs[2][K];
-    const int fx[3] = {rx.f0, rx.f1, rx.f2}, fy[3] = {ry.f0, ry.f1, ry.f2}, fz[3] = {rz.f0, rz.f1, rz.f2};
+    const int fy[3] = {ry.f0, ry.f1, ry.f2}, fz[3] = {rz.f0, rz.f1, rz.f2};
     const T wx[3] = {(T)rx.w0, (T)rx.w1, (T)rx.w2}, wy[3] = {(T)ry.w0, (T)ry.w1, (T)ry.w2};
     const T wz[3] = {(T)rz.w0, (T)rz.w1, (T)rz.w2};
 #pragma unroll
@@ -582,15 +665,52 @@ __global__ void mg_restrict_kernel(const MgLevelDev<T> F, const T* __restrict__ 
       if (wz[c] == T(0)) continue;
 #pragma unroll
       for (int bb = 0; bb < 3; ++bb) {
-        if (wy[bb] == T(0)) continue;
-        const long long base = (long long)F.nxn * (fy[bb] + (long long)F.nyn * fz[c]);
+        // an absent neighbour repeats f0 with weight 0: read in any case, so that the loads are independent
+        const T* row = wf + F.nxn * (fy[bb] + F.nyn * fz[c]);
         const T wyz = wy[bb] * wz[c];
-        b += wyz * (wx[0] * wf[base + fx[0]] + wx[1] * wf[base + fx[1]] + wx[2] * wf[base + fx[2]]);
+        b += wyz * (wx[0] * row[rx.f0] + wx[1] * row[rx.f1] + wx[2] * row[rx.f2]);
       }
     }
   }
   C.b[n] = b;
-  C.x[n] = mg_omega<T>(par, lc) * C.dinv[n] * b;
+  C.x[n] = mg_omega<T>(par, lc) * dv * b;
+}
+
+// Coarse correction of level l from the solution ec of level l+1: out = base + P ec on free
+// nodes (base on Dirichlet nodes). A thread takes KZ planes of one column: the 64-bit index divisions
+// and the x and y tables of every node cost more than the interpolation (58 us for 8.5M nodes).
+template <class T, int KZ>
+__global__ void __launch_bounds__(MG_THREADS) mg_prolong_kernel(const MgLevelDev<T> F, const T* __restrict__ ec,
+                                                                const MgLevelDev<T> C, const T* base, T* out,
+                                                                const PcgScalars* sc) {
+  if (sc->done) return;
+  const int plane = F.nxn * F.nyn;
+  const int q = blockIdx.x * MG_THREADS + threadIdx.x;
+  if (q >= plane) return;
+  const int j = q / F.nxn, i = q - j * F.nxn;
+  const MgProl px = F.pr[0][i], py = F.pr[1][j];
+  const int sy = C.nxn, sz = C.nxn * C.nyn;
+  const int a00 = py.c0 * sy + px.c0, a01 = py.c0 * sy + px.c1, a10 = py.c1 * sy + px.c0, a11 = py.c1 * sy + px.c1;
+  const T xw0 = px.w0, xw1 = px.w1, yw0 = py.w0, yw1 = py.w1;
+  T v[KZ];
+  T e[KZ];
+#pragma unroll
+  for (int z = 0; z < KZ; ++z) {
+    const int k = min((int)blockIdx.y * KZ + z, F.nzn - 1);
+    const int n = q + plane * k;
+    const MgProl pz = F.pr[2][k];
+    const T* e0 = ec + pz.c0 * sz;
+    const T* e1 = ec + pz.c1 * sz;
+    v[z] = base[n];
+    const T s0 = yw0 * (xw0 * __ldg(e0 + a00) + xw1 * __ldg(e0 + a01)) + yw1 * (xw0 * __ldg(e0 + a10) + xw1 * __ldg(e0 + a11));
+    const T s1 = yw0 * (xw0 * __ldg(e1 + a00) + xw1 * __ldg(e1 + a01)) + yw1 * (xw0 * __ldg(e1 + a10) + xw1 * __ldg(e1 + a11));
+    e[z] = F.mask[n] ? T(0) : (T)pz.w0 * s0 + (T)pz.w1 * s1;
+  }
+#pragma unroll
+  for (int z = 0; z < KZ; ++z) {
+    const int k = blockIdx.y * KZ + z;
+    if (k < F.nzn) out[q + plane * k] = v[z] + e[z];
+  }
 }
 
 // Residual after pre-smoothing on a coarse level: w = b - A x.
@@ -850,28 +970,44 @@ void mg_setup(qcad_mesh_s* m, cudaStream_t s, bool force) {
   std::deque<MgLevel>& L = H->L;
   const PcgBufs<T>& k = mesh_bufs<T>(m);
   T* par = H->par[p].template as<T>();
+  const int nl = (int)L.size();
+  auto Sl = [&](int l) { return H->Sl[p][l].template as<T>(); };
+  auto resp = [&](int l) { return H->resp[p][l].template as<unsigned char>(); };
   if (!H->stiff_ok[p]) {
-    H->S1[p].ensure((size_t)64 * L[1].ne * sizeof(T) + 64);
     H->ra0[p].ensure((size_t)L[0].n * sizeof(T) + 64);
-    mg_gersh0_kernel<T, true><<<blocks_for(L[0].n), MG_THREADS, 0, s>>>(
-        mesh_grid<T>(m), nullptr, level_dev<T>(L[0]), k.dinv.template as<T>(), H->ra0[p].template as<T>(), nullptr);
-    mg_galerkin0_kernel<T, true><<<blocks_for(L[1].ne, 128), 128, 0, s>>>(
-        mesh_grid<T>(m), nullptr, nullptr, level_dev<T>(L[0]), level_dev<T>(L[1]), H->S1[p].template as<T>());
-    note_launch(2);
+    mg_gersh0_kernel<T, true><<<blocks_for(L[0].n), MG_THREADS, 0, s>>>(mesh_grid<T>(m), nullptr, nullptr,
+                                                                        level_dev<T>(L[0]), k.dinv.template as<T>(),
+                                                                        H->ra0[p].template as<T>(), nullptr);
+    for (int l = 1; l < nl; ++l) {
+      H->Sl[p][l].ensure((size_t)64 * L[l].ne * sizeof(T) + 64);
+      H->resp[p][l].ensure((size_t)L[l].ne + 64);
+      CK(cudaMemsetAsync(H->resp[p][l].p, 1, (size_t)L[l].ne, s));
+      const int blocks = blocks_for(8 * L[l].ne, 128);
+      if (l == 1)
+        mg_galerkin0_kernel<T, true><<<blocks, 128, 0, s>>>(mesh_grid<T>(m), nullptr, nullptr, nullptr, nullptr,
+                                                            level_dev<T>(L[0]), level_dev<T>(L[1]), Sl(1));
+      else
+        mg_galerkin_kernel<T, true><<<blocks, 128, 0, s>>>(level_dev<T>(L[l - 1]), Sl(l - 1), nullptr, nullptr, nullptr,
+                                                           level_dev<T>(L[l]), Sl(l));
+    }
+    note_launch(nl);
     CK(cudaGetLastError());
     H->stiff_ok[p] = true;
   }
+  const unsigned char* act = k.act.template as<unsigned char>();
   CK(cudaMemsetAsync(par, 0, MG_MAX_LEVELS * sizeof(T), s));
   mg_gersh0_kernel<T, false><<<blocks_for(L[0].n), MG_THREADS, 0, s>>>(
-      mesh_grid<T>(m), k.c.template as<T>(), level_dev<T>(L[0]), k.dinv.template as<T>(), H->ra0[p].template as<T>(),
-      par);
-  mg_galerkin0_kernel<T, false><<<blocks_for(L[1].ne, 128), 128, 0, s>>>(
-      mesh_grid<T>(m), k.c.template as<T>(), H->S1[p].template as<T>(), level_dev<T>(L[0]), level_dev<T>(L[1]),
-      L[1].A[p].template as<T>());
-  for (size_t l = 1; l < L.size(); ++l) {
-    if (l > 1)
-      mg_galerkin_kernel<T><<<blocks_for(L[l].ne, 128), 128, 0, s>>>(level_dev<T>(L[l - 1]), level_dev<T>(L[l]),
-                                                                     L[l].A[p].template as<T>());
+      mesh_grid<T>(m), k.c.template as<T>(), act, level_dev<T>(L[0]), k.dinv.template as<T>(),
+      H->ra0[p].template as<T>(), par);
+  for (int l = 1; l < nl; ++l) {
+    const int blocks = blocks_for(8 * L[l].ne, 128);
+    T* A = L[l].A[p].template as<T>();
+    if (l == 1)
+      mg_galerkin0_kernel<T, false><<<blocks, 128, 0, s>>>(mesh_grid<T>(m), k.c.template as<T>(), act, Sl(1), resp(1),
+                                                           level_dev<T>(L[0]), level_dev<T>(L[1]), A);
+    else
+      mg_galerkin_kernel<T, false><<<blocks, 128, 0, s>>>(level_dev<T>(L[l - 1]), L[l - 1].A[p].template as<T>(),
+                                                          resp(l - 1), Sl(l), resp(l), level_dev<T>(L[l]), A);
     mg_diag_kernel<T><<<blocks_for(L[l].n), MG_THREADS, 0, s>>>(level_dev<T>(L[l]), L[l].dinv[p].template as<T>(),
                                                                 par + l);
   }
@@ -881,6 +1017,17 @@ void mg_setup(qcad_mesh_s* m, cudaStream_t s, bool force) {
 }
 template void mg_setup<float>(qcad_mesh_s*, cudaStream_t, bool);
 template void mg_setup<double>(qcad_mesh_s*, cudaStream_t, bool);
+
+template <class T>
+static void launch_prolong(const MgLevelDev<T>& F, const T* ec, const MgLevelDev<T>& C, const T* base, T* out,
+                           const PcgScalars* sc, cudaStream_t s) {
+  const int bx = blocks_for((long long)F.nxn * F.nyn);
+  // four planes per thread where that leaves the SMs four blocks each
+  if ((long long)bx * F.nzn >= 16LL * sm_count())
+    note_launch(), mg_prolong_kernel<T, 4><<<dim3(bx, (F.nzn + 3) / 4), MG_THREADS, 0, s>>>(F, ec, C, base, out, sc);
+  else
+    note_launch(), mg_prolong_kernel<T, 1><<<dim3(bx, F.nzn), MG_THREADS, 0, s>>>(F, ec, C, base, out, sc);
+}
 
 // V-cycle after the level-0 pre-smoothing (zp in d[0]): ends with z and the PCG bookkeeping.
 template <class T>
@@ -893,26 +1040,25 @@ static void enqueue_vcycle(qcad_mesh_s* m, const PcgVecs<T>& v, PcgScalars* sc, 
   launch_mg_resid0<T>(mesh_grid<T>(m), v, sc, mesh_cfg<T>(m), s);
   for (int l = 0; l + 1 < nl; ++l) {
     const T* wf = l == 0 ? v.w : L[l].w[p].template as<T>();
-    note_launch(), mg_restrict_kernel<T><<<blocks_for(L[l + 1].n), MG_THREADS, 0, s>>>(
-                       level_dev<T>(L[l]), wf, level_dev<T>(L[l + 1]), par, l + 1, sc);
+    const MgLevelDev<T>& c = level_dev<T>(L[l + 1]);
+    note_launch(), mg_restrict_kernel<T><<<dim3(blocks_for((long long)c.nxn * c.nyn), c.nzn), MG_THREADS, 0, s>>>(
+                       level_dev<T>(L[l]), wf, c, par, l + 1, sc);
     if (l + 1 < nl - 1)
-      note_launch(), mg_resid_kernel<T><<<blocks_for(L[l + 1].n), MG_THREADS, 0, s>>>(level_dev<T>(L[l + 1]), sc);
+      note_launch(), mg_resid_kernel<T><<<blocks_for(L[l + 1].n), MG_THREADS, 0, s>>>(c, sc);
   }
   const MgLevel& co = L[nl - 1];
   const int smem = (int)coarse_smem_bytes(co, sizeof(T));
   note_launch(), mg_coarse_kernel<T><<<1, MG_COARSE_NODES, smem, s>>>(level_dev<T>(L[nl - 1]), par, nl - 1, sc);
   for (int l = nl - 2; l >= 1; --l) {
-    note_launch(), mg_prolong_kernel<T><<<blocks_for(L[l].n), MG_THREADS, 0, s>>>(
-                       level_dev<T>(L[l]), L[l + 1].w[p].template as<T>(), level_dev<T>(L[l + 1]),
-                       level_dev<T>(L[l]).x, level_dev<T>(L[l]).x, sc);
-    note_launch(), mg_post_kernel<T><<<blocks_for(L[l].n), MG_THREADS, 0, s>>>(level_dev<T>(L[l]), par, l, sc);
+    const MgLevelDev<T>& f = level_dev<T>(L[l]);
+    launch_prolong<T>(f, L[l + 1].w[p].template as<T>(), level_dev<T>(L[l + 1]), f.x, f.x, sc, s);
+    note_launch(), mg_post_kernel<T><<<blocks_for(L[l].n), MG_THREADS, 0, s>>>(f, par, l, sc);
   }
-  note_launch(), mg_prolong_kernel<T><<<blocks_for(L[0].n), MG_THREADS, 0, s>>>(
-                     level_dev<T>(L[0]), L[1].w[p].template as<T>(), level_dev<T>(L[1]), v.d[0], v.d[1], sc);
+  launch_prolong<T>(level_dev<T>(L[0]), L[1].w[p].template as<T>(), level_dev<T>(L[1]), v.d[0], v.d[1], sc, s);
   launch_mg_post0<T>(mesh_grid<T>(m), v, sc, par, mesh_cfg<T>(m), s);
 }
 
-static int vec_grid(long long n) { return (int)std::min<long long>(4 * 152, std::max<long long>(1, (n + 255) / 256)); }
+static int vec_grid(long long n) { return (int)std::min<long long>(4 * 152, std::max<long long>(1, (n + 255) / 256)); }  // 4 blocks per SM
 
 template <class T>
 void mg_enqueue_init(qcad_mesh_s* m, const PcgVecs<T>& v, PcgScalars* sc, cudaStream_t s) {

@@ -55,6 +55,13 @@ template <> struct Prec<float> {
   static const int prof_apply = PROF_APPLY32, prof_update = PROF_UPDATE32;
 };
 
+// Bytes of a PCG vector, a multiple of 16: the second halves of p and d start aligned for the vector
+// loads of the update kernels.
+template <class T>
+static size_t vec_bytes(long long n) {
+  return ((size_t)n * sizeof(T) + 79) / 16 * 16;
+}
+
 // Size of a linearization's activity map.
 static size_t act_bytes(const qcad_mesh_s* m) {
   return (size_t)act_cells(m->nx, ACT_X) * act_cells(m->ny, ACT_Y) * act_cells(m->nz, ACT_Z);
@@ -63,7 +70,7 @@ static size_t act_bytes(const qcad_mesh_s* m) {
 template <class T>
 static PcgVecs<T> ensure_pcg(qcad_mesh_s* m) {
   PcgBufs<T>& b = Prec<T>::bufs(m);
-  const size_t nb = (size_t)m->n_nodes * sizeof(T) + 64;
+  const size_t nb = vec_bytes<T>(m->n_nodes);
   b.x.ensure(nb);
   b.r.ensure(nb);
   b.z.ensure(nb);
@@ -1107,7 +1114,7 @@ static void adjoint_solve_mixed(qcad_mesh_s* m, int nd, const double* G, double*
     BatchCtx& B = ctx->B;
     B.n = nd;
     B.s = s;
-    const size_t nb = (size_t)n * sizeof(float) + 64;
+    const size_t nb = vec_bytes<float>(n);
     for (int d = 0; d < nd; ++d) {
       PcgVecs<float> v = w0;
       if (d > 0) {
@@ -1383,7 +1390,7 @@ qcad_status adjoint_batch(int n, const qcad_mesh_t* ms, const qcad_bias* bs, con
   auto vecs_for = [&](qcad_mesh_s* m, int d) {
     PcgVecs<float> v = ensure_pcg<float>(m);
     if (d == 0) return v;
-    const size_t nb = (size_t)m->n_nodes * sizeof(float) + 64;
+    const size_t nb = vec_bytes<float>(m->n_nodes);
     PcgBufs<float>& k = m->k32x[d - 1];
     k.x.ensure(nb);
     k.r.ensure(nb);

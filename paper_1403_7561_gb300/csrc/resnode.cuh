@@ -189,6 +189,7 @@ __device__ __forceinline__ void residual_node_body(const Grid<double>& g, const 
     top[r] = wr[r] && g.dir_top != nullptr && g.dir_top[nrow[r + 1]] != 0;
     half[r] = (i == 0 || i == g.nx) + (j == 0 || j == g.ny);
   }
+  const bool edge = __any_sync(FULL_MASK, (half[0] | half[1]) != 0);  // a boundary tile
   // load codes of the elements (i, jb-1 .. jb+1) of a layer, a byte each; 255: no element
   const int eplane = g.nx * g.ny;
   auto codes = [&](int layer) {
@@ -226,8 +227,8 @@ __device__ __forceinline__ void residual_node_body(const Grid<double>& g, const 
       const double xs = __shfl_up_sync(FULL_MASK, c2[0][r], 1) + __shfl_down_sync(FULL_MASK, c2[0][r], 1);
       if (!wr[r]) continue;
       const int n = nrow[r + 1] + k * plane;
-      double R = c1[0][r] + (xs - 2.0 * c2[0][r]);
-      if (half[r] != 0) R *= half[r] == 1 ? 0.5 : 0.25;
+      double R = c1[0][r] + fma(-2.0, c2[0][r], xs);
+      if (edge) R *= half[r] == 0 ? 1.0 : half[r] == 1 ? 0.5 : 0.25;
       R += up[r] + lo[r];
       const bool dir = pdir || (k == g.nz && top[r]);
       if (dir) R = 0.0;
@@ -246,7 +247,7 @@ __device__ __forceinline__ void residual_node_body(const Grid<double>& g, const 
         if (a.dinv64) a.dinv64[n] = dir ? 1.0 : rs ? 1.0 / dg : __ldg(g.zs + 12 * k + 11) * (half[r] == 0 ? 1.0 : half[r] == 1 ? 2.0 : 4.0);
         if (a.dinv32 && rs) a.dinv32[n] = __frcp_rn(__double2float_rn(dg));
       }
-      acc_r2 += R * R;
+      acc_r2 = fma(R, R, acc_r2);
       // max |R| by bit pattern (NaN left out, as fmax does)
       const unsigned long long b = (unsigned long long)__double_as_longlong(R) & 0x7fffffffffffffffull;
       if (b <= 0x7ff0000000000000ull && b > acc_max) acc_max = b;
@@ -267,16 +268,16 @@ __device__ __forceinline__ void residual_node_body(const Grid<double>& g, const 
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
       const double c = v[r + 1];
-      const double dy = (v[r] + v[r + 2]) - 2.0 * c;
+      const double dy = fma(-2.0, c, v[r] + v[r + 2]);
 #pragma unroll
       for (int o = 0; o < 3; ++o) {
-        c1[o][r] += z[3 * o] * dy;
-        c2[o][r] += z[3 * o + 1] * c;
-        c2[o][r] += z[3 * o + 2] * dy;
+        c1[o][r] = fma(z[3 * o], dy, c1[o][r]);
+        c2[o][r] = fma(z[3 * o + 1], c, c2[o][r]);
+        c2[o][r] = fma(z[3 * o + 2], dy, c2[o][r]);
       }
       const double d = k > kb ? c - cold[r] : 0.0;
-      c1[0][r] -= z[9] * d;
-      c1[1][r] += z[9] * d;
+      c1[0][r] = fma(-z[9], d, c1[0][r]);
+      c1[1][r] = fma(z[9], d, c1[1][r]);
     }
     if (k > kb) {
       if (k < ke) cn = codes(k);
