@@ -61,11 +61,20 @@ static LaunchCfg fit_lin(int nxn, int nyn, int nzn, int nvec, LaunchCfg cfg) {
   return out;
 }
 
+template <class T>
+static bool has_act(const ApplyOp<T>& op) { return op.a.act != nullptr; }
+template <class Op>
+static bool has_act(const Op& op) { return op.v.act != nullptr; }
+
 // Supported (warps, rows per thread): FP32 4/8/16/32 x 1 and 4/8/16 x 2; FP64 4/8 x 1 and
 // 4/8 x 2 (shared memory). Other requests are clamped to the nearest supported shape.
 template <class T, class Op>
 static void run_lin(const Grid<T>& g, const Op& op, LaunchCfg cfg, cudaStream_t s) {
   cfg = fit_lin<T>(g.nxn, g.nyn, g.nzn, 1, cfg);
+  // With an activity map a tile with response takes about six times as long as one without in FP64, so
+  // the longest tile sets the time: half the chunk (FP64 solve of the 128 x 128 x 96 device 75 -> 67 ms;
+  // FP32, bound by latency, was 5 % slower with it).
+  if (sizeof(T) == 8 && cfg.fit && cfg.variant >= 2 && has_act(op) && cfg.kchunk > 8) cfg.kchunk = 8;
   const int kc = cfg.kchunk > 0 ? (cfg.kchunk < 128 ? cfg.kchunk : 128) : 16;  // LinShape::ZMAX
   const bool two = cfg.variant == 3;
   if constexpr (std::is_same<T, float>::value) {

@@ -75,6 +75,9 @@ __device__ __forceinline__ void lin_lds_c8<double>(const uint4* p, double* c) {
   }
 }
 
+// Nonzero, by the bit pattern (an FP64 comparison would take the FP64 pipe).
+__device__ __forceinline__ bool lin_nonzero(double c) { return (__double_as_longlong(c) << 1) != 0; }
+
 // Packed row-exchange values (one shared access per pair or quadruple).
 template <class T>
 struct alignas(2 * sizeof(T)) LinV2 {
@@ -108,22 +111,31 @@ inline dim3 lin_grid(int nxn, int nyn, int nzn, int by, int r, int kchunk, int n
   return dim3((nxn + 29) / 30, (nyn + tr - 3) / (tr - 2), ((nzn + kchunk - 1) / kchunk) * nvec);
 }
 
-// True when some cell of the activity map that the tile's output nodes touch is active (all threads).
+// Activity of a tile's planes in groups of ACT_Z (group q: planes ACT_Z (k0 / ACT_Z + q) and up): bit q is
+// set when some element that touches a node of the tile on these planes lies in an active cell. A
+// plane touches the layers below and above it, so a group sees its own cell layer and the one before.
+// All threads call it; two barriers.
 template <class T, int BY, int R>
-__device__ __forceinline__ bool tile_active(const Grid<T>& g, const unsigned char* act, int bx, int by, int k0,
-                                            int k1) {
+__device__ __forceinline__ unsigned long long tile_activity(const Grid<T>& g, const unsigned char* act, int bx, int by,
+                                                            int k0, int k1) {
+  __shared__ unsigned cells[2];
   constexpr int TR = BY * R;
-  const int nax = act_cells(g.nx, ACT_X), nay = act_cells(g.ny, ACT_Y);
+  const int tid = threadIdx.x + 32 * threadIdx.y;
+  if (tid < 2) cells[tid] = 0;
+  __syncthreads();
+  const int nax = act_cells(g.nx, ACT_X), nay = act_cells(g.ny, ACT_Y), naz = act_cells(g.nz, ACT_Z);
   const int i0 = max(bx * 30 - 1, 0) / ACT_X, i1 = min(bx * 30 + 29, g.nx - 1) / ACT_X;
   const int j0 = max(by * (TR - 2) - 1, 0) / ACT_Y, j1 = min(by * (TR - 2) + TR - 3, g.ny - 1) / ACT_Y;
-  const int l0 = max(k0 - 1, 0) / ACT_Z, l1 = min(k1 - 1, g.nz - 1) / ACT_Z;
+  // cell layers from the one before the first group's; bit 0 is that one (at most 34: 128 planes)
+  const int l0 = k0 / ACT_Z - 1, l1 = min((k1 - 1) / ACT_Z, naz - 1);
   const int ni = i1 - i0 + 1, nj = j1 - j0 + 1, nc = ni * nj * (l1 - l0 + 1);
-  int any = 0;
-  for (int q = threadIdx.x + 32 * threadIdx.y; q < nc; q += 32 * BY) {
-    const int i = i0 + q % ni, r = q / ni;
-    any |= act[i + nax * (j0 + r % nj + (long long)nay * (l0 + r / nj))];
+  for (int q = tid; q < nc; q += 32 * BY) {
+    const int i = i0 + q % ni, r = q / ni, l = r / nj;
+    if (l0 + l >= 0 && act[i + nax * (j0 + r % nj + (long long)nay * (l0 + l))] != 0) atomicOr(&cells[l >> 5], 1u << (l & 31));
   }
-  return __syncthreads_or(any) != 0;
+  __syncthreads();
+  const unsigned long long m = cells[0] | ((unsigned long long)cells[1] << 32);
+  return m | (m >> 1);  // group q: cell layers q (the one before) and q + 1, shifted to bit q
 }
 
 // The march of a tile without charge response (every coefficient zero): y = K v alone, the separable
@@ -252,14 +264,18 @@ __device__ __forceinline__ void lin_body(const Grid<T>& g, const Op& op_in, int 
                                          unsigned char* dyn) {
   using S = LinShape<T, BY, R>;
   constexpr int TR = S::TR, NCH = S::NCH, NST = S::NST;
+  constexpr bool SKIP = std::is_same<T, double>::value;
   if (op_in.skip()) return;
   const int nch = (g.nzn + kchunk - 1) / kchunk;
   Op op = op_in;
   op.set_vec(bz / nch);
+  const int c0 = (bz % nch) * kchunk, c1 = min(c0 + kchunk, g.nzn);
+  // planes of the chunk whose elements respond, by groups; without a map all of them
+  unsigned long long resp = ~0ull;
   if constexpr (!Op::SEPM) {
     if (g.zs != nullptr && op.act() != nullptr) {
-      const int c0 = (bz % nch) * kchunk, c1 = min(c0 + kchunk, g.nzn);
-      if (!tile_active<T, BY, R>(g, op.act(), bx, by, c0, c1)) {
+      resp = tile_activity<T, BY, R>(g, op.act(), bx, by, c0, c1);
+      if ((resp & ((2ull << ((c1 - 1) / ACT_Z - c0 / ACT_Z)) - 1)) == 0) {
         stiff_body<T, BY, R, Op>(g, op, bx, by, c0, c1);
         op.finish();
         return;
@@ -281,9 +297,6 @@ __device__ __forceinline__ void lin_body(const Grid<T>& g, const Op& op_in, int 
   const int tyu = min(ty + 1, BY - 1), tyd = max(ty - 1, 0);
   const int i = bx * 30 - 1 + lane;
   const int jb = by * (TR - 2) - 1 + ty * R;
-  const int k0 = (bz % nch) * kchunk;
-  const int k1 = min(k0 + kchunk, g.nzn);
-  const int kmax = min(k1, g.nzn - 1);  // last plane the chunk reads
   const int plane = (int)g.plane;
   const T A = GaussConst<T>::a(), B = GaussConst<T>::b();
   const T* __restrict__ cg = op.coeffs();
@@ -320,6 +333,23 @@ __device__ __forceinline__ void lin_body(const Grid<T>& g, const Op& op_in, int 
     }
   }
   const int eplane = g.nx * g.ny;
+
+  // the chunk in runs of planes with and without response (one run when there is no map)
+  for (int k0 = c0, k1; k0 < c1; k0 = k1) {
+  {
+    const int gb = c0 / ACT_Z;
+    int q = k0 / ACT_Z - gb;
+    const bool on = (resp >> q) & 1;
+    while ((gb + q + 1) * ACT_Z < c1 && (((resp >> (q + 1)) & 1) != 0) == on) ++q;
+    k1 = min((gb + q + 1) * ACT_Z, c1);
+    if constexpr (!Op::SEPM) {
+      if (!on) {
+        stiff_body<T, BY, R, Op>(g, op, bx, by, k0, k1);
+        continue;
+      }
+    }
+  }
+  const int kmax = min(k1, g.nzn - 1);  // last plane the run reads
 
   // one copy group: the raw inputs of node plane vplane (if >= 0; clamped into the chunk's
   // planes) and the coefficients of element layer `layer`, zeros where the element does not
@@ -402,6 +432,7 @@ __device__ __forceinline__ void lin_body(const Grid<T>& g, const Op& op_in, int 
     }
   }
   T carry[R][4];
+  bool cnz = k0 > 0;  // the warp's carry may be nonzero
 #pragma unroll
   for (int r = 0; r < R; ++r)
 #pragma unroll
@@ -440,23 +471,48 @@ __device__ __forceinline__ void lin_body(const Grid<T>& g, const Op& op_in, int 
     lin_cp_wait<2>();
     const uint4* st = cst + (size_t)(k % NST) * (TR * NCH * 32);
     T Ylo[R][2], Yhi[R][2];
+    T c[R][8];
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      T c[8];
-      lin_lds_c8<T>(st + ((ty * R + r) * NCH) * 32 + lane, c);
-      T W[4];
+    for (int r = 0; r < R; ++r) lin_lds_c8<T>(st + ((ty * R + r) * NCH) * 32 + lane, c[r]);
+    // FP64: a warp whose elements of this layer have no response passes the carry on or skips the layer
+    // (in FP32 the test cost more than the operations it saved)
+    bool nz = true;
+    if constexpr (SKIP) {
+      nz = false;
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const T w0 = c[q] * (A * Uc[r][q] + B * Un[r][q]);
-        const T w1 = c[q + 4] * (B * Uc[r][q] + A * Un[r][q]);
-        W[q] = carry[r][q] + A * w0 + B * w1;
-        carry[r][q] = B * w0 + A * w1;
-      }
-      Ylo[r][0] = A * W[0] + B * W[2];
-      Ylo[r][1] = A * W[1] + B * W[3];
-      Yhi[r][0] = B * W[0] + A * W[2];
-      Yhi[r][1] = B * W[1] + A * W[3];
+      for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int q = 0; q < 8; ++q) nz = nz || lin_nonzero(c[r][q]);
+      nz = __any_sync(FULL_MASK, nz);
     }
+    if (nz || cnz) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        T W[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) W[q] = carry[r][q];
+        if (nz) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const T w0 = c[r][q] * (A * Uc[r][q] + B * Un[r][q]);
+            const T w1 = c[r][q + 4] * (B * Uc[r][q] + A * Un[r][q]);
+            W[q] = W[q] + A * w0 + B * w1;
+            carry[r][q] = B * w0 + A * w1;
+          }
+        } else {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) carry[r][q] = T(0);
+        }
+        Ylo[r][0] = A * W[0] + B * W[2];
+        Ylo[r][1] = A * W[1] + B * W[3];
+        Yhi[r][0] = B * W[0] + A * W[2];
+        Yhi[r][1] = B * W[1] + A * W[3];
+      }
+    } else {
+#pragma unroll
+      for (int r = 0; r < R; ++r) Ylo[r][0] = Ylo[r][1] = Yhi[r][0] = Yhi[r][1] = T(0);
+    }
+    cnz = nz;
     xch_y[P][ty][lane] = LinV2<T>{Yhi[R - 1][0], Yhi[R - 1][1]};
     // stiffness, z stage
     T z[12];
@@ -551,6 +607,8 @@ __device__ __forceinline__ void lin_body(const Grid<T>& g, const Op& op_in, int 
   }
   if (k < k1) step(k, std::integral_constant<int, 0>());
   lin_cp_wait<0>();
+  __syncthreads();  // the next run refills the shared buffers
+  }
   op.finish();
 }
 
