@@ -176,15 +176,33 @@ __device__ __forceinline__ void stiff_body(const Grid<T>& g, Op& op, int bx, int
   const int kb = max(k0 - 1, 0), ke = min(k1, g.nzn - 1);
   const T* s0 = op.lin_src(0);
   const T* s1 = Op::NIN > 1 ? op.lin_src(1) : s0;
-  T raw[Op::NIN][4];
-  auto fetch = [&](int k) {
+  // A warp's plane takes far less than a memory access: the inputs of three planes and the epilogue's
+  // data of two are in flight (slot of plane k: (k - kb) % 3).
+  constexpr int PF = 3;
+  T raw[PF][Op::NIN][4];
+  typename Op::Pre pre[PF][2];
+  auto fetch = [&](int k, auto Sc) {
+    constexpr int Q = decltype(Sc)::value;
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
-      raw[0][r] = s0[nrow[r] + k * plane];
-      if (Op::NIN > 1) raw[Op::NIN - 1][r] = s1[nrow[r] + k * plane];
+      raw[Q][0][r] = s0[nrow[r] + k * plane];
+      if (Op::NIN > 1) raw[Q][Op::NIN - 1][r] = s1[nrow[r] + k * plane];
     }
   };
-  fetch(kb);
+  auto fetch_pre = [&](int k, auto Sc) {  // of output plane k, when the run has it
+    constexpr int Q = decltype(Sc)::value;
+    if (k < k0 || k >= k1) return;
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+      if (wr[r]) pre[Q][r] = op.lin_pre(nrow[r + 1] + k * plane);
+  };
+  using I0 = std::integral_constant<int, 0>;
+  using I1 = std::integral_constant<int, 1>;
+  using I2 = std::integral_constant<int, 2>;
+  fetch(kb, I0());
+  fetch(min(kb + 1, ke), I1());
+  fetch(min(kb + 2, ke), I2());
+  fetch_pre(kb, I0());
   T c1[3][2], c2[3][2], cold[2];
 #pragma unroll
   for (int r = 0; r < 2; ++r) {
@@ -192,27 +210,23 @@ __device__ __forceinline__ void stiff_body(const Grid<T>& g, Op& op, int bx, int
     for (int o = 0; o < 3; ++o) c1[o][r] = c2[o][r] = T(0);
     cold[r] = T(0);
   }
-  auto put = [&](int k, const typename Op::Pre* pre) {  // output plane k from the oldest sums
+  auto put = [&](int k, const typename Op::Pre* q) {  // output plane k from the oldest sums
     const bool pdir = dov && ((g.dir_bottom && k == 0) || (g.dir_boundary && (k == 0 || k == g.nz)));
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
       const T up = __shfl_up_sync(FULL_MASK, c2[0][r], 1), dn = __shfl_down_sync(FULL_MASK, c2[0][r], 1);
       const T y = f[r] * (c1[0][r] + ((up + dn) - T(2) * c2[0][r]));
       const bool isdir = pdir || bnd[r] || (k == g.nz && top[r]);
-      if (wr[r]) op.lin_out(nrow[r + 1] + k * plane, pre[r], cold[r], isdir ? cold[r] : y);
+      if (wr[r]) op.lin_out(nrow[r + 1] + k * plane, q[r], cold[r], isdir ? cold[r] : y);
     }
   };
-  for (int k = kb; k <= ke; ++k) {
+  auto step = [&](int k, auto Sc) {
+    constexpr int Q = decltype(Sc)::value;
     T v[4];
 #pragma unroll
-    for (int r = 0; r < 4; ++r) v[r] = op.lin_mix(raw[0][r], raw[Op::NIN - 1][r]);
-    if (k < ke) fetch(k + 1);
-    typename Op::Pre pre[2];
-    if (k - 1 >= k0) {
-#pragma unroll
-      for (int r = 0; r < 2; ++r)
-        if (wr[r]) pre[r] = op.lin_pre(nrow[r + 1] + (k - 1) * plane);
-    }
+    for (int r = 0; r < 4; ++r) v[r] = op.lin_mix(raw[Q][0][r], raw[Q][Op::NIN - 1][r]);
+    if (k + PF <= ke) fetch(k + PF, Sc);
+    fetch_pre(k + 1, std::integral_constant<int, (Q + 1) % PF>());
     // a1, a2, a3 towards the output planes k-1, k, k+1, then the flux weight of the layer below plane k
     T z[10];
 #pragma unroll
@@ -231,7 +245,7 @@ __device__ __forceinline__ void stiff_body(const Grid<T>& g, Op& op, int bx, int
       c1[0][r] -= z[9] * d;
       c1[1][r] += z[9] * d;
     }
-    if (k - 1 >= k0) put(k - 1, pre);
+    if (k - 1 >= k0) put(k - 1, pre[(Q + 2) % PF]);
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
       cold[r] = v[r + 1];
@@ -242,14 +256,22 @@ __device__ __forceinline__ void stiff_body(const Grid<T>& g, Op& op, int bx, int
       }
       c1[2][r] = c2[2][r] = T(0);
     }
+  };
+  int k = kb;
+  for (; k + 2 <= ke; k += 3) {
+    step(k, I0());
+    step(k + 1, I1());
+    step(k + 2, I2());
   }
+  if (k <= ke) step(k++, I0());
+  if (k <= ke) step(k++, I1());
   if (k1 == g.nzn) {
     // the top plane has no plane above it
-    typename Op::Pre pre[2];
+    typename Op::Pre last[2];
 #pragma unroll
     for (int r = 0; r < 2; ++r)
-      if (wr[r]) pre[r] = op.lin_pre(nrow[r + 1] + (k1 - 1) * plane);
-    put(k1 - 1, pre);
+      if (wr[r]) last[r] = op.lin_pre(nrow[r + 1] + (k1 - 1) * plane);
+    put(k1 - 1, last);
   }
 }
 
