@@ -346,6 +346,21 @@ __global__ void __launch_bounds__(128) hm_rows_kernel(const double* __restrict__
   }
 }
 
+__global__ void __launch_bounds__(256) hm_jacobi_kernel(int nxn, int nyn, int nzn, const double* __restrict__ dk,
+                                                        double* dinv, unsigned char* interior) {
+  const int p = blockIdx.x * 256 + threadIdx.x, k = blockIdx.y;
+  if (p >= nxn * nyn) return;
+  const int j = p / nxn, i = p - j * nxn;
+  const bool in = i > 0 && j > 0 && k > 0 && i < nxn - 1 && j < nyn - 1 && k < nzn - 1;
+  dinv[p + k * nxn * nyn] = in ? 1.0 / dk[k] : 0.0;
+  interior[p + k * nxn * nyn] = in ? 1 : 0;
+}
+void launch_hm_jacobi(int nxn, int nyn, int nzn, const double* dk, double* dinv, unsigned char* interior,
+                      cudaStream_t s) {
+  note_launch();
+  hm_jacobi_kernel<<<dim3((nxn * nyn + 255) / 256, nzn), 256, 0, s>>>(nxn, nyn, nzn, dk, dinv, interior);
+}
+
 void launch_hm_rows(const double* cV, int nxn, int nyn, int nzn, double* mom, float* S32, float2* Sdf, double* S64,
                     cudaStream_t s) {
   const int ne = (nxn - 1) * (nyn - 1) * (nzn - 1), ns = nxn * nyn * nzn;

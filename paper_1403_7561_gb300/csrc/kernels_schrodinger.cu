@@ -17,61 +17,6 @@
 
 namespace qcad {
 
-// H X and M X for nvec vectors in one z-march: field 0 = H (kinetic stencil
-// with kappa_d = hbar^2/(2 m_d) plus the V mass term), field 1 = M (consistent
-// mass). psi = 0 on the subdomain boundary: outputs there are zero.
-template <class T>
-struct HmOp {
-  static constexpr int NF = 2;
-  static constexpr bool STIFF = true;
-  using ED = C8<T>;
-  HmArgs<T> a;
-  int vec;
-  __device__ bool skip() const { return false; }
-  __device__ void set_vec(int v) { vec = v; }
-  __device__ T load(const Grid<T>&, int n, bool in, int, int, int) const {
-    return in ? a.x[(long long)vec * a.ld + n] : T(0);
-  }
-  __device__ ED edata(const Grid<T>& g, int i, int j, int k) const {
-    ED r;
-    load_c8<T>(a.cV, i + g.nx * (j + g.ny * k), r.c);
-    return r;
-  }
-  __device__ void elem(const Grid<T>& g, int i, int j, int k, const T* v, const ED& ed, T (*out)[8], bool) const {
-    qp_mass<T>(v, ed.c, out[0]);
-    const T wdet = g.hx[i] * g.hy[j] * g.hz[k] * T(0.125);
-    T u[8];
-    tp_apply(v, u, GaussConst<T>::a(), GaussConst<T>::b());
-#pragma unroll
-    for (int q = 0; q < 8; ++q) u[q] *= wdet;
-    tp_apply(u, out[1], GaussConst<T>::a(), GaussConst<T>::b());
-  }
-  __device__ void node(const Grid<T>& g, int n, int i, int j, int k, T, T stiff, const T* mass) {
-    const bool bd = grid_is_dir(g, i, j, k);
-    const long long o = (long long)vec * a.ld + n;
-    if (a.hx) a.hx[o] = bd ? T(0) : stiff + mass[0];
-    if (a.mx) a.mx[o] = bd ? T(0) : mass[1];
-  }
-  __device__ void finish() {}
-};
-
-template <class T>
-void launch_hm_apply(const Grid<T>& g, const HmArgs<T>& args, LaunchCfg cfg, cudaStream_t s) {
-  if (cfg.variant >= 2) {
-    launch_hm_apply_lin<T>(g, args, cfg, s);
-    return;
-  }
-  HmOp<T> op = {};
-  op.a = args;
-  const int by = cfg.by == 4 ? 4 : 8;
-  dim3 grid = march_grid(g.nxn, g.nyn, g.nzn, by, cfg.kchunk, args.nvec);
-  if (by == 4)
-    note_launch(), march_kernel<T, 4, HmOp<T>><<<grid, dim3(QCAD_BX, 4), 0, s>>>(g, op, cfg.kchunk);
-  else
-    note_launch(), march_kernel<T, 8, HmOp<T>><<<grid, dim3(QCAD_BX, 8), 0, s>>>(g, op, cfg.kchunk);
-}
-template void launch_hm_apply<double>(const Grid<double>&, const HmArgs<double>&, LaunchCfg, cudaStream_t);
-
 constexpr int DT = 256;
 static int dblocks(long long n) {
   long long b = (n + DT - 1) / DT;

@@ -275,9 +275,7 @@ __device__ __forceinline__ void stiff_body(const Grid<T>& g, Op& op, int bx, int
   }
 }
 
-// Op: the linear ops of pcg_ops.cuh (lin_in, lin_out, lin_dir, skip, set_vec, finish, coeffs),
-// or an op with SEPM = true (m_scale, lin_out2), which writes the operator with zero Dirichlet
-// rows and, as a second output, the separable consistent mass (Schrodinger H and M).
+// Op: the linear ops of pcg_ops.cuh (lin_in, lin_out, lin_dir, skip, set_vec, finish, coeffs, act).
 // Loads are unpredicated: node indices are clamped into the mesh (and into the chunk's
 // planes), and every value read outside the operator's support meets a zero table entry or
 // a zero coefficient, so only finiteness of the input matters there.
@@ -294,14 +292,12 @@ __device__ __forceinline__ void lin_body(const Grid<T>& g, const Op& op_in, int 
   const int c0 = (bz % nch) * kchunk, c1 = min(c0 + kchunk, g.nzn);
   // planes of the chunk whose elements respond, by groups; without a map all of them
   unsigned long long resp = ~0ull;
-  if constexpr (!Op::SEPM) {
-    if (g.zs != nullptr && op.act() != nullptr) {
-      resp = tile_activity<T, BY, R>(g, op.act(), bx, by, c0, c1);
-      if ((resp & ((2ull << ((c1 - 1) / ACT_Z - c0 / ACT_Z)) - 1)) == 0) {
-        stiff_body<T, BY, R, Op>(g, op, bx, by, c0, c1);
-        op.finish();
-        return;
-      }
+  if (g.zs != nullptr && op.act() != nullptr) {
+    resp = tile_activity<T, BY, R>(g, op.act(), bx, by, c0, c1);
+    if ((resp & ((2ull << ((c1 - 1) / ACT_Z - c0 / ACT_Z)) - 1)) == 0) {
+      stiff_body<T, BY, R, Op>(g, op, bx, by, c0, c1);
+      op.finish();
+      return;
     }
   }
   // [relative plane parity][...][BY][32]: X (qx = 0, 1) of each warp's first row; upper-row
@@ -364,11 +360,9 @@ __device__ __forceinline__ void lin_body(const Grid<T>& g, const Op& op_in, int 
     const bool on = (resp >> q) & 1;
     while ((gb + q + 1) * ACT_Z < c1 && (((resp >> (q + 1)) & 1) != 0) == on) ++q;
     k1 = min((gb + q + 1) * ACT_Z, c1);
-    if constexpr (!Op::SEPM) {
-      if (!on) {
-        stiff_body<T, BY, R, Op>(g, op, bx, by, k0, k1);
-        continue;
-      }
+    if (!on) {
+      stiff_body<T, BY, R, Op>(g, op, bx, by, k0, k1);
+      continue;
     }
   }
   const int kmax = min(k1, g.nzn - 1);  // last plane the run reads
@@ -590,14 +584,8 @@ __device__ __forceinline__ void lin_body(const Grid<T>& g, const Op& op_in, int 
       const T dp = __shfl_down_sync(FULL_MASK, d, 1);
       const T stiff = ckx[0] * c1m + ckx[1] * c1 + ckx[2] * c1p + cmx[0] * dm + cmx[1] * d + cmx[2] * dp;
       const bool isdir = pdir || bnd[r] || (ptop && top[r]);
-      if constexpr (Op::SEPM) {
-        // second output: the separable consistent mass Mx My Mz v (the x stage of c1 rescaled)
-        const T mm = op.m_scale() * (cmx[0] * c1m + cmx[1] * c1 + cmx[2] * c1p);
-        if (wr[r]) op.lin_out2(nrow[r] + k * plane, isdir ? T(0) : stiff + mass, isdir ? T(0) : mm);
-      } else {
-        const T y = isdir ? vc[r] : stiff + mass;
-        if (wr[r]) op.lin_out(nrow[r] + k * plane, pre[r], vc[r], y);
-      }
+      const T y = isdir ? vc[r] : stiff + mass;
+      if (wr[r]) op.lin_out(nrow[r] + k * plane, pre[r], vc[r], y);
     }
     // interpolation of plane k+2 for the next layer, then shift the plane window (plane k+3
     // from its stage)

@@ -27,9 +27,6 @@ Phys make_phys(const qcad_mesh_s* m, const qcad_bias* b);
 GridTables make_tables(const std::vector<double>& x, const std::vector<double>& y, const std::vector<double>& z,
                        const std::vector<double>& kx_layer, const std::vector<double>& ky_layer,
                        const std::vector<double>& kz_layer);
-template <class T>
-void build_grid(GridDev<T>& gd, const GridTables& t, const std::vector<double>& hx, const std::vector<double>& hy,
-                const std::vector<double>& hz, cudaStream_t s);
 double host_h2m0();
 void set_message(const std::string& msg);
 
@@ -51,20 +48,21 @@ struct SubSetup {
   SubdomainMap sm;
   long long ns;     // subdomain nodes
   long long ndof;   // interior nodes
-  GridDev<double> g64;
-  DevBuf cV64, dinv, interior;
+  DevBuf &cV64, &dinv, &interior;  // the mesh's workspaces
   // the assembled operators: FP32, double-float (the FP64 phase's applies) and FP64
   HmStencil<float> st32{};
   HmStencil<float2> stdf{};
   HmStencil<double> st64{};
-  DevBuf zt32, ztdf, zt64;
-  double vmin;
+  std::vector<unsigned char> tab;  // host side of the plane tables while their upload may be pending
+  double vmin = 0.0;
   double inv_kx;    // 1 / kappa_x = 2 m_x / hbar^2 (scale of the separable mass stencil)
   double shift = 0.0;  // constant added to the potential (eV)
+  explicit SubSetup(qcad_mesh_s* m) : cV64(m->s_cV), dinv(m->s_dinv), interior(m->s_interior) {}
 };
 
-// rows: the precisions to assemble (ROWS_*; 0 none).
-enum { ROWS_32 = 1, ROWS_DF = 2, ROWS_64 = 4 };
+// rows: the precisions to assemble (ROWS_*).
+// SETUP_EIGS: an eigensolve (the Jacobi scale and the interior mask too).
+enum { ROWS_32 = 1, ROWS_DF = 2, ROWS_64 = 4, SETUP_EIGS = 8 };
 static void assemble_rows(qcad_mesh_s* m, const GridTables& t, double hx, double hy, int rows, SubSetup& S,
                           cudaStream_t s) {
   const int nxn = S.sm.nxs + 1, nyn = S.sm.nys + 1, nzn = S.sm.nzs + 1;
@@ -79,33 +77,42 @@ static void assemble_rows(qcad_mesh_s* m, const GridTables& t, double hx, double
   float2* sdf = static_cast<float2*>(buf(m->s_Sdf, ROWS_DF, sizeof(float2)));
   double* s64 = static_cast<double*>(buf(m->s_S64, ROWS_64, sizeof(double)));
   launch_hm_rows(S.cV64.as<double>(), nxn, nyn, nzn, m->s_mom.as<double>(), s32, sdf, s64, s);
-  // kinetic and mass coefficients of the planes, with the x and y step sizes of the a and b sums
-  std::vector<double> z((size_t)12 * nzn);
-  std::vector<float> zf(z.size());
-  std::vector<float2> zd(z.size());
+  // kinetic and mass coefficients of the planes, with the x and y step sizes of the a and b sums, in the
+  // three precisions, then the interior diagonal of the kinetic part: one upload
+  const size_t nz = (size_t)12 * nzn;
+  S.tab.resize(nz * (sizeof(double) + sizeof(float2) + sizeof(float)) + (size_t)nzn * sizeof(double));
+  double* z = reinterpret_cast<double*>(S.tab.data());
+  double* dk = z + nz;
+  float2* zd = reinterpret_cast<float2*>(dk + nzn);
+  float* zf = reinterpret_cast<float*>(zd + nz);
   const double mxy = hx * hy / 36.0;
-  for (int k = 0; k < nzn; ++k)
+  for (int k = 0; k < nzn; ++k) {
     for (int q = 0; q < 3; ++q) {
       z[12 * k + q] = t.mzx[3 * k + q] * (hy / (6.0 * hx));
       z[12 * k + 3 + q] = t.mzy[3 * k + q] * (hx / (6.0 * hy));
       z[12 * k + 6 + q] = t.kzz[3 * k + q] * mxy;
       z[12 * k + 9 + q] = S.inv_kx * t.mzx[3 * k + q] * mxy;
     }
-  for (size_t q = 0; q < z.size(); ++q) {
-    zf[q] = (float)z[q];
-    zd[q] = make_float2((float)z[q], (float)(z[q] - (double)(float)z[q]));
+    dk[k] = 8.0 * z[12 * k + 1] + 8.0 * z[12 * k + 4] + 16.0 * z[12 * k + 7];
   }
-  auto up = [&](DevBuf& b, const void* src, size_t bytes) {
-    b.ensure(bytes + 64);
-    CK(cudaMemcpyAsync(b.p, src, bytes, cudaMemcpyHostToDevice, s));
-  };
-  if (rows & ROWS_32) up(S.zt32, zf.data(), zf.size() * sizeof(float));
-  if (rows & ROWS_DF) up(S.ztdf, zd.data(), zd.size() * sizeof(float2));
-  if (rows & ROWS_64) up(S.zt64, z.data(), z.size() * sizeof(double));
-  CK(cudaStreamSynchronize(s));
-  S.st32 = {s32, S.zt32.as<float>(), nxn, nyn, nzn};
-  S.stdf = {sdf, S.ztdf.as<float2>(), nxn, nyn, nzn};
-  S.st64 = {s64, S.zt64.as<double>(), nxn, nyn, nzn};
+  for (size_t q = 0; q < nz; ++q) {
+    zf[q] = (float)z[q];
+    zd[q] = make_float2(zf[q], (float)(z[q] - (double)zf[q]));
+  }
+  m->s_tab.ensure(S.tab.size() + 64);
+  CK(cudaMemcpyAsync(m->s_tab.p, S.tab.data(), S.tab.size(), cudaMemcpyHostToDevice, s));
+  const double* z64 = m->s_tab.as<double>();
+  const double* dkd = z64 + nz;
+  const float2* zdf = reinterpret_cast<const float2*>(dkd + nzn);
+  const float* z32 = reinterpret_cast<const float*>(zdf + nz);
+  if (rows & SETUP_EIGS) {
+    S.dinv.ensure(S.ns * sizeof(double) + 64);
+    S.interior.ensure(S.ns + 64);
+    launch_hm_jacobi(nxn, nyn, nzn, dkd, S.dinv.as<double>(), S.interior.as<unsigned char>(), s);
+  }
+  S.st32 = {s32, z32, nxn, nyn, nzn};
+  S.stdf = {sdf, zdf, nxn, nyn, nzn};
+  S.st64 = {s64, z64, nxn, nyn, nzn};
 }
 
 // vxq: an extra potential energy at the subdomain's Gauss points (eV, [element][point]) or null;
@@ -140,22 +147,17 @@ static void setup_sub(qcad_mesh_s* m, const qcad_bias* b, const double* phi, con
   // kinetic coefficients hbar^2 / (2 m_d) for each direction (Eq. Schrodinger3D)
   std::vector<double> kx(sm.nzs, h2m / m_eff[0]), ky(sm.nzs, h2m / m_eff[1]), kz(sm.nzs, h2m / m_eff[2]);
   GridTables t = make_tables(xs, ys, zs, kx, ky, kz);
-  build_grid<double>(S.g64, t, hx, hy, hz, s);
-  S.g64.g.dir_boundary = 1;
-  S.g64.g.dir_bottom = 0;
-  S.g64.g.dir_top = nullptr;
   // potential energy at the qp: V = q phi_ref - chi - q phi (Eq. SchrodPotEnergy, no V_xc)
   const Phys P = make_phys(m, b);
   const long long nes = (long long)sm.nxs * sm.nys * sm.nzs;
   S.cV64.ensure(nes * 8 * sizeof(double) + 64);
   double* vmin_d = io.stats + 40;
-  const double big = 1e300;
-  CK(cudaMemcpyAsync(vmin_d, &big, sizeof(double), cudaMemcpyHostToDevice, s));
   auto potentials = [&](double V0) {
-    CK(cudaMemcpyAsync(vmin_d, &big, sizeof(double), cudaMemcpyHostToDevice, s));
+    CK(cudaMemsetAsync(vmin_d, 0x7f, sizeof(double), s));  // 1.4e306, above any potential
     launch_potential<double>(sm, phi, V0, m->g64.g.hx, m->g64.g.hy, m->g64.g.hz, vxq, S.cV64.as<double>(), vmin_d,
                              s);
     CK(cudaGetLastError());
+    if (!(shift_floor > 0.0)) return;  // nothing asks for the minimum
     double vmin_shift = 0;
     CK(cudaMemcpyAsync(&vmin_shift, vmin_d, sizeof(double), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
@@ -167,30 +169,10 @@ static void setup_sub(qcad_mesh_s* m, const qcad_bias* b, const double* phi, con
     S.shift = shift_floor - S.vmin;
     potentials(P.phi_ref - P.chi + S.shift);
   }
-  if (rows) assemble_rows(m, t, hx[0], hy[0], rows, S, s);
-  // Jacobi preconditioner from the kinetic diagonal, interior mask
-  std::vector<double> dinv(S.ns, 0.0);
-  std::vector<unsigned char> inter(S.ns, 0);
-  const int nxn = sm.nxs + 1, nyn = sm.nys + 1;
-  for (int k = 1; k < sm.nzs; ++k)
-    for (int j = 1; j < sm.nys; ++j)
-      for (int i = 1; i < sm.nxs; ++i) {
-        const long long n = i + (long long)nxn * (j + (long long)nyn * k);
-        const double d = t.kx[3 * i + 1] * t.my[3 * j + 1] * t.mzx[3 * k + 1] +
-                         t.mx[3 * i + 1] * t.ky[3 * j + 1] * t.mzy[3 * k + 1] +
-                         t.mx[3 * i + 1] * t.my[3 * j + 1] * t.kzz[3 * k + 1];
-        dinv[n] = 1.0 / d;
-        inter[n] = 1;
-      }
-  S.dinv.ensure(S.ns * sizeof(double) + 64);
-  S.interior.ensure(S.ns + 64);
-  CK(cudaMemcpyAsync(S.dinv.p, dinv.data(), S.ns * sizeof(double), cudaMemcpyHostToDevice, s));
-  CK(cudaMemcpyAsync(S.interior.p, inter.data(), S.ns, cudaMemcpyHostToDevice, s));
-  CK(cudaStreamSynchronize(s));
+  assemble_rows(m, t, hx[0], hy[0], rows, S, s);
 }
 
-static void hm_apply(qcad_mesh_s* m, SubSetup& S, int prec, int nvec, const double* X, double* HX, double* MX,
-                     DevBuf* tmp32) {
+static void hm_apply(qcad_mesh_s* m, SubSetup& S, int prec, int nvec, const double* X, double* HX, double* MX) {
   cudaStream_t s = m->stream;
   Profiler::Pair pp;
   if (prec == 0) {
@@ -198,20 +180,15 @@ static void hm_apply(qcad_mesh_s* m, SubSetup& S, int prec, int nvec, const doub
     a.x = X;
     a.hx = HX;
     a.mx = MX;
-    a.cV = S.cV64.as<double>();
     a.ld = S.ns;
     a.nvec = nvec;
-    a.mscale = S.inv_kx;
     if (m->prof.on) m->prof.begin(PROF_HM, s, pp);
-    if (S.st64.S)
-      launch_hm_stencil(S.st64, a, s);
-    else
-      launch_hm_apply<double>(S.g64.g, a, LaunchCfg{8, 16}, s);
+    launch_hm_stencil(S.st64, a, s);
     if (m->prof.on) m->prof.end(pp, s);
   } else {
     const long long tot = S.ns * nvec;
-    tmp32->ensure(3 * tot * sizeof(float) + 64);
-    float* x32 = tmp32->as<float>();
+    m->s_tmp32.ensure(3 * tot * sizeof(float) + 64);
+    float* x32 = m->s_tmp32.as<float>();
     float* h32 = x32 + tot;
     float* m32 = h32 + tot;
     launch_d2f(tot, X, x32, s);
@@ -234,18 +211,16 @@ qcad_status schrodinger_apply(qcad_mesh_s* m, const qcad_bias* b, const double* 
                               const double* X, double* HX, double* MX, int precision) {
   if (!b || !phi || !m_eff || !X || nvec < 1) throw Error(QCAD_ERR_INVALID_ARG, "null pointer or nvec < 1");
   if (precision != 0 && precision != 1) throw Error(QCAD_ERR_INVALID_ARG, "precision must be 0 or 1");
-  SubSetup S;
-  // FP64: assembling the rows costs about as much as applying the Gauss-point form to two vectors
-  setup_sub(m, b, phi, m_eff, precision ? ROWS_32 : nvec >= 3 ? ROWS_64 : 0, S, mesh_io(m));
+  SubSetup S(m);
+  setup_sub(m, b, phi, m_eff, precision ? ROWS_32 : ROWS_64, S, mesh_io(m));
   cudaStream_t s = m->stream;
-  DevBuf full, tmp;
-  full.ensure(3 * S.ns * nvec * sizeof(double) + 64);
-  double* xf = full.as<double>();
+  m->s_full.ensure(3 * S.ns * nvec * sizeof(double) + 64);
+  double* xf = m->s_full.as<double>();
   double* hf = xf + S.ns * nvec;
   double* mf = hf + S.ns * nvec;
   CK(cudaMemsetAsync(xf, 0, S.ns * nvec * sizeof(double), s));
   launch_pack(S.sm, nvec, xf, S.ns, const_cast<double*>(X), S.ndof, 1, s);
-  hm_apply(m, S, precision, nvec, xf, HX ? hf : nullptr, MX ? mf : nullptr, &tmp);
+  hm_apply(m, S, precision, nvec, xf, HX ? hf : nullptr, MX ? mf : nullptr);
   if (HX) launch_pack(S.sm, nvec, hf, S.ns, HX, S.ndof, 0, s);
   if (MX) launch_pack(S.sm, nvec, mf, S.ns, MX, S.ndof, 0, s);
   CK(cudaGetLastError());
@@ -786,8 +761,8 @@ qcad_status schrodinger_eigs_io(qcad_mesh_s* m, const EigIo& io, const qcad_bias
   if (!b || !phi || !m_eff || !evals) throw Error(QCAD_ERR_INVALID_ARG, "null pointer");
   if (nev < 1 || nev > 16) throw Error(QCAD_ERR_INVALID_ARG, "nev must be in [1, 16]");
   if (!(tol > 0)) throw Error(QCAD_ERR_INVALID_ARG, "tol must be > 0");
-  SubSetup S;
-  setup_sub(m, b, phi, m_eff, ROWS_32 | ROWS_DF | ROWS_64, S, io, vxq, shift_floor);
+  SubSetup S(m);
+  setup_sub(m, b, phi, m_eff, ROWS_32 | ROWS_DF | ROWS_64 | SETUP_EIGS, S, io, vxq, shift_floor);
   const double t_setup = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
   if (S.ndof < 3 * (nev + 4)) throw Error(QCAD_ERR_INVALID_ARG, "subdomain too small for nev");
   cudaStream_t s = io.s;

@@ -185,7 +185,9 @@ struct qcad_mesh_s {
   double lam_cache[2] = {0.0, 0.0};
   qcad::Profiler prof;                     // thread-safe: concurrent calls may record
   // Schrodinger workspace
-  qcad::DevBuf s_mx, s_kx, s_my, s_ky, s_mzx, s_mzy, s_kzz, s_cV, s_dinv, s_interior, s_blocks, s_gram;
-  qcad::DevBuf s_mom, s_S32, s_Sdf, s_S64;  // the V rows of the subdomain and the scratch of their assembly
+  // (kept between calls; one eigensolve or block apply runs on a mesh at a time)
+  qcad::DevBuf s_cV, s_dinv, s_interior, s_tab;   // potential coefficients, Jacobi scale, interior mask, plane tables
+  qcad::DevBuf s_mom, s_S32, s_Sdf, s_S64;        // the V rows of the subdomain and the scratch of their assembly
+  qcad::DevBuf s_full, s_tmp32;                   // block applies: vectors on all subdomain nodes
   ~qcad_mesh_s();
 };

@@ -207,21 +207,13 @@ struct HmArgs {
   const T* x;      // nvec full-subdomain vectors, stride ldx
   T* hx;           // or null
   T* mx;           // or null
-  const T* cV;     // V * w|J| at the qp of every subdomain element
   long long ld;    // vector stride (n_sub_nodes)
   int nvec;
-  double mscale;   // 1 / kappa_x: the consistent mass is the kappa_x-weighted z mass stencil times this
 };
-// variant >= 2: plane-factorized kernel (M applied as the separable mass stencil), else
-// element-gather.
-template <class T>
-void launch_hm_apply(const Grid<T>& g, const HmArgs<T>& a, LaunchCfg cfg, cudaStream_t s);
-template <class T>
-void launch_hm_apply_lin(const Grid<T>& g, const HmArgs<T>& a, LaunchCfg cfg, cudaStream_t s);
 // H and M with the V term assembled into a 27-point row per node (kernels_hm.cu): S [27][nodes], zt
 // [planes][12] the kinetic coefficients of an output plane along x, y, z and its mass, each for the
 // input planes below, at and above it. C: float, double, or float2 for double-float arithmetic on
-// FP64 vectors (a.cV and a.mscale are not used).
+// FP64 vectors.
 template <class C>
 struct HmStencil {
   const C* S;
@@ -235,6 +227,8 @@ void launch_hm_stencil(const HmStencil<float2>& st, const HmArgs<double>& a, cud
 // output is not null; mom: scratch of 27 doubles per element.
 void launch_hm_rows(const double* cV, int nxn, int nyn, int nzn, double* mom, float* S32, float2* Sdf, double* S64,
                     cudaStream_t s);
+// Jacobi scale 1 / dk[k] of the interior nodes (0 on the boundary) and the interior mask.
+void launch_hm_jacobi(int nxn, int nyn, int nzn, const double* dk, double* dinv, unsigned char* interior, cudaStream_t s);
 // One fused step of the LOBPCG Chebyshev-Jacobi block preconditioner (kernels_hm.cu): the H apply
 // of D_in (nvec columns at stride ld) with the recurrence W -= H D_in,
 // D_out = c1 D_in + c2 D^-1 W, Z += D_out in its epilogue.
