@@ -193,7 +193,7 @@ __device__ __forceinline__ void df_acc(float& ah, float& al, float bh, float bl)
 // partial sums to its own slot of `part` (no atomics); gram_reduce_kernel adds the slots in a
 // fixed order, so the result is deterministic.
 constexpr int GR = 32;                   // rows per shared-memory tile
-constexpr int GRAM_MAX_BLOCKS = 2 * 152;
+constexpr int GRAM_MAX_BLOCKS = 3 * 152;
 
 // 4 consecutive values of a shared row (16-byte aligned for float, two 16-byte loads for double).
 __device__ __forceinline__ void gram_ld4(const float* p, float* v) {
@@ -217,12 +217,11 @@ __device__ __forceinline__ void gram_cp(T* smem, const T* gmem, bool valid) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(s), "l"(gmem), "r"(n) : "memory");
 }
 
-// GC > 0: the row-group count G at compile time (FP32 storage takes one group), so that the row loop
-// over a shared tile unrolls completely.
-template <class T, int GC = 0>
-__global__ void __launch_bounds__(512) gram_kernel(long long n, int p, int nb2, const T* A, long long lda,
-                                                   const T* B1, const T* B2, long long ldb, double* part, int G_) {
-  const int G = GC > 0 ? GC : G_;
+// FP64 storage (QCAD_FP64_DENSE=native): G row groups of 4 x 4 output tiles.
+__global__ void __launch_bounds__(512) gram_kernel(long long n, int p, int nb2, const double* A, long long lda,
+                                                   const double* B1, const double* B2, long long ldb, double* part,
+                                                   int G) {
+  using T = double;
   extern __shared__ __align__(16) unsigned char sh_raw[];
   T* sh = reinterpret_cast<T*>(sh_raw);      // two stages of GR x W
   const int q = p;
@@ -240,16 +239,9 @@ __global__ void __launch_bounds__(512) gram_kernel(long long n, int p, int nb2, 
   const bool active = tid < G * nt;
   const int grp = active ? tid / nt : 0, tt = active ? tid % nt : 0;
   const int ta = tt / tb_n, tb = tt % tb_n;
-  // across tiles: FP64 (double storage) or double-float on the FP32 pipes (float storage, where
-  // an FP64 add per output and tile would cost more than the tile's products)
   double acc[16];
-  float acch[16], accl[16];
 #pragma unroll
-  for (int s = 0; s < 16; ++s) {
-    acc[s] = 0.0;
-    acch[s] = 0.0f;
-    accl[s] = 0.0f;
-  }
+  for (int s = 0; s < 16; ++s) acc[s] = 0.0;
   const long long ntiles = (n + GR - 1) / GR;
   auto issue = [&](long long tile, int stage) {
     if (tile < ntiles) {
@@ -285,7 +277,7 @@ __global__ void __launch_bounds__(512) gram_kernel(long long n, int p, int nb2, 
       T s16[16];
 #pragma unroll
       for (int s = 0; s < 16; ++s) s16[s] = T(0);
-#pragma unroll(GC > 0 ? GR / (GC > 0 ? GC : 1) : 4)
+#pragma unroll 4
       for (int rr = grp; rr < GR; rr += G) {
         const T* row = st + rr * W;
         T av[4], bv[4];
@@ -297,21 +289,12 @@ __global__ void __launch_bounds__(512) gram_kernel(long long n, int p, int nb2, 
           for (int v = 0; v < 4; ++v) s16[4 * u + v] += av[u] * bv[v];
       }
 #pragma unroll
-      for (int s = 0; s < 16; ++s) {
-        if constexpr (sizeof(T) == 4)
-          df_acc(acch[s], accl[s], (float)s16[s], 0.0f);
-        else
-          acc[s] += (double)s16[s];
-      }
+      for (int s = 0; s < 16; ++s) acc[s] += s16[s];
     }
     __syncthreads();  // the stage is refilled by the next iteration's copies
     stage ^= 1;
   }
   asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-  if constexpr (sizeof(T) == 4) {
-#pragma unroll
-    for (int s = 0; s < 16; ++s) acc[s] = df_join(acch[s], accl[s]);
-  }
   // the groups' sums in a fixed order (the staging area is free now)
   __syncthreads();
   double* red = reinterpret_cast<double*>(sh_raw);  // [G][nt][16]
@@ -335,6 +318,109 @@ __global__ void __launch_bounds__(512) gram_kernel(long long n, int p, int nb2, 
       if (bc >= qt) continue;
       out[bc < q ? a * q + bc : p * q + a * q + (bc - q)] = acc[4 * u + v];
     }
+  }
+}
+
+// FP32 storage. The tile keeps the columns' order ([column][row], a copy of 32 rows per column is
+// contiguous), each thread owns 4 columns of A times 4 of [B1 B2] (columns ta + ta_n u and tb + tb_n v,
+// so that the lanes of a warp read neighbouring columns without bank conflicts) and reads four rows per
+// 16-byte load: 8 loads for 64 products without an index computation per copied value, and three
+// blocks of 192 threads on an SM (one of 256 with a transposed copy took 314 us for 36 columns and
+// 735k rows). About 32 rows per thread (G tiles) are summed in FP32, these sums in double-float on the FP32 pipes.
+constexpr int G32_ROWS = 32, G32_STRIDE = G32_ROWS + 4;
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS, THREADS == 192 ? 3 : 1) gram32_kernel(long long n, int p, int nb2, const float* A,
+                                                                        long long lda, const float* B1, const float* B2,
+                                                                        long long ldb, double* part, int G) {
+  extern __shared__ __align__(16) unsigned char sh_raw[];
+  float* sh = reinterpret_cast<float*>(sh_raw);  // three stages of [cols][G32_STRIDE]
+  const int q = p, qt = q * nb2;
+  const int ta_n = (p + 3) / 4, tb_n = (qt + 3) / 4, nt = ta_n * tb_n;
+  const int pc = 4 * ta_n, cols = pc + 4 * tb_n, stage_len = cols * G32_STRIDE;
+  const int tid = threadIdx.x, nth = blockDim.x, lane = tid & 31, warp = tid >> 5, nwarp = nth >> 5;
+  for (int t = tid; t < 3 * stage_len; t += nth) sh[t] = 0.0f;  // padding columns stay zero
+  __syncthreads();
+  const bool active = tid < G * nt;
+  const int grp = active ? tid / nt : 0, tt = active ? tid % nt : 0;
+  const int ta = tt / tb_n, tb = tt % tb_n;
+  float acch[16], accl[16];
+#pragma unroll
+  for (int s = 0; s < 16; ++s) acch[s] = accl[s] = 0.0f;
+  const long long ntiles = (n + G32_ROWS - 1) / G32_ROWS;
+  auto issue = [&](long long tile, int stage) {  // lane: row of the tile, warps: columns
+    if (tile < ntiles) {
+      const long long row = tile * G32_ROWS + lane;
+      const bool ok = row < n;
+      const long long r = ok ? row : 0;
+      float* st = sh + stage * stage_len + lane;
+      for (int c = warp; c < p; c += nwarp) gram_cp<float>(st + c * G32_STRIDE, A + c * lda + r, ok);
+      for (int c = warp; c < qt; c += nwarp)
+        gram_cp<float>(st + (pc + c) * G32_STRIDE, (c < q ? B1 + c * ldb : B2 + (c - q) * ldb) + r, ok);
+    }
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  };
+  // three stages, one barrier per tile: the stage that a tile's barrier frees takes the copy two tiles on
+  float s32[16];
+#pragma unroll
+  for (int s = 0; s < 16; ++s) s32[s] = 0.0f;
+  int stage = 0, since = 0;
+  issue(blockIdx.x, 0);
+  issue(blockIdx.x + (long long)gridDim.x, 1);
+  for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+    __syncthreads();
+    issue(tile + 2LL * gridDim.x, stage == 0 ? 2 : stage - 1);
+    if (active) {
+      const float* st = sh + stage * stage_len;
+      const float* pa = st + ta * G32_STRIDE;
+      const float* pb = st + (pc + tb) * G32_STRIDE;
+#pragma unroll 1
+      for (int rr = 4 * grp; rr < G32_ROWS; rr += 4 * G) {
+        float av[4][4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) gram_ld4(pa + u * ta_n * G32_STRIDE + rr, av[u]);
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+          float bv[4];
+          gram_ld4(pb + v * tb_n * G32_STRIDE + rr, bv);
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int w = 0; w < 4; ++w) s32[4 * u + v] = fmaf(av[u][w], bv[w], s32[4 * u + v]);
+        }
+      }
+      if (++since == G) {  // about 32 rows
+        since = 0;
+#pragma unroll
+        for (int s = 0; s < 16; ++s) {
+          df_acc(acch[s], accl[s], s32[s], 0.0f);
+          s32[s] = 0.0f;
+        }
+      }
+    }
+    stage = stage == 2 ? 0 : stage + 1;
+  }
+#pragma unroll
+  for (int s = 0; s < 16; ++s) df_acc(acch[s], accl[s], s32[s], 0.0f);
+  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+  __syncthreads();
+  // the groups' sums in a fixed order (the staging area is free now), one group after the other
+  double* red = reinterpret_cast<double*>(sh_raw);  // [nt][16]
+  for (int g = 0; g < G; ++g) {
+    if (active && grp == g)
+#pragma unroll
+      for (int s = 0; s < 16; ++s) {
+        const double v = df_join(acch[s], accl[s]);
+        red[(size_t)tt * 16 + s] = g == 0 ? v : red[(size_t)tt * 16 + s] + v;
+      }
+    __syncthreads();
+  }
+  // slot layout: product 0 (p*q) then product 1
+  double* out = part + (size_t)blockIdx.x * p * qt;
+  for (int t = tid; t < nt * 16; t += nth) {
+    const int o = t >> 4, s = t & 15;
+    const int a = o / tb_n + ta_n * (s >> 2), bc = o % tb_n + tb_n * (s & 3);
+    if (a < p && bc < qt) out[bc < q ? a * q + bc : p * q + a * q + (bc - q)] = red[t];
   }
 }
 
@@ -372,7 +458,7 @@ size_t gram_part_doubles(int p, int q) { return (size_t)GRAM_MAX_BLOCKS * p * 2 
 // 735k rows, 58 % of the issue slots).
 // Products with more than 256 output tiles (14 or more columns per block without the triangle) take one
 // block of 512 threads.
-constexpr int DGR = 32;
+constexpr int DGR = 32;  // rows of a tile, one per lane of the copies
 template <int THREADS>
 __global__ void __launch_bounds__(THREADS, 512 / THREADS) gram_df_kernel(long long n, int p, int nb2, const double* A, long long lda,
                                                       const double* B1, const double* B2, long long ldb,
@@ -383,11 +469,13 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) gram_df_kernel(long lo
   const int ta_n = (p + 3) / 4, tb_n = (qt + 3) / 4;
   const int pp = 4 * ta_n, qp = 4 * tb_n;
   const int W = pp + qp + 4;
-  double* sh = reinterpret_cast<double*>(sh_raw);                 // two stages of DGR x W doubles
-  float* fh = reinterpret_cast<float*>(sh + (size_t)2 * DGR * W);  // DGR x W hi words
+  const int cols = p + qt;
+  double* sh = reinterpret_cast<double*>(sh_raw);  // two stages of [cols][DGR] doubles, as copied
+  float* fh = reinterpret_cast<float*>(sh + (size_t)2 * cols * DGR);  // [DGR][W] hi words
   float* fl = fh + (size_t)DGR * W;                                // DGR x W lo words
   const int tid = threadIdx.x, nth = blockDim.x;
-  for (int t = tid; t < 2 * DGR * W; t += nth) sh[t] = 0.0;
+  const int lane = tid & 31, warp = tid >> 5, nwarp = nth >> 5;
+  for (int t = tid; t < DGR * W; t += nth) fh[t] = fl[t] = 0.0f;  // padding columns stay zero
   __syncthreads();
   // G row groups of nt output tiles, as in gram_kernel
   const int tq = ta_n, tri = tq * (tq + 1) / 2;  // upper: tiles per product on or above its diagonal
@@ -415,26 +503,15 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) gram_df_kernel(long lo
     accl[s] = 0.0f;
   }
   const long long ntiles = (n + DGR - 1) / DGR;
-  auto issue = [&](long long tile, int stage) {
+  auto issue = [&](long long tile, int stage) {  // lane: row of the tile, warps: columns
     if (tile < ntiles) {
-      const long long r0 = tile * DGR;
-      double* st = sh + (size_t)stage * DGR * W;
-      for (int t = tid; t < (p + qt) * DGR; t += nth) {
-        const int col = t / DGR, rr = t % DGR;
-        const long long row = r0 + rr;
-        const bool ok = row < n;
-        const double* src;
-        int sc;
-        if (col < p) {
-          src = A + col * lda + (ok ? row : 0);
-          sc = col;
-        } else {
-          const int bc = col - p;
-          src = (bc < q ? B1 + bc * ldb : B2 + (bc - q) * ldb) + (ok ? row : 0);
-          sc = pp + bc;
-        }
-        gram_cp<double>(st + rr * W + sc, src, ok);
-      }
+      const long long row = tile * DGR + lane;
+      const bool ok = row < n;
+      const long long r = ok ? row : 0;
+      double* st = sh + (size_t)stage * cols * DGR + lane;
+      for (int c = warp; c < p; c += nwarp) gram_cp<double>(st + c * DGR, A + c * lda + r, ok);
+      for (int c = warp; c < qt; c += nwarp)
+        gram_cp<double>(st + (p + c) * DGR, (c < q ? B1 + c * ldb : B2 + (c - q) * ldb) + r, ok);
     }
     asm volatile("cp.async.commit_group;\n" ::: "memory");
   };
@@ -445,8 +522,11 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) gram_df_kernel(long lo
     asm volatile("cp.async.wait_group 1;\n" ::: "memory");
     __syncthreads();
     {
-      const double* st = sh + (size_t)stage * DGR * W;
-      for (int t = tid; t < DGR * W; t += nth) df_split_i(st[t], fh[t], fl[t]);
+      const double* st = sh + (size_t)stage * cols * DGR + lane;
+      for (int c = warp; c < cols; c += nwarp) {
+        const int o = lane * W + (c < p ? c : pp + c - p);
+        df_split_i(st[c * DGR], fh[o], fl[o]);
+      }
     }
     __syncthreads();
     if (active) {
@@ -524,18 +604,39 @@ void launch_gram(long long n, int p, int q, const T* A, long long lda, const T* 
   // 8), so that the double-float products of small blocks occupy the block; with float storage a
   // tile's products are cheap next to the per-tile accumulation, so one group
   const int nt = ta_n * tb_n;
-  const int G = sizeof(T) == 8 ? std::max(1, std::min(8, 512 / nt)) : 1;
+  if constexpr (std::is_same<T, float>::value) {
+    const int cap = nt <= 192 ? 192 : 512;
+    const int G = std::max(1, std::min(8, cap / nt));
+    const int nth = std::min(cap, ((G * nt + 31) / 32) * 32);
+    const long long want = cap == 192 ? 3LL * sm_count() : GRAM_MAX_BLOCKS;
+    const int nblk = (int)std::max<long long>(
+        1, std::min<long long>(std::min<long long>(want, GRAM_MAX_BLOCKS), (n + G32_ROWS - 1) / G32_ROWS));
+    const size_t shm = std::max((size_t)nt * 16 * sizeof(double),
+                                (size_t)3 * 4 * (ta_n + tb_n) * G32_STRIDE * sizeof(float));
+    static bool attr = false;
+    if (!attr)
+      attr = cudaFuncSetAttribute(gram32_kernel<192>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024) ==
+                 cudaSuccess &&
+             cudaFuncSetAttribute(gram32_kernel<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024) ==
+                 cudaSuccess;
+    if (cap == 192)
+      note_launch(), gram32_kernel<192><<<nblk, nth, shm, s>>>(n, p, nb2, A, lda, B1, B2, ldb, part, G);
+    else
+      note_launch(), gram32_kernel<512><<<nblk, nth, shm, s>>>(n, p, nb2, A, lda, B1, B2, ldb, part, G);
+    const int tot = p * p * nb2;
+    note_launch(), gram_reduce_kernel<<<(tot + 31) / 32, dim3(32, 8), 0, s>>>(nblk, tot, p * p, part, G1, G2);
+    return;
+  } else {
+  const int G = std::max(1, std::min(8, 512 / nt));
   const int nth = std::min(512, std::max(256, ((G * nt + 31) / 32) * 32));
   const long long ntiles = (n + GR - 1) / GR;
-  const int nblk = (int)std::max<long long>(1, std::min<long long>(GRAM_MAX_BLOCKS, ntiles));
+  const int nblk = (int)std::max<long long>(1, std::min<long long>(2LL * sm_count(), ntiles));
   const size_t red = (size_t)G * nt * 16 * sizeof(double);  // the groups' sums, after the tiles
   const size_t shm = std::max(red, (size_t)2 * GR * (4 * ta_n + 4 * tb_n + 4) * sizeof(T));
   static bool attr = false;
   if (!attr)
-    attr = cudaFuncSetAttribute(gram_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024) == cudaSuccess &&
-           cudaFuncSetAttribute(gram_kernel<T, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024) ==
-               cudaSuccess;
-  if constexpr (std::is_same<T, double>::value) {
+    attr = cudaFuncSetAttribute(gram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024) == cudaSuccess;
+  {
     if (dense_df()) {
       // the upper triangles only (the caller mirrors them), where the tiles align with the products
       const int up = (upper && p == q && p % 4 == 0) ? 1 : 0;
@@ -546,7 +647,7 @@ void launch_gram(long long n, int p, int q, const T* A, long long lda, const T* 
       const size_t red_df = (size_t)G_df * nt_df * 16 * sizeof(double);
       // two double stages plus the hi and lo float tiles
       const size_t shm_df =
-          std::max(red_df, (size_t)2 * DGR * (4 * ta_n + 4 * tb_n + 4) * (sizeof(double) + sizeof(float)));
+          std::max(red_df, (size_t)2 * DGR * (p * (1 + nb2) * sizeof(double) + (4 * ta_n + 4 * tb_n + 4) * sizeof(float)));
       static bool attr_df = false;
       if (!attr_df)
         attr_df = cudaFuncSetAttribute(gram_df_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) ==
@@ -562,12 +663,10 @@ void launch_gram(long long n, int p, int q, const T* A, long long lda, const T* 
       return;
     }
   }
-  if (G == 1)
-    note_launch(), gram_kernel<T, 1><<<nblk, nth, shm, s>>>(n, p, nb2, A, lda, B1, B2, ldb, part, G);
-  else
-    note_launch(), gram_kernel<T><<<nblk, nth, shm, s>>>(n, p, nb2, A, lda, B1, B2, ldb, part, G);
+  note_launch(), gram_kernel<<<nblk, nth, shm, s>>>(n, p, nb2, A, lda, B1, B2, ldb, part, G);
   const int tot = p * p * nb2;
   note_launch(), gram_reduce_kernel<<<(tot + 31) / 32, dim3(32, 8), 0, s>>>(nblk, tot, p * p, part, G1, G2);
+  }
 }
 template void launch_gram<float>(long long, int, int, const float*, long long, const float*, const float*, long long,
                                  double*, double*, double*, cudaStream_t, bool);
