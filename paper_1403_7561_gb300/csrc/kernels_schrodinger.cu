@@ -451,8 +451,8 @@ size_t gram_part_doubles(int p, int q) { return (size_t)GRAM_MAX_BLOCKS * p * 2 
 // gram_kernel for FP64 blocks in double-float arithmetic: the double tile lands in shared
 // memory as before, is split once into hi and lo float tiles, and each 32-row tile is summed in
 // double-float before it is added to the FP64 accumulators.
-// upper: only the output tiles on or above the diagonal of each product (p == q, q a multiple of
-// 4); the entries below are left unwritten.
+// upper: only the output tiles on or above the diagonal of each product; the entries below are left
+// unwritten.
 // A block of at most 256 threads, two on an SM: while one waits at its barriers or copies the other
 // computes (one block of 480 threads per SM and scalar products took 1.01 ms for 36 columns and
 // 735k rows, 58 % of the issue slots).
@@ -466,9 +466,10 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) gram_df_kernel(long lo
   extern __shared__ __align__(16) unsigned char sh_raw[];
   const int q = p;
   const int qt = q * nb2;
-  const int ta_n = (p + 3) / 4, tb_n = (qt + 3) / 4;
-  const int pp = 4 * ta_n, qp = 4 * tb_n;
-  const int W = pp + qp + 4;
+  // the columns of A, B1 and B2 each padded to whole tiles, so that the triangles need no alignment
+  const int ta_n = (p + 3) / 4, tb_n = nb2 * ta_n;
+  const int pp = 4 * ta_n;
+  const int W = pp * (1 + nb2) + 4;
   const int cols = p + qt;
   double* sh = reinterpret_cast<double*>(sh_raw);  // two stages of [cols][DGR] doubles, as copied
   float* fh = reinterpret_cast<float*>(sh + (size_t)2 * cols * DGR);  // [DGR][W] hi words
@@ -524,7 +525,7 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) gram_df_kernel(long lo
     {
       const double* st = sh + (size_t)stage * cols * DGR + lane;
       for (int c = warp; c < cols; c += nwarp) {
-        const int o = lane * W + (c < p ? c : pp + c - p);
+        const int o = lane * W + c + (c < p ? 0 : c < p + q ? pp - p : 2 * pp - 2 * p);
         df_split_i(st[c * DGR], fh[o], fl[o]);
       }
     }
@@ -577,9 +578,8 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) gram_df_kernel(long lo
     if (a >= p) continue;
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
-      const int bc = 4 * tb + v;
-      if (bc >= qt) continue;
-      out[bc < q ? a * q + bc : p * q + a * q + (bc - q)] = acc[4 * u + v];
+      const int j = 4 * (tb % ta_n) + v;
+      if (j < q) out[(tb / ta_n) * p * q + a * q + j] = acc[4 * u + v];
     }
   }
 }
@@ -638,16 +638,16 @@ void launch_gram(long long n, int p, int q, const T* A, long long lda, const T* 
     attr = cudaFuncSetAttribute(gram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024) == cudaSuccess;
   {
     if (dense_df()) {
-      // the upper triangles only (the caller mirrors them), where the tiles align with the products
-      const int up = (upper && p == q && p % 4 == 0) ? 1 : 0;
-      const int nt_df = up ? nb2 * (ta_n * (ta_n + 1) / 2) : nt;
+      // the upper triangles only (the caller mirrors them)
+      const int up = (upper && p == q) ? 1 : 0, tb_df = nb2 * ta_n;
+      const int nt_df = up ? nb2 * (ta_n * (ta_n + 1) / 2) : ta_n * tb_df;
       const int cap = nt_df <= 256 ? 256 : 512;
       const int G_df = std::max(1, std::min(8, cap / nt_df));
       const int nth_df = std::min(cap, std::max(128, ((G_df * nt_df + 31) / 32) * 32));
       const size_t red_df = (size_t)G_df * nt_df * 16 * sizeof(double);
       // two double stages plus the hi and lo float tiles
       const size_t shm_df =
-          std::max(red_df, (size_t)2 * DGR * (p * (1 + nb2) * sizeof(double) + (4 * ta_n + 4 * tb_n + 4) * sizeof(float)));
+          std::max(red_df, (size_t)2 * DGR * (p * (1 + nb2) * sizeof(double) + (4 * ta_n + 4 * tb_df + 4) * sizeof(float)));
       static bool attr_df = false;
       if (!attr_df)
         attr_df = cudaFuncSetAttribute(gram_df_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) ==

@@ -610,7 +610,7 @@ struct LobpcgRun {
       // of P is applied to the small matrices on the host (G -> T^T G T), which gives the
       // Rayleigh-Ritz problem of the orthonormalized blocks without forming them
       int nuse = haveP ? nb + 2 * na : nb + na;
-      const bool up = gram_upper() && nuse % 4 == 0;
+      const bool up = gram_upper();
       gram_async(nuse, nuse, Sx, HS, MS, up);
       sync();
       ++iters;
