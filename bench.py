@@ -307,9 +307,10 @@ def load_peaks():
 def algorithmic_bytes(cls, n_nodes, n_elems):
     """Bytes each launch must move at minimum given its stored linearization (per class)."""
     return {
-        # p = z + beta p_prev (read z, p_prev; write p), Ap written, 8 FP32 qp coefficients per element
-        "apply32": 16 * n_nodes + 32 * n_elems,
-        "apply64": 32 * n_nodes + 64 * n_elems,
+        # p = z + beta p_prev (read z, p_prev; write p), Ap written. The qp coefficients (32 or 64 bytes per
+        # element) are read only where an element responds to the potential, so they are left out
+        "apply32": 16 * n_nodes,
+        "apply64": 32 * n_nodes,
         # x, r, p, Ap, D^-1 read; x, r, z written
         "update32": 32 * n_nodes,
         "update64": 64 * n_nodes,

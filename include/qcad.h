@@ -378,7 +378,9 @@ qcad_status qcad_profile_read(qcad_mesh_t m, int kernel_class, int64_t* launches
  * plane-factorized kernel with one node row per thread, 3 plane-factorized
  * with two node rows per thread. Shapes a variant does not support are
  * clamped to the nearest supported one (FP64 plane-factorized: at most 8
- * warps). Defaults: variant 3, 8 warps, z chunk 16.
+ * warps; family 0 uses z_chunk alone, its node pass runs four warps of two rows).
+ * Defaults: variant 3, 8 warps, z chunk 16; while a family's default stands, its
+ * launches fit tile rows and z chunk to the grid (small grids take smaller ones).
  * qcad_autotune times the Jacobian apply of the given precision (0 FP64,
  * 1 FP32) over variants, tile rows and z chunks on the mesh, keeps the
  * fastest for that family and returns it (outputs may be NULL); best_ms is
