@@ -600,9 +600,8 @@ void launch_gram(long long n, int p, int q, const T* A, long long lda, const T* 
   (void)q;  // the products of LOBPCG are square: q == p
   const int nb2 = B2 ? 2 : 1;
   const int ta_n = (p + 3) / 4, tb_n = (p * nb2 + 3) / 4;
-  // row groups (double storage): as many copies of the output tiles as fit 512 threads (at most
-  // 8), so that the double-float products of small blocks occupy the block; with float storage a
-  // tile's products are cheap next to the per-tile accumulation, so one group
+  // row groups: as many copies of the output tiles as fit the block (at most 8), so that the products of
+  // small blocks occupy it
   const int nt = ta_n * tb_n;
   if constexpr (std::is_same<T, float>::value) {
     const int cap = nt <= 192 ? 192 : 512;
