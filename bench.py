@@ -86,7 +86,7 @@ def parse(argv=None):
                     help="ncu --csv metrics capture of one kernel class to record in profiles/ncu_counters.json "
                          "(with --kernel-class, --workload, --launch, --per, --profile-md)")
     ap.add_argument("--kernel-class", default="residual")
-    ap.add_argument("--per", type=int, default=1, help="launches per unit of --ncu-counters (residual: 2 passes)")
+    ap.add_argument("--per", type=int, default=1, help="launches per unit of --ncu-counters (residual: 3 passes)")
     ap.add_argument("--profile-md", default=None, help="the profiles/ summary that records the capture command")
     return ap.parse_args(argv)
 
@@ -251,7 +251,7 @@ def counter(counters, cur_hash, kernel, workload, launch, key):
 
 def ingest_ncu(args):
     """Average an ncu CSV capture (--metrics ... --csv) of one kernel class over its units (a unit is
-    `--per` consecutive launches: 2 for the two-pass residual) and record DRAM bytes and FP64 flops
+    `--per` consecutive launches: 3 for the three-pass residual) and record DRAM bytes and FP64 flops
     per unit in the counters file, with the class's current source hash."""
     import csv
     rows = list(csv.reader(open(args.ncu_counters)))
