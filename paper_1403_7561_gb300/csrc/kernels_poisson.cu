@@ -249,7 +249,7 @@ __device__ __forceinline__ void residual_qp_body(const Grid<double>& g, const Re
   // semiconductor) skips the interpolation and the transposed interpolation.
   if (a.counts == nullptr && a.qd.w == nullptr) {
     // -2: no charge term at all (oxide, padding)
-    const int zone = semi ? charge_zone_key(a.P, double_key((unsigned long long)__double_as_longlong(v))) : -2;
+    const int zone = semi ? charge_zone_key(a.P, double_key(v)) : -2;
     int zmin = zone, zmax = zone;
 #pragma unroll
     for (int sft = 1; sft < 8; sft <<= 1) {

@@ -22,11 +22,11 @@ constexpr int NODE_WARPS = 4;  // warps of the node pass, two node rows each
 // A double rounded to float (to nearest) on the integer pipes: the conversion instruction runs on the
 // FP64 pipe.
 __device__ __forceinline__ float d2f_bits(double a) {
-  const unsigned long long u = (unsigned long long)__double_as_longlong(a);
-  const unsigned e = (unsigned)(u >> 52) & 0x7FFu;
+  const unsigned hi = (unsigned)__double2hiint(a);
+  const unsigned e = (hi >> 20) & 0x7FFu;
   if (e < 897u || e > 1149u) return __double2float_rn(a);
-  const unsigned long long m = (u & 0x7FFFFFFFFFFFFFFFull) - (896ull << 52);
-  return __uint_as_float((unsigned)((m + 0x0FFFFFFFull + ((m >> 29) & 1)) >> 29) | ((unsigned)(u >> 32) & 0x80000000u));
+  const unsigned long long m = abs_bits(a) - (896ull << 52);
+  return __uint_as_float((unsigned)((m + 0x0FFFFFFFull + ((m >> 29) & 1)) >> 29) | (hi & 0x80000000u));
 }
 // 4 a by the exponent.
 __device__ __forceinline__ double times4(double a) {
@@ -51,7 +51,7 @@ __device__ __forceinline__ void residual_classify_body(const Grid<double>& g, co
     hi = -99;
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-      const int z = charge_zone_key(a.P, double_key((unsigned long long)__double_as_longlong(v[c])));
+      const int z = charge_zone_key(a.P, double_key(v[c]));
       lo = min(lo, z);
       hi = max(hi, z);
     }
@@ -228,13 +228,16 @@ __device__ __forceinline__ void residual_node_body(const Grid<double>& g, const 
       if (!wr[r]) continue;
       const int n = nrow[r + 1] + k * plane;
       double R = c1[0][r] + fma(-2.0, c2[0][r], xs);
-      if (edge) R *= half[r] == 0 ? 1.0 : half[r] == 1 ? 0.5 : 0.25;
+      if (edge) {
+        asm volatile("");  // keeps the product inside the branch
+        R *= half[r] == 0 ? 1.0 : half[r] == 1 ? 0.5 : 0.25;
+      }
       R += up[r] + lo[r];
       const bool dir = pdir || (k == g.nz && top[r]);
       if (dir) R = 0.0;
       a.R[n] = R;
-      if (a.b64) a.b64[n] = -R;
-      if (a.b32) a.b32[n] = d2f_bits(-R);
+      if (a.b64) a.b64[n] = neg_bits(R);
+      if (a.b32) a.b32[n] = -d2f_bits(R);
       const float ff = half[r] == 0 ? 1.0f : half[r] == 1 ? 0.5f : 0.25f;
       const bool rs = resp[r] || dresp[r];
       if (a.dinv32 && !rs)  // the FP32 Jacobi scale as an FP32 reciprocal (within an ulp of the rounded inverse)
@@ -249,7 +252,7 @@ __device__ __forceinline__ void residual_node_body(const Grid<double>& g, const 
       }
       acc_r2 = fma(R, R, acc_r2);
       // max |R| by bit pattern (NaN left out, as fmax does)
-      const unsigned long long b = (unsigned long long)__double_as_longlong(R) & 0x7fffffffffffffffull;
+      const unsigned long long b = abs_bits(R);
       if (b <= 0x7ff0000000000000ull && b > acc_max) acc_max = b;
     }
   };
