@@ -76,7 +76,7 @@ __device__ __forceinline__ void lin_lds_c8<double>(const uint4* p, double* c) {
 }
 
 // Nonzero, by the bit pattern (an FP64 comparison would take the FP64 pipe).
-__device__ __forceinline__ bool lin_nonzero(double c) { return (__double_as_longlong(c) << 1) != 0; }
+__device__ __forceinline__ bool lin_nonzero(double c) { return nonzero_bits(c); }
 
 // Packed row-exchange values (one shared access per pair or quadruple).
 template <class T>

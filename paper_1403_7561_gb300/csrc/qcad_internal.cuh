@@ -150,6 +150,9 @@ __device__ __forceinline__ unsigned long long abs_bits(double a) {
 __device__ __forceinline__ double neg_bits(double a) {
   return __hiloint2double(__double2hiint(a) ^ (int)0x80000000u, __double2loint(a));
 }
+__device__ __forceinline__ bool nonzero_bits(double a) {
+  return (((unsigned)__double2hiint(a) << 1) | (unsigned)__double2loint(a)) != 0u;
+}
 __device__ __forceinline__ unsigned long long double_key(double a) {
   const int hi = __double2hiint(a), s = hi >> 31;
   return ((unsigned long long)(unsigned)(hi ^ (s | (int)0x80000000u)) << 32) | (unsigned)(__double2loint(a) ^ s);
