@@ -200,25 +200,11 @@ constexpr int WQ_ZERO = 6;           // 0: no charge (oxide, padding)
 
 // The residual's charge outside the dots: where phi lies outside every cutoff band (n and p below
 // resolution, each dopant fully ionized or below resolution) the charge is a constant and its
-// derivative zero, found by a few comparisons; elsewhere the full evaluation with the residual's
-// cutoffs. Both give the same values as charge_at(P, phi, true).
+// derivative zero, found by a few integer comparisons; elsewhere the full evaluation with the
+// residual's cutoffs. Both give the same values as charge_at(P, phi, true).
 __device__ __forceinline__ Charge charge_resid(const Phys& P, double phi) {
-  const bool no_n = phi < P.phi_n_on, no_p = phi > P.phi_p_on;
-  bool flat = no_n && no_p;
-  double rho = 0.0;
-  if (P.incomplete) {
-    if (P.na_on) {
-      flat = flat && (phi < P.phi_a_lo || phi > P.phi_a_hi);
-      rho -= phi > P.phi_a_hi ? P.NA : 0.0;  // z_a < -45: fully ionized; above the cutoff: none
-    }
-    if (P.nd_on) {
-      flat = flat && (phi < P.phi_d_lo || phi > P.phi_d_hi);
-      rho += phi < P.phi_d_lo ? P.ND : 0.0;
-    }
-  } else {
-    rho = P.ND - P.NA;
-  }
-  if (flat) return Charge{rho, 0.0, 0.0, 0.0};
+  const int zone = charge_zone_key(P, double_key(phi));
+  if (zone >= 0) return Charge{zone_charge(P, zone), 0.0, 0.0, 0.0};
   return charge_at(P, phi, true);
 }
 

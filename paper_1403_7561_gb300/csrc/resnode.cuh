@@ -24,14 +24,14 @@ constexpr int NODE_WARPS = 4;  // warps of the node pass, two node rows each
 __device__ __forceinline__ float d2f_bits(double a) {
   const unsigned hi = (unsigned)__double2hiint(a);
   const unsigned e = (hi >> 20) & 0x7FFu;
+  if (e < 872u) return __uint_as_float(hi & 0x80000000u);  // below half the smallest float
   if (e < 897u || e > 1149u) return __double2float_rn(a);
   const unsigned long long m = abs_bits(a) - (896ull << 52);
   return __uint_as_float((unsigned)((m + 0x0FFFFFFFull + ((m >> 29) & 1)) >> 29) | (hi & 0x80000000u));
 }
 // 4 a by the exponent.
 __device__ __forceinline__ double times4(double a) {
-  const long long u = __double_as_longlong(a);
-  return (u << 1) == 0 ? a : __longlong_as_double(u + (2ll << 52));
+  return nonzero_bits(a) ? __hiloint2double(__double2hiint(a) + (2 << 20), __double2loint(a)) : a;
 }
 
 // Pass 1a for one element column (lanes hold consecutive columns) and layers [k0, k1).
@@ -86,7 +86,7 @@ __device__ __forceinline__ void residual_classify_body(const Grid<double>& g, co
     }
     if (valid && flat) {
       const double th = a.theta ? a.theta[e] : 0.0;
-      if (th == 0.0) {
+      if (!nonzero_bits(th)) {
         // the element's corner loads are one table entry and its diagonal contributions zero
         a.ecode[e] = (unsigned char)(1 + (zone >= 0 ? (a.P.incomplete ? zone : WQ_ZONE_COMPLETE) : WQ_ZERO));
       } else {
@@ -140,14 +140,16 @@ __device__ __forceinline__ void residual_density_body(const Grid<double>& g, con
     v = A * v + B * __shfl_xor_sync(FULL_MASK, v, 4);
     const double w = a.wq[8 * k + WQ_WEIGHT];  // -(q/eps0) w|J|
     const Charge ch = charge_resid(a.P, v);
-    double f = w * (ch.rho + (a.theta ? a.theta[e] : 0.0));
+    double f = ch.rho;
+    if (a.theta) f += a.theta[e];
+    f *= w;
     double c = w * ch.drho;
     if (valid) {
       if (a.c64) a.c64[8LL * e + l] = c;
-      if (a.c32) a.c32[8LL * e + l] = (float)c;
+      if (a.c32) a.c32[8LL * e + l] = d2f_bits(c);
     }
     // an element with a nonzero coefficient marks its cell of the activity map
-    const unsigned nz = __ballot_sync(FULL_MASK, c != 0.0);
+    const unsigned nz = __ballot_sync(FULL_MASK, nonzero_bits(c));
     if (valid && l == 0 && ((nz >> (threadIdx.x & 24)) & 0xffu) != 0) {
       const size_t cell = i / ACT_X + (size_t)act_cells(g.nx, ACT_X) * (j / ACT_Y + act_cells(g.ny, ACT_Y) * (k / ACT_Z));
       if (a.act64) a.act64[cell] = 1;
