@@ -664,7 +664,7 @@ def native_arm(args):
         ach = flops / (ms / nl / 1000.0) / 1e12 if (nl and flops) else None
         return {"bound": "alu", "kernel": cls, "achieved": ach, "peak": pk, "unit": "TFLOP/s",
                 "frac": (ach / pk) if ach else None, "traffic": traffic,
-                "traffic_unit": "bytes per evaluation (ncu dram read + write, cold cache, both passes)",
+                "traffic_unit": "bytes per evaluation (ncu dram read + write, cold cache, all its launches)",
                 "traffic_source": note, "flops_source": fnote,
                 "peak_kind": "derived: 2 DFMA lanes/SM/clock x 2 flops x 152 SMs x median SM clock under load",
                 "flops_kind": "FP64 flops per evaluation counted by ncu (2 DFMA + DADD + DMUL)",

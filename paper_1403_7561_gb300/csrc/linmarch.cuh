@@ -491,7 +491,8 @@ __device__ __forceinline__ void lin_body(const Grid<T>& g, const Op& op_in, int 
 #pragma unroll
     for (int r = 0; r < R; ++r) lin_lds_c8<T>(st + ((ty * R + r) * NCH) * 32 + lane, c[r]);
     // FP64: a warp whose elements of this layer have no response passes the carry on or skips the layer
-    // (in FP32 the test cost more than the operations it saved)
+    // (in FP32 the test cost more than the operations it saved). The test is of bits, off the FP64 pipe: as
+    // eight comparisons an element a J v call took 345 us instead of 329 at 128 x 128 x 96 elements
     bool nz = true;
     if constexpr (SKIP) {
       nz = false;

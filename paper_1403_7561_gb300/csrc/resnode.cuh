@@ -1,18 +1,23 @@
-// The two-pass residual without dot counts, quantum density or surface terms (the path of every
+// The residual without dot counts, quantum density or surface terms (the path of every
 // Newton step and line-search trial, single and batched): a classification pass over the elements, the
 // density at the Gauss points of the listed elements, and a node pass. Included by kernels_poisson.cu.
 //
 // FP64 runs at 2 lanes per SM and clock, so each pass is held to the FP64 work that its outputs need:
 //  - Classification (one thread per element column, marching z): charge zones of the node potentials by
 //    integer keys, once per node and column. An element whose corners share a constant-charge zone gets
-//    its load code and zero coefficients; the others are appended to a list. No FP64 arithmetic.
+//    its load code and zero coefficients; the others are appended to a list. No FP64 arithmetic: signs,
+//    keys and zero tests are taken on the halves of the pattern (written on the whole pattern they came
+//    out as five FP64 additions an element: 87 us at 256 x 256 x 128 elements, 60 us now; the coefficient
+//    stores take 40).
 //  - Density (8 lanes per listed element): full warps whatever the shape of the charged region. In one
 //    pass over all elements the charged ones left lanes idle in mixed warps and every element paid the
 //    index arithmetic eight times over (256 x 256 x 128 elements at 0.5 K: 0.74 ms for the former pass).
+//    The comparisons that find a point's zone are of integer keys (200 -> 186 us, fourth evaluation there).
 //  - Node pass: K phi in the difference form of stiff_body (17 operations per node, where the three-stage
 //    stencil took 25 and two gathered fields 14 more on tiles with 1.3 times the nodes), the corner loads
 //    of four equal codes as one table entry, the diagonal from a per-plane table where no element adds to
-//    it. 1.12 ms before at that size.
+//    it. 1.12 ms before at that size, 0.56 with the signs, magnitudes and zero tests on the FP64 pipe, 0.48
+//    without them (24 operations per node with the halos; the pipe is 86 % busy).
 #pragma once
 
 namespace qcad {
