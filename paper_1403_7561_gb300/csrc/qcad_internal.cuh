@@ -141,22 +141,9 @@ __host__ __device__ __forceinline__ unsigned long long double_key(unsigned long 
 }
 
 #ifdef __CUDACC__
-// Sign operations of a double on the halves of its bit pattern. Written on the whole pattern (and on
-// the 64-bit key above) they are recognised as negation and magnitude of a double, which take an
-// addition each on the 2-lane FP64 pipe.
-__device__ __forceinline__ unsigned long long abs_bits(double a) {
-  return ((unsigned long long)((unsigned)__double2hiint(a) & 0x7fffffffu) << 32) | (unsigned)__double2loint(a);
-}
-__device__ __forceinline__ double neg_bits(double a) {
-  return __hiloint2double(__double2hiint(a) ^ (int)0x80000000u, __double2loint(a));
-}
-__device__ __forceinline__ bool nonzero_bits(double a) {
-  return (((unsigned)__double2hiint(a) << 1) | (unsigned)__double2loint(a)) != 0u;
-}
-__device__ __forceinline__ unsigned long long double_key(double a) {
-  const int hi = __double2hiint(a), s = hi >> 31;
-  return ((unsigned long long)(unsigned)(hi ^ (s | (int)0x80000000u)) << 32) | (unsigned)(__double2loint(a) ^ s);
-}
+}  // namespace qcad
+#include "fpbits.cuh"
+namespace qcad {
 #endif
 
 struct DotBoxes {

@@ -24,21 +24,6 @@ namespace qcad {
 
 constexpr int NODE_WARPS = 4;  // warps of the node pass, two node rows each
 
-// A double rounded to float (to nearest) on the integer pipes: the conversion instruction runs on the
-// FP64 pipe.
-__device__ __forceinline__ float d2f_bits(double a) {
-  const unsigned hi = (unsigned)__double2hiint(a);
-  const unsigned e = (hi >> 20) & 0x7FFu;
-  if (e < 872u) return __uint_as_float(hi & 0x80000000u);  // below half the smallest float
-  if (e < 897u || e > 1149u) return __double2float_rn(a);
-  const unsigned long long m = abs_bits(a) - (896ull << 52);
-  return __uint_as_float((unsigned)((m + 0x0FFFFFFFull + ((m >> 29) & 1)) >> 29) | (hi & 0x80000000u));
-}
-// 4 a by the exponent.
-__device__ __forceinline__ double times4(double a) {
-  return nonzero_bits(a) ? __hiloint2double(__double2hiint(a) + (2 << 20), __double2loint(a)) : a;
-}
-
 // Pass 1a for one element column (lanes hold consecutive columns) and layers [k0, k1).
 __device__ __forceinline__ void residual_classify_body(const Grid<double>& g, const ResidualArgs& a, double* elR,
                                                        double* elD, int col, int k0, int k1) {
