@@ -43,15 +43,18 @@ __device__ __forceinline__ void fd_half_d(double x, double& F, double& dF, doubl
   const double C = 1.32934038817913702047;  // 3 sqrt(pi) / 4
   // y = v^(-1/8) from an FP32 estimate by Newton's iteration for v y^8 = 1, y <- y + y (1 - v y^8) / 8
   // (quadratic: 3e-7, 4e-13, below an ulp), where pow and the division by v took about 120 FP64
-  // operations; v >= 40, and beyond the FP32 range the estimate comes from pow
-  double y = (double)rsqrtf(sqrtf(sqrtf((float)v)));
-  if (y == 0.0) y = pow(v, -0.125);
-  double y8 = 0.0;
+  // operations; v > 36 (36.9 at x = -1.79). Beyond the FP32 range y comes from pow, so that an
+  // infinite v gives an infinite F
+  const float est = rsqrtf(sqrtf(sqrtf((float)v)));
+  double y = (double)est;
+  if (est == 0.0f) {
+    y = pow(v, -0.125);
+  } else {
 #pragma unroll
-  for (int it = 0; it < 2; ++it) {
-    const double y2 = y * y, y4 = y2 * y2;
-    y8 = y4 * y4;
-    y = fma(0.125 * y, fma(-v, y8, 1.0), y);
+    for (int it = 0; it < 2; ++it) {
+      const double y2 = y * y, y4 = y2 * y2;
+      y = fma(0.125 * y, fma(-v, y4 * y4, 1.0), y);
+    }
   }
   const double y2 = y * y;
   const double cvp = C * (y2 * y);  // C v^(-3/8)

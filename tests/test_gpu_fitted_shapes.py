@@ -49,3 +49,17 @@ def test_residual_and_jv_with_default_shapes(q, n, T):
     for precision, tol in ((0, 1e-12), (1, 2e-6)):
         q.qcad_poisson_jv(m, dev["bias"], t(phi), t(v), y, precision)
         assert np.max(np.abs(y.cpu().numpy() - y0)) <= tol * np.max(np.abs(y0)), precision
+
+
+def test_residual_of_an_overflowing_density_is_infinite(q):
+    # phi = 1e80 V: eta^4 exceeds the FP64 range and the Fermi-Dirac density with it. A constant phi has
+    # K phi = 0, so every silicon node above the Ohmic contact holds the infinite charge alone
+    dev = W.five_gate_device(n=(16, 16, 16), T=300.0, with_subdomain=False)
+    m = q.qcad_mesh_create(dev)
+    phi = torch.full((m.n_nodes,), 1e80, dtype=torch.float64, device="cuda")
+    R = torch.zeros_like(phi)
+    rmax, r2 = q.qcad_poisson_residual(m, dev["bias"], phi, R)
+    n_si = dev["layers"][0]["n"]
+    planes = R.cpu().numpy().reshape(-1, 17 * 17)
+    assert np.all(planes[1:n_si + 1] == np.inf) and np.all(planes[0] == 0.0)
+    assert rmax == np.inf and r2 == np.inf
