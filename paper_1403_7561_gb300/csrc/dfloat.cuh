@@ -1,17 +1,14 @@
 // Double-float arithmetic on the FP32 pipes: a value is the unevaluated sum h + l of two floats
-// (about 46 significant bits). The product uses Dekker's fused-multiply-add split, the sum Knuth's
-// two-sum, each renormalized by a fast two-sum; relative error of a product or sum about 2^-46.
-// On this part FP32 runs at 64 times the FP64 rate, so a double-float multiply-add (some twenty
-// FP32 instructions) costs a third of an FP64 one. Conversions to and from FP64 go through the
-// bit patterns (integer instructions), because the FP32<->FP64 conversion instructions run on the
-// FP64 pipe.
+// (about 46 significant bits). The sum is Knuth's two-sum, renormalized by a fast two-sum (relative
+// error about 2^-46); products are split by a fused multiply-add. On this part FP32 runs at 64 times
+// the FP64 rate, so a double-float multiply-add (some twelve FP32 instructions) costs a fraction of
+// an FP64 one. Conversions to and from FP64 go through the bit patterns (integer instructions),
+// because the FP32<->FP64 conversion instructions run on the FP64 pipe.
 //
-// Used as the scalar type T of the plane-factorized z-march for the FP64 phase of the
-// eigensolver's H and M applies (kernels_lin.cu).
+// Used by the eigensolver's FP64 phase: the H and M applies (kernels_hm.cu), the Gram and block
+// products (kernels_schrodinger.cu).
 #pragma once
 #include <cuda_runtime.h>
-
-#include "qcad_internal.cuh"
 
 namespace qcad {
 
@@ -20,8 +17,6 @@ struct dfl {
   __host__ __device__ dfl() : h(0.0f), l(0.0f) {}
   __host__ __device__ dfl(int v) : h((float)v), l(0.0f) {}
   __host__ __device__ dfl(float hh, float ll) : h(hh), l(ll) {}
-  // host only: the split of a double by FP32 rounding (device code uses dfl_from_bits)
-  __host__ dfl(double v) : h((float)v), l((float)(v - (double)(float)v)) {}
 };
 
 __device__ __forceinline__ dfl dfl_quick(float s, float e) {
@@ -38,29 +33,7 @@ __device__ __forceinline__ dfl operator+(dfl a, dfl b) {
 }
 __device__ __forceinline__ dfl operator-(dfl a) { return dfl(-a.h, -a.l); }
 __device__ __forceinline__ dfl operator-(dfl a, dfl b) { return a + (-b); }
-__device__ __forceinline__ dfl operator*(dfl a, dfl b) {
-  const float p = a.h * b.h;
-  float e = fmaf(a.h, b.h, -p);
-  e = fmaf(a.h, b.l, e);
-  e = fmaf(a.l, b.h, e);
-  return dfl_quick(p, e);
-}
 __device__ __forceinline__ dfl& operator+=(dfl& a, dfl b) { return a = a + b; }
-__device__ __forceinline__ dfl& operator*=(dfl& a, dfl b) { return a = a * b; }
-
-// Warp shuffles of both words (the built-in overloads stay visible beside these).
-using ::__shfl_down_sync;
-using ::__shfl_up_sync;
-using ::__shfl_xor_sync;
-__device__ __forceinline__ dfl __shfl_down_sync(unsigned mask, dfl v, unsigned d) {
-  return dfl(::__shfl_down_sync(mask, v.h, d), ::__shfl_down_sync(mask, v.l, d));
-}
-__device__ __forceinline__ dfl __shfl_up_sync(unsigned mask, dfl v, unsigned d) {
-  return dfl(::__shfl_up_sync(mask, v.h, d), ::__shfl_up_sync(mask, v.l, d));
-}
-__device__ __forceinline__ dfl __shfl_xor_sync(unsigned mask, dfl v, int d) {
-  return dfl(::__shfl_xor_sync(mask, v.h, d), ::__shfl_xor_sync(mask, v.l, d));
-}
 
 // a = h + l for 2^-80 <= |a| < 2^127 by the bit pattern: h keeps the sign, exponent and top 23
 // mantissa bits of a (truncation, exact), l the next 23 (bits 28..6), |a - h - l| <= 2^-46 |a|;
@@ -89,11 +62,5 @@ __device__ __forceinline__ double dfl_f2d(float x) {
 
 // h + l rounded to FP64 (one FP64 addition).
 __device__ __forceinline__ double dfl_to_double(dfl a) { return dfl_f2d(a.h) + dfl_f2d(a.l); }
-
-// The Gauss weights (1 +- 1/sqrt 3) / 2 of the linear shape functions as double-float pairs.
-template <> struct GaussConst<dfl> {
-  static __device__ __forceinline__ dfl a() { return dfl(0x1.93cd3ap-1f, 0x1.640cc8p-28f); }
-  static __device__ __forceinline__ dfl b() { return dfl(0x1.b0cb18p-3f, -0x1.640cc8p-28f); }
-};
 
 }  // namespace qcad

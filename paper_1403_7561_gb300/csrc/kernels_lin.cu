@@ -37,10 +37,10 @@ static void lin_launch(const Grid<T>& g, const Op& op, int kchunk, cudaStream_t 
 // rows. FP64 is bound by the SM's FP64 pipe, which all resident blocks share: one slot per SM, the
 // cost of a plane is its rows, and smaller tiles (more halo, but more SMs at work) compete.
 template <class T>
-static LaunchCfg fit_lin(int nxn, int nyn, int nzn, int nvec, LaunchCfg cfg) {
+static LaunchCfg fit_lin(int nxn, int nyn, int nzn, LaunchCfg cfg) {
   if (!cfg.fit || cfg.variant < 2) return cfg;
   constexpr bool F32 = std::is_same<T, float>::value;
-  const long long tx = (long long)((nxn + 29) / 30) * nvec;
+  const long long tx = (nxn + 29) / 30;
   const long long slots = (F32 ? 2LL : 1LL) * sm_count();
   const double over = F32 ? 3.0 : 2.0;
   auto tiles = [&](int tr) { return tx * ((nyn + tr - 3) / (tr - 2)); };
@@ -70,7 +70,7 @@ static bool has_act(const Op& op) { return op.v.act != nullptr; }
 // 4/8 x 2 (shared memory). Other requests are clamped to the nearest supported shape.
 template <class T, class Op>
 static void run_lin(const Grid<T>& g, const Op& op, LaunchCfg cfg, cudaStream_t s) {
-  cfg = fit_lin<T>(g.nxn, g.nyn, g.nzn, 1, cfg);
+  cfg = fit_lin<T>(g.nxn, g.nyn, g.nzn, cfg);
   // With an activity map a tile with response takes about six times as long as one without in FP64, so
   // the longest tile sets the time: half the chunk (FP64 solve of the 128 x 128 x 96 device 75 -> 67 ms;
   // FP32, bound by latency, was 5 % slower with it).

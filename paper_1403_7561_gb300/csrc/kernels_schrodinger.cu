@@ -24,9 +24,8 @@ static int dblocks(long long n) {
 }
 
 // cV_q = (q phi_ref - chi - q phi(x_q)) * w|J| for every subdomain element (Eq. SchrodPotEnergy).
-template <class T>
 __global__ void potential_kernel(SubdomainMap sm, const double* phi, double V0, const double* hx,
-                                 const double* hy, const double* hz, const double* vxq, T* cV, double* vmin) {
+                                 const double* hy, const double* hz, const double* vxq, double* cV, double* vmin) {
   const long long ne = (long long)sm.nxs * sm.nys * sm.nzs;
   double lo = 1e300;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < ne; e += (long long)gridDim.x * blockDim.x) {
@@ -51,7 +50,7 @@ __global__ void potential_kernel(SubdomainMap sm, const double* phi, double V0, 
     for (int s = 0; s < 8; ++s) {
       const double V = V0 - q[s] + (vxq ? vxq[8 * e + s] : 0.0);
       lo = fmin(lo, V);
-      cV[8 * e + s] = (T)(V * wdet);
+      cV[8 * e + s] = V * wdet;
     }
   }
   // min over the block via shuffles, then an atomic on the ordered bits of (V + offset)
@@ -62,16 +61,11 @@ __global__ void potential_kernel(SubdomainMap sm, const double* phi, double V0, 
   }
 }
 
-template <class T>
 void launch_potential(const SubdomainMap& sm, const double* phi, double V0, const double* hx, const double* hy,
-                      const double* hz, const double* vxq, T* cV, double* vmin, cudaStream_t s) {
+                      const double* hz, const double* vxq, double* cV, double* vmin, cudaStream_t s) {
   const long long ne = (long long)sm.nxs * sm.nys * sm.nzs;
-  note_launch(), potential_kernel<T><<<dblocks(ne), DT, 0, s>>>(sm, phi, V0, hx, hy, hz, vxq, cV, vmin);
+  note_launch(), potential_kernel<<<dblocks(ne), DT, 0, s>>>(sm, phi, V0, hx, hy, hz, vxq, cV, vmin);
 }
-template void launch_potential<float>(const SubdomainMap&, const double*, double, const double*, const double*,
-                                      const double*, const double*, float*, double*, cudaStream_t);
-template void launch_potential<double>(const SubdomainMap&, const double*, double, const double*, const double*,
-                                       const double*, const double*, double*, double*, cudaStream_t);
 
 // Interior-DOF <-> full subdomain node vector (column-major blocks).
 __global__ void pack_kernel(SubdomainMap sm, int nvec, double* full, long long ldf, double* dof, long long ldd,

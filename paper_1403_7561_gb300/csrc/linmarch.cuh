@@ -104,11 +104,10 @@ struct LinShape {
 };
 
 // Launch geometry (kchunk at most LinShape::ZMAX): x tiles of 30 interior nodes, y tiles of
-// BY*R - 2 interior rows,
-// (vector, z chunk) pairs along z.
-inline dim3 lin_grid(int nxn, int nyn, int nzn, int by, int r, int kchunk, int nvec = 1) {
+// BY*R - 2 interior rows, z chunks.
+inline dim3 lin_grid(int nxn, int nyn, int nzn, int by, int r, int kchunk) {
   const int tr = by * r;
-  return dim3((nxn + 29) / 30, (nyn + tr - 3) / (tr - 2), ((nzn + kchunk - 1) / kchunk) * nvec);
+  return dim3((nxn + 29) / 30, (nyn + tr - 3) / (tr - 2), (nzn + kchunk - 1) / kchunk);
 }
 
 // Activity of a tile's planes in groups of ACT_Z (group q: planes ACT_Z (k0 / ACT_Z + q) and up): bit q is
@@ -286,10 +285,9 @@ __device__ __forceinline__ void lin_body(const Grid<T>& g, const Op& op_in, int 
   constexpr int TR = S::TR, NCH = S::NCH, NST = S::NST;
   constexpr bool SKIP = std::is_same<T, double>::value;
   if (op_in.skip()) return;
-  const int nch = (g.nzn + kchunk - 1) / kchunk;
   Op op = op_in;
-  op.set_vec(bz / nch);
-  const int c0 = (bz % nch) * kchunk, c1 = min(c0 + kchunk, g.nzn);
+  op.set_vec(0);
+  const int c0 = bz * kchunk, c1 = min(c0 + kchunk, g.nzn);
   // planes of the chunk whose elements respond, by groups; without a map all of them
   unsigned long long resp = ~0ull;
   if (g.zs != nullptr && op.act() != nullptr) {

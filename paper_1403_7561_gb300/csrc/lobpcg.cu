@@ -154,8 +154,7 @@ static void setup_sub(qcad_mesh_s* m, const qcad_bias* b, const double* phi, con
   double* vmin_d = io.stats + 40;
   auto potentials = [&](double V0) {
     CK(cudaMemsetAsync(vmin_d, 0x7f, sizeof(double), s));  // 1.4e306, above any potential
-    launch_potential<double>(sm, phi, V0, m->g64.g.hx, m->g64.g.hy, m->g64.g.hz, vxq, S.cV64.as<double>(), vmin_d,
-                             s);
+    launch_potential(sm, phi, V0, m->g64.g.hx, m->g64.g.hy, m->g64.g.hz, vxq, S.cV64.as<double>(), vmin_d, s);
     CK(cudaGetLastError());
     if (!(shift_floor > 0.0)) return;  // nothing asks for the minimum
     double vmin_shift = 0;

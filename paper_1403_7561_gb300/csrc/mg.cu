@@ -723,32 +723,6 @@ __global__ void __launch_bounds__(MG_THREADS) mg_resid_kernel(const MgLevelDev<T
   L.w[n] = L.b[n] - mg_stencil_dot<T>(L, nn, n, L.x);
 }
 
-// Coarse correction of level l from the solution ec of level l+1: out = base + P ec on free
-// nodes (base on Dirichlet nodes).
-template <class T>
-__global__ void mg_prolong_kernel(const MgLevelDev<T> F, const T* __restrict__ ec, const MgLevelDev<T> C,
-                                  const T* base, T* out, const PcgScalars* sc) {
-  if (sc->done) return;
-  const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  const long long nn = (long long)F.nxn * F.nyn * F.nzn;
-  if (n >= nn) return;
-  T v = base[n];
-  if (!F.mask[n]) {
-    int i, j, k;
-    node_ijk(F, n, i, j, k);
-    const MgProl px = F.pr[0][i], py = F.pr[1][j], pz = F.pr[2][k];
-    const long long sy = C.nxn, sz = (long long)C.nxn * C.nyn;
-    const long long z0 = pz.c0 * sz, z1 = pz.c1 * sz, y0 = py.c0 * sy, y1 = py.c1 * sy;
-    const T xw0 = px.w0, xw1 = px.w1, yw0 = py.w0, yw1 = py.w1, zw0 = pz.w0, zw1 = pz.w1;
-    const T e00 = xw0 * ec[z0 + y0 + px.c0] + xw1 * ec[z0 + y0 + px.c1];
-    const T e01 = xw0 * ec[z0 + y1 + px.c0] + xw1 * ec[z0 + y1 + px.c1];
-    const T e10 = xw0 * ec[z1 + y0 + px.c0] + xw1 * ec[z1 + y0 + px.c1];
-    const T e11 = xw0 * ec[z1 + y1 + px.c0] + xw1 * ec[z1 + y1 + px.c1];
-    v += zw0 * (yw0 * e00 + yw1 * e01) + zw1 * (yw0 * e10 + yw1 * e11);
-  }
-  out[n] = v;
-}
-
 // Post-smoothing on a coarse level: w = x + omega D^-1 (b - A x) (the level's solution).
 template <class T>
 __global__ void __launch_bounds__(MG_THREADS) mg_post_kernel(const MgLevelDev<T> L, const T* par, int l,

@@ -17,9 +17,8 @@ struct SubdomainMap {
   long long nxn, nyn;  // global mesh nodes per axis (x, y)
 };
 
-template <class T>
 void launch_potential(const SubdomainMap& sm, const double* phi, double V0, const double* hx, const double* hy,
-                      const double* hz, const double* vxq /* extra potential at the Gauss points or null */, T* cV,
+                      const double* hz, const double* vxq /* extra potential at the Gauss points or null */, double* cV,
                       double* vmin, cudaStream_t s);
 void launch_pack(const SubdomainMap& sm, int nvec, double* full, long long ldf, double* dof, long long ldd,
                  int unpack, cudaStream_t s);

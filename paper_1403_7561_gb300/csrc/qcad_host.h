@@ -96,7 +96,7 @@ struct LaunchCfg {
   int by = 8;
   int kchunk = 16;
   int variant = 3;
-  bool fit = true;  // the shape is a default: the launch fits it to the grid (fit_march); a shape
+  bool fit = true;  // the shape is a default: the launch fits it to the grid (fit_lin, fit_march64); a shape
                     // set or autotuned for the mesh runs as given
 };
 
