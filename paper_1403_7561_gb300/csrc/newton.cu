@@ -1251,6 +1251,7 @@ static void adjoint_prepare(AdjWork& A, qcad_mesh_s* m, const qcad_bias* b, cons
   gtop.mzy = g64.mzy + 3 * kl;
   gtop.kzz = g64.kzz + 3 * kl;
   gtop.zt = g64.zt ? g64.zt + 12 * kl : nullptr;
+  gtop.zs = nullptr;  // its rows carry the layer below the view too: the view has no stiffness-only form
   gtop.hz = g64.hz + kl;
   gtop.dir_bottom = 0;
   const long long plane = g64.plane, off = (long long)kl * plane, top = (long long)m->nz * plane;
