@@ -5,9 +5,9 @@
 // uniform x and y spacings, applied per node plane from nine values as
 //   a_r = 4 v + (v- + v+), b_r = 2 v - (v- + v+)       along x, for the rows r = j-1, j, j+1,
 //   P2 = 4 a_0 + (a_- + a_+), P1x = 4 b_0 + (b_- + b_+), P1y = 2 a_0 - (a_- + a_+),
-// then along z with the step sizes folded into the plane's coefficients (zt): the differences of
-// neighbouring values stay differences, so a smooth field loses no digits to the assembly. M uses P2
-// alone. The V term sum_q w|J| V_q N_a(q) N_b(q) has no such structure; its row costs 27 products
+// then along z with the step sizes folded into the plane's coefficients (zt), the z stiffness as fluxes
+// w (P2 of one plane less that of the one below): the differences of neighbouring values stay
+// differences, so a smooth field loses no digits to the assembly. M uses P2 alone. The V term sum_q w|J| V_q N_a(q) N_b(q) has no such structure; its row costs 27 products
 // per node and vector, where evaluating it at the Gauss points took the plane-factorized march of
 // linmarch.cuh about 100 operations, 20 shuffles and shared-memory exchanges and a barrier per plane.
 //
@@ -54,17 +54,30 @@ template <> struct HmT<dfl> {
 
 __device__ __forceinline__ void hm_fma(float& s, float a, float b) { s = fmaf(a, b, s); }
 __device__ __forceinline__ void hm_fma(double& s, double a, double b) { s = fma(a, b, s); }
-// The low word collects the rounding errors of the high sums and the low products; it is folded in
-// once at the end (dfl_to_double), which saves the renormalization of every step.
-__device__ __forceinline__ void hm_fma(dfl& s, dfl a, dfl b) {
-  const float p = a.h * b.h;
-  float e = fmaf(a.h, b.h, -p);
-  e = fmaf(a.h, b.l, e);
-  e = fmaf(a.l, b.h, e);
-  const float t = s.h + p, bb = t - s.h;
-  e += (s.h - (t - bb)) + (p - bb);
-  s.h = t;
-  s.l += e;
+__device__ __forceinline__ void hm_fma(dfl& s, dfl a, dfl b) { s += dfl_prod(a, b); }
+// s += c0 x0 + c1 x1 + c2 x2. Double-float renormalizes once per three products: with the low word
+// collecting the errors of a node's 36 products unrenormalized, H of smooth vectors on 24 x 22 x 20
+// elements was off by up to 7.2e-14 of its largest entry against 64-bit extended arithmetic; now 1.4e-14
+// (the march evaluating Gauss points, renormalized at each step, 1.6e-14).
+template <class T>
+__device__ __forceinline__ void hm_mac3(T& s, T c0, T x0, T c1, T x1, T c2, T x2) {
+  hm_fma(s, c0, x0);
+  hm_fma(s, c1, x1);
+  hm_fma(s, c2, x2);
+}
+__device__ __forceinline__ void hm_mac3(dfl& s, dfl c0, dfl x0, dfl c1, dfl x1, dfl c2, dfl x2) {
+  dfl_mac3(s, c0, x0, c1, x1, c2, x2);
+}
+// s += a x + b y
+template <class T>
+__device__ __forceinline__ void hm_mac2(T& s, T a, T x, T b, T y) {
+  hm_fma(s, a, x);
+  hm_fma(s, b, y);
+}
+__device__ __forceinline__ void hm_mac2(dfl& s, dfl a, dfl x, dfl b, dfl y) {
+  dfl t = dfl_prod(a, x);
+  dfl_mac(t, b, y);
+  s += t;
 }
 __device__ __forceinline__ float hm_4p(float v, float s) { return fmaf(4.0f, v, s); }
 __device__ __forceinline__ double hm_4p(double v, double s) { return fma(4.0, v, s); }
@@ -157,12 +170,12 @@ __global__ void __launch_bounds__(HM_THREADS, HmT<T>::MINB)
   const X* x[NV];
 #pragma unroll
   for (int v = 0; v < NV; ++v) x[v] = xs + (long long)(v0 + (v < nv ? v : 0)) * ld + p;
-  T h[3][NV], m[3][NV], xprev[NV];
+  T h[3][NV], m[3][NV], xprev[NV], p2prev[NV];
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
 #pragma unroll
     for (int o = 0; o < 3; ++o) h[o][v] = m[o][v] = T(0);
-    xprev[v] = T(0);
+    xprev[v] = p2prev[v] = T(0);
   }
   const int ke = min(k1, a.nzn - 1);
   for (int kp = max(k0 - 1, 0); kp <= ke; ++kp) {
@@ -203,28 +216,30 @@ __global__ void __launch_bounds__(HM_THREADS, HmT<T>::MINB)
           sb[v] += bv;
         }
 #pragma unroll
-        for (int o = 0; o < 3; ++o) {
-          hm_fma(h[o][v], c[o][0], xm);
-          hm_fma(h[o][v], c[o][1], xc);
-          hm_fma(h[o][v], c[o][2], xp);
-        }
+        for (int o = 0; o < 3; ++o) hm_mac3(h[o][v], c[o][0], xm, c[o][1], xc, c[o][2], xp);
       }
     }
-    // per output plane: x, y and z kinetic coefficients and the mass, for input planes o-1, o, o+1
-    T z[3][4];
+    // per output plane: x and y kinetic coefficients and the mass, for input planes o-1, o, o+1
+    T z[3][3];
 #pragma unroll
     for (int o = 0; o < 3; ++o)
 #pragma unroll
-      for (int q = 0; q < 4; ++q) z[o][q] = on[o] ? Tr::co(__ldg(zt + 12 * (kp + o - 1) + 3 * q + (2 - o))) : T(0);
+      for (int q = 0; q < 3; ++q)
+        z[o][q] = on[o] ? Tr::co(__ldg(zt + 12 * (kp + o - 1) + 3 * (q == 2 ? 3 : q) + (2 - o))) : T(0);
+    // z stiffness of the layer below plane kp, -w: plane kp gains w d, plane kp - 1 loses it. The first
+    // plane's sums towards planes that are not the chunk's are dropped, and plane 0 has no layer below
+    const T wz = Tr::co(__ldg(zt + 12 * kp + 6));
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
       const T p2 = hm_4p(a0[v], sa[v]), p1x = hm_4p(b0[v], sb[v]), p1y = hm_2m(a0[v], sa[v]);
+      const T d = p2 - p2prev[v];
+      p2prev[v] = p2;
+      hm_mac3(h[0][v], z[0][0], p1x, z[0][1], p1y, wz, d);
+      hm_mac3(h[1][v], z[1][0], p1x, z[1][1], p1y, wz, -d);
+      hm_mac2(h[2][v], z[2][0], p1x, z[2][1], p1y);
+      if (Op::mass) {
 #pragma unroll
-      for (int o = 0; o < 3; ++o) {
-        hm_fma(h[o][v], z[o][0], p1x);
-        hm_fma(h[o][v], z[o][1], p1y);
-        hm_fma(h[o][v], z[o][2], p2);
-        if (Op::mass) hm_fma(m[o][v], z[o][3], p2);
+        for (int o = 0; o < 3; ++o) hm_fma(m[o][v], z[o][2], p2);
       }
     }
 #pragma unroll
@@ -339,8 +354,9 @@ __global__ void __launch_bounds__(128) hm_rows_kernel(const double* __restrict__
     const size_t o = (size_t)q * ns + n;
     if (S32) S32[o] = (float)s;
     if (Sdf) {
-      const dfl f = dfl_from_bits(s);
-      Sdf[o] = make_float2(f.h, f.l);
+      // rounded to 49 bits (a truncated row entry biases a node's 27 products one way)
+      const float f = d2f_bits(s);
+      Sdf[o] = make_float2(f, d2f_bits(s - dfl_f2d(f)));
     }
     if (S64) S64[o] = s;
   }

@@ -25,7 +25,15 @@ static inline unsigned __float_as_uint(float a) { return pattern<unsigned>(a); }
 static inline float __uint_as_float(unsigned a) { return pattern<float>(a); }
 static inline float __double2float_rn(double a) { return (float)a; }
 
+#include "dfloat.cuh"
 #include "fpbits.cuh"
+
+using qcad::dfl;
+// One step of a double-float sum, product and sum renormalized.
+static dfl step(dfl s, dfl a, dfl b) {
+  const dfl p = qcad::dfl_prod(a, b);
+  return s + qcad::dfl_quick(p.h, p.l);
+}
 
 extern "C" {
 void h_times4(int n, const double* a, double* out) {
@@ -33,5 +41,26 @@ void h_times4(int n, const double* a, double* out) {
 }
 void h_d2f(int n, const double* a, float* out) {
   for (int i = 0; i < n; ++i) out[i] = qcad::d2f_bits(a[i]);
+}
+void h_split(int n, const double* a, double* out) {
+  for (int i = 0; i < n; ++i) {
+    const dfl d = qcad::dfl_from_bits(a[i]);
+    out[i] = (double)d.h + (double)d.l;
+  }
+}
+// Sums of 27 products c x (values already double-float exact): by groups of three as the stencil's rows,
+// and renormalized at every step.
+void h_rows(int n, const double* c, const double* x, double* grouped, double* stepped) {
+  for (int i = 0; i < n; ++i) {
+    dfl a(0), b(0), cd[27], xd[27];
+    for (int q = 0; q < 27; ++q) {
+      cd[q] = qcad::dfl_from_bits(c[27 * i + q]);
+      xd[q] = qcad::dfl_from_bits(x[27 * i + q]);
+    }
+    for (int q = 0; q < 27; q += 3) qcad::dfl_mac3(a, cd[q], xd[q], cd[q + 1], xd[q + 1], cd[q + 2], xd[q + 2]);
+    for (int q = 0; q < 27; ++q) b = step(b, cd[q], xd[q]);
+    grouped[i] = qcad::dfl_to_double(a);
+    stepped[i] = qcad::dfl_to_double(b);
+  }
 }
 }
