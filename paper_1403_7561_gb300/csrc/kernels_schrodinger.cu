@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include "dfloat.cuh"
+#include "launch_rules.h"
 
 #include <cstdlib>
 #include <cstring>
@@ -320,12 +321,13 @@ __global__ void __launch_bounds__(512) gram_kernel(long long n, int p, int nb2, 
 // so that the lanes of a warp read neighbouring columns without bank conflicts) and reads four rows per
 // 16-byte load: 8 loads for 64 products without an index computation per copied value, and three
 // blocks of 192 threads on an SM (one of 256 with a transposed copy took 314 us for 36 columns and
-// 735k rows). About 32 rows per thread (G tiles) are summed in FP32, these sums in double-float on the FP32 pipes.
+// 735k rows). At most 32 rows per thread (flush tiles) are summed in FP32, these sums in double-float on
+// the FP32 pipes.
 constexpr int G32_ROWS = 32, G32_STRIDE = G32_ROWS + 4;
 template <int THREADS>
 __global__ void __launch_bounds__(THREADS, THREADS == 192 ? 3 : 1) gram32_kernel(long long n, int p, int nb2, const float* A,
                                                                         long long lda, const float* B1, const float* B2,
-                                                                        long long ldb, double* part, int G) {
+                                                                        long long ldb, double* part, int G, int flush) {
   extern __shared__ __align__(16) unsigned char sh_raw[];
   float* sh = reinterpret_cast<float*>(sh_raw);  // three stages of [cols][G32_STRIDE]
   const int q = p, qt = q * nb2;
@@ -383,7 +385,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == 192 ? 3 : 1) gram32_kernel
             for (int w = 0; w < 4; ++w) s32[4 * u + v] = fmaf(av[u][w], bv[w], s32[4 * u + v]);
         }
       }
-      if (++since == G) {  // about 32 rows
+      if (++since == flush) {
         since = 0;
 #pragma unroll
         for (int s = 0; s < 16; ++s) {
@@ -599,7 +601,7 @@ void launch_gram(long long n, int p, int q, const T* A, long long lda, const T* 
   const int nt = ta_n * tb_n;
   if constexpr (std::is_same<T, float>::value) {
     const int cap = nt <= 192 ? 192 : 512;
-    const int G = std::max(1, std::min(8, cap / nt));
+    const int G = std::max(1, std::min(8, cap / nt)), flush = gram32_flush_tiles(G);
     const int nth = std::min(cap, ((G * nt + 31) / 32) * 32);
     const long long want = cap == 192 ? 3LL * sm_count() : GRAM_MAX_BLOCKS;
     const int nblk = (int)std::max<long long>(
@@ -613,9 +615,9 @@ void launch_gram(long long n, int p, int q, const T* A, long long lda, const T* 
              cudaFuncSetAttribute(gram32_kernel<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024) ==
                  cudaSuccess;
     if (cap == 192)
-      note_launch(), gram32_kernel<192><<<nblk, nth, shm, s>>>(n, p, nb2, A, lda, B1, B2, ldb, part, G);
+      note_launch(), gram32_kernel<192><<<nblk, nth, shm, s>>>(n, p, nb2, A, lda, B1, B2, ldb, part, G, flush);
     else
-      note_launch(), gram32_kernel<512><<<nblk, nth, shm, s>>>(n, p, nb2, A, lda, B1, B2, ldb, part, G);
+      note_launch(), gram32_kernel<512><<<nblk, nth, shm, s>>>(n, p, nb2, A, lda, B1, B2, ldb, part, G, flush);
     const int tot = p * p * nb2;
     note_launch(), gram_reduce_kernel<<<(tot + 31) / 32, dim3(32, 8), 0, s>>>(nblk, tot, p * p, part, G1, G2);
     return;

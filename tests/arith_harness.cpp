@@ -27,6 +27,7 @@ static inline float __double2float_rn(double a) { return (float)a; }
 
 #include "dfloat.cuh"
 #include "fpbits.cuh"
+#include "launch_rules.h"
 
 using qcad::dfl;
 // One step of a double-float sum, product and sum renormalized.
@@ -63,4 +64,5 @@ void h_rows(int n, const double* c, const double* x, double* grouped, double* st
     stepped[i] = qcad::dfl_to_double(b);
   }
 }
+int h_gram32_flush(int groups) { return qcad::gram32_flush_tiles(groups); }
 }

@@ -92,3 +92,10 @@ def test_grouped_sums_are_as_accurate_as_renormalized_steps(lib):
         return np.sqrt(np.mean([float(Fraction(v[i]) - exact[i]) ** 2 for i in range(n)])) / size
 
     assert rms(g) <= 1.2 * rms(s), (rms(g), rms(s))
+
+
+@pytest.mark.parametrize("groups", range(1, 9))
+def test_fp32_gram_sums_at_most_32_rows(lib, groups):
+    flush = lib.h_gram32_flush(groups)
+    chunks = max(len(range(g, 8, groups)) for g in range(groups))  # of four rows, per tile and group
+    assert 16 < 4 * chunks * flush <= 32
