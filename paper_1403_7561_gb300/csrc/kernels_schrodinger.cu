@@ -590,6 +590,17 @@ static bool dense_df() {
   return df;
 }
 
+// Up to `bytes` of dynamic shared memory for the kernels on the current device; a failure shows as the
+// launch's error, which the callers check.
+template <class... K>
+static void shared_opt_in(PerDevice& state, int bytes, K... kernels) {
+  int dev = -1;
+  cudaGetDevice(&dev);
+  once_per_device(state, dev, [&] {
+    return ((cudaFuncSetAttribute(kernels, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess) && ...);
+  });
+}
+
 template <class T>
 void launch_gram(long long n, int p, int q, const T* A, long long lda, const T* B1, const T* B2, long long ldb,
                  double* G1, double* G2, double* part, cudaStream_t s, bool upper) {
@@ -608,12 +619,8 @@ void launch_gram(long long n, int p, int q, const T* A, long long lda, const T* 
         1, std::min<long long>(std::min<long long>(want, GRAM_MAX_BLOCKS), (n + G32_ROWS - 1) / G32_ROWS));
     const size_t shm = std::max((size_t)nt * 16 * sizeof(double),
                                 (size_t)3 * 4 * (ta_n + tb_n) * G32_STRIDE * sizeof(float));
-    static bool attr = false;
-    if (!attr)
-      attr = cudaFuncSetAttribute(gram32_kernel<192>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024) ==
-                 cudaSuccess &&
-             cudaFuncSetAttribute(gram32_kernel<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024) ==
-                 cudaSuccess;
+    static PerDevice attr;
+    shared_opt_in(attr, 128 * 1024, gram32_kernel<192>, gram32_kernel<512>);
     if (cap == 192)
       note_launch(), gram32_kernel<192><<<nblk, nth, shm, s>>>(n, p, nb2, A, lda, B1, B2, ldb, part, G, flush);
     else
@@ -628,9 +635,8 @@ void launch_gram(long long n, int p, int q, const T* A, long long lda, const T* 
   const int nblk = (int)std::max<long long>(1, std::min<long long>(2LL * sm_count(), ntiles));
   const size_t red = (size_t)G * nt * 16 * sizeof(double);  // the groups' sums, after the tiles
   const size_t shm = std::max(red, (size_t)2 * GR * (4 * ta_n + 4 * tb_n + 4) * sizeof(T));
-  static bool attr = false;
-  if (!attr)
-    attr = cudaFuncSetAttribute(gram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024) == cudaSuccess;
+  static PerDevice attr;
+  shared_opt_in(attr, 160 * 1024, gram_kernel);
   {
     if (dense_df()) {
       // the upper triangles only (the caller mirrors them)
@@ -643,12 +649,8 @@ void launch_gram(long long n, int p, int q, const T* A, long long lda, const T* 
       // two double stages plus the hi and lo float tiles
       const size_t shm_df =
           std::max(red_df, (size_t)2 * DGR * (p * (1 + nb2) * sizeof(double) + (4 * ta_n + 4 * tb_df + 4) * sizeof(float)));
-      static bool attr_df = false;
-      if (!attr_df)
-        attr_df = cudaFuncSetAttribute(gram_df_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) ==
-                      cudaSuccess &&
-                  cudaFuncSetAttribute(gram_df_kernel<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) ==
-                      cudaSuccess;
+      static PerDevice attr_df;
+      shared_opt_in(attr_df, 200 * 1024, gram_df_kernel<256>, gram_df_kernel<512>);
       if (cap == 256)
         note_launch(), gram_df_kernel<256><<<nblk, nth_df, shm_df, s>>>(n, p, nb2, A, lda, B1, B2, ldb, part, G_df, up);
       else

@@ -65,4 +65,16 @@ void h_rows(int n, const double* c, const double* x, double* grouped, double* st
   }
 }
 int h_gram32_flush(int groups) { return qcad::gram32_flush_tiles(groups); }
+// once_per_device over a list of devices whose set() fails for the first `fails` calls: the calls of
+// set() per launch.
+void h_once(int n, const int* devices, int fails, int* calls) {
+  qcad::PerDevice state;
+  for (int i = 0; i < n; ++i) {
+    calls[i] = 0;
+    qcad::once_per_device(state, devices[i], [&] {
+      ++calls[i];
+      return fails-- <= 0;
+    });
+  }
+}
 }

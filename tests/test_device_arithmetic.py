@@ -99,3 +99,12 @@ def test_fp32_gram_sums_at_most_32_rows(lib, groups):
     flush = lib.h_gram32_flush(groups)
     chunks = max(len(range(g, 8, groups)) for g in range(groups))  # of four rows, per tile and group
     assert 16 < 4 * chunks * flush <= 32
+
+
+@pytest.mark.parametrize("devices,fails,want", [([0, 0, 1, 1, 0, 63, 63], 0, [1, 0, 1, 0, 0, 1, 0]),
+                                                ([0, 0, 0, 1, 1], 1, [1, 1, 0, 1, 0]),
+                                                ([-1, -1, 64, 64], 0, [1, 1, 1, 1])])
+def test_function_attributes_are_set_on_every_device(lib, devices, fails, want):
+    calls = (C.c_int * len(devices))()
+    lib.h_once(len(devices), (C.c_int * len(devices))(*devices), fails, calls)
+    assert list(calls) == want
