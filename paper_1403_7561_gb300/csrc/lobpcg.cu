@@ -60,6 +60,18 @@ struct SubSetup {
   explicit SubSetup(qcad_mesh_s* m) : cV64(m->s_cV), dinv(m->s_dinv), interior(m->s_interior) {}
 };
 
+// The mesh's Schrodinger workspace for the duration of a call on stream s. A call that returns has
+// synchronized s; one that throws may leave work behind, which ends before the next call may start.
+struct SchrodingerUse {
+  std::unique_lock<std::mutex> lock;
+  cudaStream_t s;
+  int thrown;
+  SchrodingerUse(qcad_mesh_s* m, cudaStream_t s_) : lock(m->s_mu), s(s_), thrown(std::uncaught_exceptions()) {}
+  ~SchrodingerUse() {
+    if (std::uncaught_exceptions() > thrown) cudaStreamSynchronize(s);
+  }
+};
+
 // rows: the precisions to assemble (ROWS_*).
 // SETUP_EIGS: an eigensolve (the Jacobi scale and the interior mask too).
 enum { ROWS_32 = 1, ROWS_DF = 2, ROWS_64 = 4, SETUP_EIGS = 8 };
@@ -210,6 +222,7 @@ qcad_status schrodinger_apply(qcad_mesh_s* m, const qcad_bias* b, const double* 
                               const double* X, double* HX, double* MX, int precision) {
   if (!b || !phi || !m_eff || !X || nvec < 1) throw Error(QCAD_ERR_INVALID_ARG, "null pointer or nvec < 1");
   if (precision != 0 && precision != 1) throw Error(QCAD_ERR_INVALID_ARG, "precision must be 0 or 1");
+  SchrodingerUse use(m, m->stream);
   SubSetup S(m);
   setup_sub(m, b, phi, m_eff, precision ? ROWS_32 : ROWS_64, S, mesh_io(m));
   cudaStream_t s = m->stream;
@@ -760,6 +773,7 @@ qcad_status schrodinger_eigs_io(qcad_mesh_s* m, const EigIo& io, const qcad_bias
   if (!b || !phi || !m_eff || !evals) throw Error(QCAD_ERR_INVALID_ARG, "null pointer");
   if (nev < 1 || nev > 16) throw Error(QCAD_ERR_INVALID_ARG, "nev must be in [1, 16]");
   if (!(tol > 0)) throw Error(QCAD_ERR_INVALID_ARG, "tol must be > 0");
+  SchrodingerUse use(m, io.s);
   SubSetup S(m);
   setup_sub(m, b, phi, m_eff, ROWS_32 | ROWS_DF | ROWS_64 | SETUP_EIGS, S, io, vxq, shift_floor);
   const double t_setup = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();

@@ -184,8 +184,10 @@ struct qcad_mesh_s {
   long long lam_ver[2] = {-1, -1};
   double lam_cache[2] = {0.0, 0.0};
   qcad::Profiler prof;                     // thread-safe: concurrent calls may record
-  // Schrodinger workspace
-  // (kept between calls; one eigensolve or block apply runs on a mesh at a time)
+  // Schrodinger workspace, kept between calls: an eigensolve or block apply holds s_mu (SchrodingerUse)
+  // from its first launch until its stream has finished, so that calls of several host threads and on both
+  // of the mesh's streams follow one another
+  std::mutex s_mu;
   qcad::DevBuf s_cV, s_dinv, s_interior, s_tab;   // potential coefficients, Jacobi scale, interior mask, plane tables
   qcad::DevBuf s_mom, s_S32, s_Sdf, s_S64;        // the V rows of the subdomain and the scratch of their assembly
   qcad::DevBuf s_full, s_tmp32;                   // block applies: vectors on all subdomain nodes
