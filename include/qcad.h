@@ -240,7 +240,11 @@ qcad_status qcad_adjoint(qcad_mesh_t m, const qcad_bias* b, const qcad_solver_op
  * Eq. SchrodPotEnergy without V_xc): for the nvec columns of X (device,
  * n_sub_dof x nvec, column-major, interior subdomain nodes in node order),
  * HX = H X and MX = M X (either may be NULL). phi: device [n_nodes].
- * m_eff: host [3] (m_x, m_y, m_z) in m0. precision 0 FP64, 1 FP32 apply. */
+ * m_eff: host [3] (m_x, m_y, m_z) in m0. precision 0 FP64, 1 FP32 apply.
+ * The mesh keeps the workspace of this call and of the eigensolves for the next
+ * one, up to 1 GiB (about 400 bytes per subdomain node, 64 MB, and 24 bytes per
+ * node and vector of the widest block); calls of several host threads on one
+ * mesh wait for one another. */
 qcad_status qcad_schrodinger_apply(qcad_mesh_t m, const qcad_bias* b, const double* phi, const double* m_eff,
                                    int nvec, const double* X, double* HX, double* MX, int precision);
 

@@ -19,6 +19,7 @@
 #include <cuda_runtime.h>
 
 #include "dfloat.cuh"
+#include "launch_rules.h"
 #include "qcad_host.h"
 #include "qcad_internal.cuh"
 
@@ -326,15 +327,16 @@ __global__ void __launch_bounds__(256) hm_moments_kernel(const double* __restric
 // Row of node (i, j, k): along each axis the offset -1 comes from the left element's pair (0, 1), the
 // offset +1 from the right one's, the offset 0 from the left's (1, 1) and the right's (0, 0). Rows of
 // boundary nodes are zero.
-__global__ void __launch_bounds__(128) hm_rows_kernel(const double* __restrict__ mom, int nxn, int nyn, int nzn,
-                                                      float* S32, float2* Sdf, double* S64) {
-  const int n = blockIdx.x * 128 + threadIdx.x;
+// (p0, p1): the node planes of the launch; mom holds the layers from e0 on, ne elements.
+__global__ void __launch_bounds__(128) hm_rows_kernel(const double* __restrict__ mom, int nxn, int nyn, int nzn, int p0,
+                                                      int p1, int e0, int ne, float* S32, float2* Sdf, double* S64) {
+  const int n = blockIdx.x * 128 + threadIdx.x + nxn * nyn * p0;
   const int ns = nxn * nyn * nzn;
-  if (n >= ns) return;
+  if (n >= nxn * nyn * p1) return;
   const int i = n % nxn, j = (n / nxn) % nyn, k = n / (nxn * nyn);
-  const int nx = nxn - 1, ny = nyn - 1, nz = nzn - 1, ne = nx * ny * nz;
+  const int nx = nxn - 1, ny = nyn - 1, nz = nzn - 1;
   const bool in = i > 0 && j > 0 && k > 0 && i < nx && j < ny && k < nz;
-  const int e = in ? (i - 1) + nx * ((j - 1) + ny * (k - 1)) : 0;  // the lower left element
+  const int e = in ? (i - 1) + nx * ((j - 1) + ny * (k - 1 - e0)) : 0;  // the lower left element
 #pragma unroll
   for (int q = 0; q < 27; ++q) {
     const int d[3] = {q % 3, (q / 3) % 3, q / 9};  // offset + 1
@@ -377,12 +379,18 @@ void launch_hm_jacobi(int nxn, int nyn, int nzn, const double* dk, double* dinv,
   hm_jacobi_kernel<<<dim3((nxn * nyn + 255) / 256, nzn), 256, 0, s>>>(nxn, nyn, nzn, dk, dinv, interior);
 }
 
-void launch_hm_rows(const double* cV, int nxn, int nyn, int nzn, double* mom, float* S32, float2* Sdf, double* S64,
-                    cudaStream_t s) {
-  const int ne = (nxn - 1) * (nyn - 1) * (nzn - 1), ns = nxn * nyn * nzn;
-  note_launch(2);
-  hm_moments_kernel<<<(ne + 255) / 256, 256, 0, s>>>(cV, ne, mom);
-  hm_rows_kernel<<<(ns + 127) / 128, 128, 0, s>>>(mom, nxn, nyn, nzn, S32, Sdf, S64);
+void launch_hm_rows(const double* cV, int nxn, int nyn, int nzn, int slab, double* mom, float* S32, float2* Sdf,
+                    double* S64, cudaStream_t s) {
+  const int layer = (nxn - 1) * (nyn - 1), plane = nxn * nyn;
+  for (int p0 = 0; p0 < nzn;) {
+    const HmSlab b = hm_next_slab(p0, nzn - 1, slab);
+    const int ne = layer * (b.e1 - b.e0);
+    note_launch(2);
+    hm_moments_kernel<<<(ne + 255) / 256, 256, 0, s>>>(cV + 8LL * layer * b.e0, ne, mom);
+    hm_rows_kernel<<<(plane * (b.p1 - b.p0) + 127) / 128, 128, 0, s>>>(mom, nxn, nyn, nzn, b.p0, b.p1, b.e0, ne, S32,
+                                                                       Sdf, S64);
+    p0 = b.p1;
+  }
 }
 
 }  // namespace qcad

@@ -18,7 +18,7 @@
 #include <string>
 #include <vector>
 
-#include "dfloat.cuh"
+#include "launch_rules.h"
 #include "mesh.h"
 
 namespace qcad {
@@ -49,7 +49,8 @@ struct SubSetup {
   long long ns;     // subdomain nodes
   long long ndof;   // interior nodes
   DevBuf &cV64, &dinv, &interior;  // the mesh's workspaces
-  // the assembled operators: FP32, double-float (the FP64 phase's applies) and FP64
+  // the assembled operators: FP32, and double-float (the FP64 phase's applies) or FP64 (its last ones), which
+  // share one buffer: S is null in the one that it does not hold
   HmStencil<float> st32{};
   HmStencil<float2> stdf{};
   HmStencil<double> st64{};
@@ -61,34 +62,57 @@ struct SubSetup {
 };
 
 // The mesh's Schrodinger workspace for the duration of a call on stream s. A call that returns has
-// synchronized s; one that throws may leave work behind, which ends before the next call may start.
+// synchronized s; one that throws may leave work behind, which ends before the next call may start. What
+// the call leaves above SCHRODINGER_KEEP is given back, the block vectors first: up to there a repeated
+// call finds its buffers (allocating them took two thirds of a 1.09 ms block apply), above it a mesh would
+// hold gigabytes for one wide block or a subdomain of millions of nodes.
 struct SchrodingerUse {
   std::unique_lock<std::mutex> lock;
+  qcad_mesh_s* m;
   cudaStream_t s;
   int thrown;
-  SchrodingerUse(qcad_mesh_s* m, cudaStream_t s_) : lock(m->s_mu), s(s_), thrown(std::uncaught_exceptions()) {}
+  SchrodingerUse(qcad_mesh_s* m_, cudaStream_t s_)
+      : lock(m_->s_mu), m(m_), s(s_), thrown(std::uncaught_exceptions()) {}
   ~SchrodingerUse() {
     if (std::uncaught_exceptions() > thrown) cudaStreamSynchronize(s);
+    DevBuf* const bufs[] = {&m->s_full, &m->s_tmp32, &m->s_S8, &m->s_S32, &m->s_mom,
+                            &m->s_cV,   &m->s_dinv,  &m->s_interior, &m->s_tab};
+    size_t held = 0;
+    for (const DevBuf* b : bufs) held += b->bytes;
+    for (DevBuf* b : bufs) {
+      if (held <= SCHRODINGER_KEEP) break;
+      held -= b->bytes;
+      b->release();
+    }
   }
 };
 
 // rows: the precisions to assemble (ROWS_*).
 // SETUP_EIGS: an eigensolve (the Jacobi scale and the interior mask too).
 enum { ROWS_32 = 1, ROWS_DF = 2, ROWS_64 = 4, SETUP_EIGS = 8 };
+static void build_rows(qcad_mesh_s* m, int rows, SubSetup& S, cudaStream_t s) {
+  const SubdomainMap& sm = S.sm;
+  const int slab = hm_slab_layers(sm.nxs, sm.nys, sm.nzs);
+  m->s_mom.ensure((size_t)27 * sm.nxs * sm.nys * slab * sizeof(double) + 64);
+  float* s32 = nullptr;
+  if (rows & ROWS_32) {
+    m->s_S32.ensure((size_t)27 * S.ns * sizeof(float) + 64);
+    s32 = m->s_S32.as<float>();
+    S.st32.S = s32;
+  }
+  if (rows & (ROWS_DF | ROWS_64)) {
+    static_assert(sizeof(float2) == sizeof(double), "the rows share a buffer");
+    m->s_S8.ensure((size_t)27 * S.ns * sizeof(double) + 64);
+    S.stdf.S = rows & ROWS_DF ? m->s_S8.as<float2>() : nullptr;
+    S.st64.S = rows & ROWS_64 ? m->s_S8.as<double>() : nullptr;
+  }
+  launch_hm_rows(S.cV64.as<double>(), sm.nxs + 1, sm.nys + 1, sm.nzs + 1, slab, m->s_mom.as<double>(), s32,
+                 rows & ROWS_DF ? m->s_S8.as<float2>() : nullptr, rows & ROWS_64 ? m->s_S8.as<double>() : nullptr, s);
+}
 static void assemble_rows(qcad_mesh_s* m, const GridTables& t, double hx, double hy, int rows, SubSetup& S,
                           cudaStream_t s) {
   const int nxn = S.sm.nxs + 1, nyn = S.sm.nys + 1, nzn = S.sm.nzs + 1;
-  const long long nes = (long long)S.sm.nxs * S.sm.nys * S.sm.nzs;
-  m->s_mom.ensure((size_t)27 * nes * sizeof(double) + 64);
-  auto buf = [&](DevBuf& b, int bit, size_t e) -> void* {
-    if (!(rows & bit)) return nullptr;
-    b.ensure((size_t)27 * S.ns * e + 64);
-    return b.p;
-  };
-  float* s32 = static_cast<float*>(buf(m->s_S32, ROWS_32, sizeof(float)));
-  float2* sdf = static_cast<float2*>(buf(m->s_Sdf, ROWS_DF, sizeof(float2)));
-  double* s64 = static_cast<double*>(buf(m->s_S64, ROWS_64, sizeof(double)));
-  launch_hm_rows(S.cV64.as<double>(), nxn, nyn, nzn, m->s_mom.as<double>(), s32, sdf, s64, s);
+  build_rows(m, rows, S, s);
   // kinetic and mass coefficients of the planes, with the x and y step sizes of the a and b sums, in the
   // three precisions, then the interior diagonal of the kinetic part: one upload
   const size_t nz = (size_t)12 * nzn;
@@ -122,9 +146,9 @@ static void assemble_rows(qcad_mesh_s* m, const GridTables& t, double hx, double
     S.interior.ensure(S.ns + 64);
     launch_hm_jacobi(nxn, nyn, nzn, dkd, S.dinv.as<double>(), S.interior.as<unsigned char>(), s);
   }
-  S.st32 = {s32, z32, nxn, nyn, nzn};
-  S.stdf = {sdf, zdf, nxn, nyn, nzn};
-  S.st64 = {s64, z64, nxn, nyn, nzn};
+  S.st32 = {S.st32.S, z32, nxn, nyn, nzn};
+  S.stdf = {S.stdf.S, zdf, nxn, nyn, nzn};
+  S.st64 = {S.st64.S, z64, nxn, nyn, nzn};
 }
 
 // vxq: an extra potential energy at the subdomain's Gauss points (eV, [element][point]) or null;
@@ -404,7 +428,9 @@ struct LobpcgRun {
     if constexpr (sizeof(T) == 8) {
       // FP64 vectors: H and M in double-float arithmetic on the FP32 pipes while the residuals are
       // above DF_FLOOR, FP64 applies below it; QCAD_LOBPCG_NATIVE64 selects FP64 ones throughout
-      if (df_ok && use_df_apply())
+      const bool df = df_ok && use_df_apply();
+      if (df ? S->stdf.S == nullptr : S->st64.S == nullptr) build_rows(m, df ? ROWS_DF : ROWS_64, *S, s);
+      if (df)
         launch_hm_stencil(S->stdf, a, s);
       else
         launch_hm_stencil(S->st64, a, s);
@@ -775,7 +801,7 @@ qcad_status schrodinger_eigs_io(qcad_mesh_s* m, const EigIo& io, const qcad_bias
   if (!(tol > 0)) throw Error(QCAD_ERR_INVALID_ARG, "tol must be > 0");
   SchrodingerUse use(m, io.s);
   SubSetup S(m);
-  setup_sub(m, b, phi, m_eff, ROWS_32 | ROWS_DF | ROWS_64 | SETUP_EIGS, S, io, vxq, shift_floor);
+  setup_sub(m, b, phi, m_eff, ROWS_32 | ROWS_DF | SETUP_EIGS, S, io, vxq, shift_floor);
   const double t_setup = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
   if (S.ndof < 3 * (nev + 4)) throw Error(QCAD_ERR_INVALID_ARG, "subdomain too small for nev");
   cudaStream_t s = io.s;

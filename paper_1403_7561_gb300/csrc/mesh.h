@@ -64,6 +64,9 @@ struct GridTables {
   std::vector<double> mx, kx, my, ky, mzx, mzy, kzz;
 };
 
+// Device memory that a mesh keeps of its Schrodinger workspace between calls, at most.
+constexpr size_t SCHRODINGER_KEEP = (size_t)1 << 30;
+
 // Per-precision device copy of a grid's tables.
 template <class T>
 struct GridDev {
@@ -189,7 +192,8 @@ struct qcad_mesh_s {
   // of the mesh's streams follow one another
   std::mutex s_mu;
   qcad::DevBuf s_cV, s_dinv, s_interior, s_tab;   // potential coefficients, Jacobi scale, interior mask, plane tables
-  qcad::DevBuf s_mom, s_S32, s_Sdf, s_S64;        // the V rows of the subdomain and the scratch of their assembly
+  // the scratch of the V rows' assembly (a slab of layers), the rows in FP32, and in double-float or FP64
+  qcad::DevBuf s_mom, s_S32, s_S8;
   qcad::DevBuf s_full, s_tmp32;                   // block applies: vectors on all subdomain nodes
   ~qcad_mesh_s();
 };

@@ -224,9 +224,10 @@ void launch_hm_stencil(const HmStencil<float>& st, const HmArgs<float>& a, cudaS
 void launch_hm_stencil(const HmStencil<double>& st, const HmArgs<double>& a, cudaStream_t s);
 void launch_hm_stencil(const HmStencil<float2>& st, const HmArgs<double>& a, cudaStream_t s);
 // The rows of the subdomain grid from its coefficients cV (8 per element), in the precisions whose
-// output is not null; mom: scratch of 27 doubles per element.
-void launch_hm_rows(const double* cV, int nxn, int nyn, int nzn, double* mom, float* S32, float2* Sdf, double* S64,
-                    cudaStream_t s);
+// output is not null; mom: scratch of 27 doubles per element of `slab` element layers, which are
+// assembled at a time (hm_slab_layers).
+void launch_hm_rows(const double* cV, int nxn, int nyn, int nzn, int slab, double* mom, float* S32, float2* Sdf,
+                    double* S64, cudaStream_t s);
 // Jacobi scale 1 / dk[k] of the interior nodes (0 on the boundary) and the interior mask.
 void launch_hm_jacobi(int nxn, int nyn, int nzn, const double* dk, double* dinv, unsigned char* interior, cudaStream_t s);
 // One fused step of the LOBPCG Chebyshev-Jacobi block preconditioner (kernels_hm.cu): the H apply

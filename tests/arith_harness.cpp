@@ -77,4 +77,15 @@ void h_once(int n, const int* devices, int fails, int* calls) {
     });
   }
 }
+int h_slab_layers(int nx, int ny, int nz) { return qcad::hm_slab_layers(nx, ny, nz); }
+// The slabs of an assembly as rows of e0, e1, p0, p1; returns their number (at most max).
+int h_slabs(int nz, int slab, int max, int* out) {
+  int n = 0;
+  for (int p0 = 0; p0 <= nz && n < max; ++n) {
+    const qcad::HmSlab b = qcad::hm_next_slab(p0, nz, slab);
+    out[4 * n] = b.e0, out[4 * n + 1] = b.e1, out[4 * n + 2] = b.p0, out[4 * n + 3] = b.p1;
+    p0 = b.p1;
+  }
+  return n;
+}
 }

@@ -108,3 +108,17 @@ def test_function_attributes_are_set_on_every_device(lib, devices, fails, want):
     calls = (C.c_int * len(devices))()
     lib.h_once(len(devices), (C.c_int * len(devices))(*devices), fails, calls)
     assert list(calls) == want
+
+
+@pytest.mark.parametrize("nx,ny,nz", [(1, 1, 1), (2, 2, 2), (64, 64, 32), (128, 128, 44), (500, 620, 7), (8192, 30, 9),
+                                      (4, 4, 65535)])
+def test_slabs_cover_every_plane_with_its_layers(lib, nx, ny, nz):
+    slab = lib.h_slab_layers(nx, ny, nz)
+    assert slab * 216 * nx * ny <= 64 << 20 or slab == min(2, nz)
+    out = (C.c_int * (4 * (nz + 1)))()
+    n = lib.h_slabs(nz, slab, nz + 1, out)
+    rows = np.array(out).reshape(-1, 4)[:n]
+    assert rows[0, 2] == 0 and rows[-1, 3] == nz + 1 and np.array_equal(rows[1:, 2], rows[:-1, 3])
+    for e0, e1, p0, p1 in rows:
+        assert 0 <= e0 < e1 <= nz and e1 - e0 <= slab and p0 < p1
+        assert e0 <= max(p0 - 1, 0) and min(p1 - 1, nz - 1) < e1  # the layers below and above every plane

@@ -65,3 +65,43 @@ def test_block_applies_of_several_threads(q):
     for t in threads:
         t.join()
     assert not errors, errors
+
+
+def held(q, call):
+    """Device bytes that a call leaves allocated (torch's own stay in its pool)."""
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    call()
+    torch.cuda.synchronize()
+    return before - torch.cuda.mem_get_info()[0]
+
+
+def test_a_wide_block_apply_gives_its_memory_back(q):
+    # 400 vectors on 65 x 65 x 33 nodes take 1.3 GB of block vectors; 1 GiB stays at most
+    dev = W.five_gate_device(n=(128, 128, 96), T=4.0)
+    m = q.qcad_mesh_create(dev)
+    phi = torch.zeros(m.n_nodes, dtype=torch.float64, device="cuda")
+    X = torch.ones(400, interior(dev), dtype=torch.float64, device="cuda")
+    HX, M1 = torch.empty_like(X), torch.empty_like(X[:1])
+    H1 = torch.empty_like(M1)
+    q.qcad_schrodinger_apply(m, dev["bias"], phi, M_EFF, X[:1].contiguous(), H1, M1)
+    assert held(q, lambda: q.qcad_schrodinger_apply(m, dev["bias"], phi, M_EFF, X, HX)) <= (1 << 30) + (4 << 20)
+    assert torch.equal(HX[399], H1[0])
+    q.qcad_schrodinger_apply(m, dev["bias"], phi, M_EFF, X[:1].contiguous(), H1, M1)  # after the release
+    assert torch.equal(HX[0], H1[0])
+
+
+def test_an_eigensolve_holds_what_its_rows_take(q):
+    # per subdomain node: rows in FP32 and in double-float or FP64 (27 x 12 B), potential coefficients (64 B),
+    # Jacobi scale and mask (9 B); the assembly's 64 MB; 2 MB pages of nine buffers
+    dev = W.five_gate_device(n=(256, 256, 128), T=0.5)
+    s = dev["subdomain"]
+    nodes = (s["i1"] - s["i0"] + 1) * (s["j1"] - s["j0"] + 1) * (s["k1"] - s["k0"] + 1)
+    small = W.five_gate_device(n=(64, 64, 48), T=0.5)  # loads the kernels
+    ms = q.qcad_mesh_create(small)
+    q.qcad_schrodinger_eigs(ms, small["bias"], torch.zeros(ms.n_nodes, dtype=torch.float64, device="cuda"), nev=2,
+                            m_eff=M_EFF, tol=1e-6)
+    m = q.qcad_mesh_create(dev)
+    phi = torch.zeros(m.n_nodes, dtype=torch.float64, device="cuda")
+    bytes_ = held(q, lambda: q.qcad_schrodinger_eigs(m, dev["bias"], phi, nev=2, m_eff=M_EFF, tol=1e-6))
+    assert bytes_ <= 397 * nodes + (64 << 20) + 9 * (2 << 20)
