@@ -366,17 +366,18 @@ __global__ void __launch_bounds__(128) hm_rows_kernel(const double* __restrict__
 
 __global__ void __launch_bounds__(256) hm_jacobi_kernel(int nxn, int nyn, int nzn, const double* __restrict__ dk,
                                                         double* dinv, unsigned char* interior) {
-  const int p = blockIdx.x * 256 + threadIdx.x, k = blockIdx.y;
-  if (p >= nxn * nyn) return;
-  const int j = p / nxn, i = p - j * nxn;
+  const int n = blockIdx.x * 256 + threadIdx.x;
+  if (n >= nxn * nyn * nzn) return;
+  const int k = n / (nxn * nyn), p = n - k * (nxn * nyn), j = p / nxn, i = p - j * nxn;
   const bool in = i > 0 && j > 0 && k > 0 && i < nxn - 1 && j < nyn - 1 && k < nzn - 1;
-  dinv[p + k * nxn * nyn] = in ? 1.0 / dk[k] : 0.0;
-  interior[p + k * nxn * nyn] = in ? 1 : 0;
+  dinv[n] = in ? 1.0 / dk[k] : 0.0;
+  interior[n] = in ? 1 : 0;
 }
+// One row of blocks over all nodes: a subdomain may have more planes than a grid's second axis (65535).
 void launch_hm_jacobi(int nxn, int nyn, int nzn, const double* dk, double* dinv, unsigned char* interior,
                       cudaStream_t s) {
   note_launch();
-  hm_jacobi_kernel<<<dim3((nxn * nyn + 255) / 256, nzn), 256, 0, s>>>(nxn, nyn, nzn, dk, dinv, interior);
+  hm_jacobi_kernel<<<(nxn * nyn * nzn + 255) / 256, 256, 0, s>>>(nxn, nyn, nzn, dk, dinv, interior);
 }
 
 void launch_hm_rows(const double* cV, int nxn, int nyn, int nzn, int slab, double* mom, float* S32, float2* Sdf,
