@@ -4,6 +4,7 @@ subdomain of as many planes as a mesh may have.
 Calls of several threads on one mesh give what they give one after the other (bit for bit: the
 block operators sum in a fixed order).
 """
+import math
 import threading
 
 import pytest
@@ -109,15 +110,16 @@ def test_an_eigensolve_holds_what_its_rows_take(q):
 
 
 def test_a_subdomain_of_65536_planes(q):
-    # a column of one interior node by 65534: its lowest level is that of 64 layers over the same height, but
-    # for the z discretization ((pi / 64)^2 / 12 of a z energy of 2e-4 eV)
+    # columns of one interior node by 63 and by 65534, layers of 1.5 nm: the lowest levels differ by the z
+    # energy of 64 layers, kappa 6 (1 - cos t) / ((2 + cos t) h^2) with t = pi / 64 (the other one's is 2e-10 eV)
     E = {}
     for nz in (64, 65535):
-        dev = dict(Lx=200.0, Ly=200.0, nx=2, ny=2, layers=[dict(material=0, thickness=100.0, n=nz)],
+        dev = dict(Lx=200.0, Ly=200.0, nx=2, ny=2, layers=[dict(material=0, thickness=1.5 * nz, n=nz)],
                    materials=[dict(W.SI)], gates=[], gate_work_function=None, bottom_ohmic=1, dots=[],
                    subdomain=dict(i0=0, i1=2, j0=0, j1=2, k0=0, k1=nz))
         m = q.qcad_mesh_create(dev)
         bias = dict(T=4.0, V_gate=[], V_sub=0.0, statistics=1, incomplete_ionization=1)
         phi = torch.zeros(m.n_nodes, dtype=torch.float64, device="cuda")
         E[nz] = q.qcad_schrodinger_eigs(m, bias, phi, nev=1, m_eff=M_EFF, tol=1e-8)[0][0]
-    assert abs(E[64] - E[65535]) < 1e-7
+    kappa, c = 0.0380998 / 0.19, math.cos(math.pi / 64)
+    assert abs(E[64] - E[65535] - kappa * 6 * (1 - c) / ((2 + c) * 1.5 ** 2)) < 1e-7
