@@ -386,9 +386,11 @@ qcad_status qcad_profile_read(qcad_mesh_t m, int kernel_class, int64_t* launches
  * Defaults: variant 3, 8 warps, z chunk 16; while a family's default stands, its
  * launches fit tile rows and z chunk to the grid (small grids take smaller ones).
  * qcad_autotune times the Jacobian apply of the given precision (0 FP64,
- * 1 FP32) over variants, tile rows and z chunks on the mesh, keeps the
- * fastest for that family and returns it (outputs may be NULL); best_ms is
- * its time per apply. */
+ * 1 FP32) over variants, tile rows and z chunks on the mesh, with the charge
+ * response of a coarse Newton solve at the bias (with response everywhere where
+ * b is NULL or cannot be solved), keeps the fastest for that family (the fitted
+ * default unless another is 3 % faster) and returns it (outputs may be NULL);
+ * best_ms is its time per apply. */
 qcad_status qcad_set_launch(qcad_mesh_t m, int family, int variant, int tile_rows, int z_chunk);
 /* The current launch shape of a family (as qcad_set_launch) and, for families 1 (FP64) and
  * 2 (FP32), the preconditioner the mesh's autotuner chose, coded as cheb_degree in

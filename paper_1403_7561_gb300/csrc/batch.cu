@@ -13,27 +13,53 @@ namespace qcad {
 qcad_status poisson_solve(qcad_mesh_s* m, const qcad_bias* b, const qcad_solver_opts* o, const double* theta,
                           double* phi, qcad_solve_report* rep);
 
-// Times the Jacobian apply (zero input and coefficients: the time does not depend on the
-// values) for every (variant, tile rows, z chunk) candidate and keeps the fastest for that
-// precision.
+bool linearize_for_tuning(qcad_mesh_s* m, const qcad_bias* b, int precision);
+
+// The vectors that a PCG overwrites, on a mesh of n nodes (the halves of p and d as in ensure_pcg).
+template <class T>
+static std::vector<void*> pcg_work_vectors(const PcgBufs<T>& k, long long n) {
+  const size_t half = vec_bytes<T>(n);
+  auto second = [&](const DevBuf& b) { return static_cast<void*>(b.as<unsigned char>() + half); };
+  return {k.z.p, k.Ap.p, k.x.p, k.p.p, k.r.p, second(k.p), k.w.p, k.d.p, second(k.d)};
+}
+
+// Times the Jacobian apply for every (variant, tile rows, z chunk) candidate and keeps the fastest
+// for that precision. The time depends on where the charge responds (the marches skip the mass term
+// elsewhere): at 256 x 256 x 128 elements the FP64 apply with response everywhere takes 1.07 ms, the one
+// of a solve 0.50 ms, so it runs the linearization of a solve at the bias, with its activity map, on the
+// PCG's vectors in turn: one pair of them would stay in the L2, which the nine of a solve do not at that
+// size. The fitted default stands unless a shape is FIT_MARGIN faster: the solve's other operators
+// (residual, smoother) take the same shape and rank differently within that. Without a linearization (no
+// valid bias) every element counts as responding. The vectors are zero: the time does not depend on them.
+constexpr float FIT_MARGIN = 0.03f;
 qcad_status autotune(qcad_mesh_s* m, const qcad_bias* b, int precision, int* variant_out, int* tile_rows,
                      int* z_chunk, float* best) {
-  (void)b;
   if (precision != 0 && precision != 1) throw Error(QCAD_ERR_INVALID_ARG, "precision must be 0 or 1");
+  const bool lin = linearize_for_tuning(m, b, precision);
   cudaStream_t s = m->stream;
   const long long n = m->n_nodes;
   const size_t es = precision == 0 ? sizeof(double) : sizeof(float);
   DevBuf v, y, c;
-  v.ensure(n * es + 64);
-  y.ensure(n * es + 64);
-  c.ensure((size_t)m->n_elems * 8 * es + 64);
-  CK(cudaMemsetAsync(v.p, 0, n * es, s));
-  CK(cudaMemsetAsync(c.p, 0, (size_t)m->n_elems * 8 * es, s));
+  std::vector<void*> vec;  // taken in turn as input and output
+  if (lin) {
+    vec = precision == 0 ? pcg_work_vectors(m->k64, n) : pcg_work_vectors(m->k32, n);
+  } else {
+    v.ensure(n * es + 64);
+    y.ensure(n * es + 64);
+    c.ensure((size_t)m->n_elems * 8 * es + 64);
+    CK(cudaMemsetAsync(c.p, 0, (size_t)m->n_elems * 8 * es, s));
+    vec = {v.p, y.p};
+  }
+  for (void* q : vec) CK(cudaMemsetAsync(q, 0, n * es, s));
+  const void* cp = !lin ? c.p : precision == 0 ? m->k64.c.p : m->k32.c.p;
+  const unsigned char* act =
+      !lin ? nullptr : precision == 0 ? m->k64.act.as<unsigned char>() : m->k32.act.as<unsigned char>();
+  const LaunchCfg fitted = default_lin_shape(precision, m->nxn, m->nyn, m->nzn, lin);
   const int chunks[5] = {8, 16, 32, 64, 128};
   cudaEvent_t e0, e1;
   CK(cudaEventCreate(&e0));
   CK(cudaEventCreate(&e1));
-  float best_ms = 1e30f;
+  float best_ms = 1e30f, def_ms = 1e30f;
   LaunchCfg best_cfg;
   int sms = 0;
   CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device));
@@ -60,6 +86,7 @@ qcad_status autotune(qcad_mesh_s* m, const qcad_bias* b, int precision, int* var
       const long long nch = std::max<long long>(1, (long long)w * sms * bps / std::max<long long>(1, tiles_xy));
       cands.push_back((int)std::max<long long>(2, (m->nzn + nch - 1) / nch));
     }
+    if (variant == fitted.variant && r == fitted.by) cands.push_back(fitted.kchunk);
     std::sort(cands.begin(), cands.end());
     cands.erase(std::unique(cands.begin(), cands.end()), cands.end());
     for (int ch : cands) {
@@ -69,31 +96,37 @@ qcad_status autotune(qcad_mesh_s* m, const qcad_bias* b, int precision, int* var
       cfg.kchunk = ch;
       cfg.variant = variant;
       cfg.fit = false;
-      auto run = [&]() {
+      auto run = [&](int q) {
+        const void* in = vec[q % vec.size()];
+        void* out = vec[(q + 1) % vec.size()];
         if (precision == 0) {
           ApplyArgs<double> a{};
-          a.v = v.as<double>();
-          a.y = y.as<double>();
-          a.c = c.as<double>();
+          a.v = static_cast<const double*>(in);
+          a.y = static_cast<double*>(out);
+          a.c = static_cast<const double*>(cp);
+          a.act = act;
           launch_apply<double>(m->g64.g, a, cfg, s, m->has_robin ? m->d_face64.as<double>() : nullptr);
         } else {
           ApplyArgs<float> a{};
-          a.v = v.as<float>();
-          a.y = y.as<float>();
-          a.c = c.as<float>();
+          a.v = static_cast<const float*>(in);
+          a.y = static_cast<float*>(out);
+          a.c = static_cast<const float*>(cp);
+          a.act = act;
           launch_apply<float>(m->g32.g, a, cfg, s, m->has_robin ? m->d_face32.as<float>() : nullptr);
         }
       };
-      run();
+      run(0);
       CK(cudaGetLastError());
       const int reps = 20;
       CK(cudaEventRecord(e0, s));
-      for (int q = 0; q < reps; ++q) run();
+      for (int q = 0; q < reps; ++q) run(q);
       CK(cudaEventRecord(e1, s));
       CK(cudaEventSynchronize(e1));
       float ms = 0.f;
       CK(cudaEventElapsedTime(&ms, e0, e1));
       ms /= reps;
+      const bool def = !m->has_robin && variant == fitted.variant && r == fitted.by && ch == fitted.kchunk;
+      if (def) def_ms = ms;
       if (ms < best_ms) {
         best_ms = ms;
         best_cfg = cfg;
@@ -102,6 +135,10 @@ qcad_status autotune(qcad_mesh_s* m, const qcad_bias* b, int precision, int* var
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
+  if (best_ms > (1.0f - FIT_MARGIN) * def_ms) {
+    best_ms = def_ms;
+    best_cfg = fitted;
+  }
   if (precision == 0)
     m->cfg64 = best_cfg;
   else

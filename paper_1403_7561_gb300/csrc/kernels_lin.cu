@@ -61,6 +61,23 @@ static LaunchCfg fit_lin(int nxn, int nyn, int nzn, LaunchCfg cfg) {
   return out;
 }
 
+// The shape that a launch with configuration cfg takes, with an activity map or without.
+template <class T>
+static LaunchCfg lin_shape(int nxn, int nyn, int nzn, LaunchCfg cfg, bool act) {
+  const bool fit = cfg.fit;
+  cfg = fit_lin<T>(nxn, nyn, nzn, cfg);
+  // With an activity map a tile with response takes about six times as long as one without in FP64, so
+  // the longest tile sets the time: half the chunk (FP64 solve of the 128 x 128 x 96 device 75 -> 67 ms;
+  // FP32, bound by latency, was 5 % slower with it).
+  if (sizeof(T) == 8 && fit && cfg.variant >= 2 && act && cfg.kchunk > 8) cfg.kchunk = 8;
+  cfg.fit = false;
+  return cfg;
+}
+LaunchCfg default_lin_shape(int precision, int nxn, int nyn, int nzn, bool act) {
+  return precision == 0 ? lin_shape<double>(nxn, nyn, nzn, LaunchCfg(), act)
+                        : lin_shape<float>(nxn, nyn, nzn, LaunchCfg(), act);
+}
+
 template <class T>
 static bool has_act(const ApplyOp<T>& op) { return op.a.act != nullptr; }
 template <class Op>
@@ -70,11 +87,7 @@ static bool has_act(const Op& op) { return op.v.act != nullptr; }
 // 4/8 x 2 (shared memory). Other requests are clamped to the nearest supported shape.
 template <class T, class Op>
 static void run_lin(const Grid<T>& g, const Op& op, LaunchCfg cfg, cudaStream_t s) {
-  cfg = fit_lin<T>(g.nxn, g.nyn, g.nzn, cfg);
-  // With an activity map a tile with response takes about six times as long as one without in FP64, so
-  // the longest tile sets the time: half the chunk (FP64 solve of the 128 x 128 x 96 device 75 -> 67 ms;
-  // FP32, bound by latency, was 5 % slower with it).
-  if (sizeof(T) == 8 && cfg.fit && cfg.variant >= 2 && has_act(op) && cfg.kchunk > 8) cfg.kchunk = 8;
+  cfg = lin_shape<T>(g.nxn, g.nyn, g.nzn, cfg, has_act(op));
   const int kc = cfg.kchunk > 0 ? (cfg.kchunk < 128 ? cfg.kchunk : 128) : 16;  // LinShape::ZMAX
   const bool two = cfg.variant == 3;
   if constexpr (std::is_same<T, float>::value) {

@@ -103,6 +103,13 @@ struct PcgBufs {
   DevBuf act;  // activity map of c (qcad_internal.cuh)
 };
 
+// Bytes of a PCG vector, a multiple of 16: the second halves of p and d start aligned for the vector
+// loads of the update kernels.
+template <class T>
+size_t vec_bytes(long long n) {
+  return ((size_t)n * sizeof(T) + 79) / 16 * 16;
+}
+
 struct PcgGraph {
   cudaGraphExec_t exec = nullptr;
   const void* key = nullptr;  // vector buffer the graph was captured with

@@ -55,13 +55,6 @@ template <> struct Prec<float> {
   static const int prof_apply = PROF_APPLY32, prof_update = PROF_UPDATE32;
 };
 
-// Bytes of a PCG vector, a multiple of 16: the second halves of p and d start aligned for the vector
-// loads of the update kernels.
-template <class T>
-static size_t vec_bytes(long long n) {
-  return ((size_t)n * sizeof(T) + 79) / 16 * 16;
-}
-
 // Size of a linearization's activity map.
 static size_t act_bytes(const qcad_mesh_s* m) {
   return (size_t)act_cells(m->nx, ACT_X) * act_cells(m->ny, ACT_Y) * act_cells(m->nz, ACT_Z);
@@ -617,6 +610,37 @@ qcad_status poisson_solve(qcad_mesh_s* m, const qcad_bias* b, const qcad_solver_
   if (!phi) throw Error(QCAD_ERR_INVALID_ARG, "null phi");
   if (o->precision == 0) return newton_impl<double>(m, b, o, theta, phi, rep);
   return newton_impl<float>(m, b, o, theta, phi, rep);
+}
+
+// The linearization that the solves at bias b apply, in the mesh's buffers of the precision: at the
+// potential of a coarse Newton solve. False where there is none to time with: no valid bias, or a solve
+// that broke down.
+bool linearize_for_tuning(qcad_mesh_s* m, const qcad_bias* b, int precision) {
+  if (!b || m->has_robin) return false;
+  const bool prof = m->prof.on;
+  m->prof.on = false;  // the profile counts the caller's work
+  bool ok = false;
+  try {
+    validate_bias(m, b);
+    m->scratch.ensure(m->n_nodes * sizeof(double) + 64);
+    double* phi = m->scratch.as<double>();
+    qcad_solver_opts o{};
+    o.precision = 1;
+    o.cheb_degree = DEG_MG;
+    o.newton_tol_R = o.newton_tol_dphi = 1e-3;  // what responds is settled long before the potential
+    o.max_newton = 20;
+    qcad_solve_report rep{};
+    const qcad_status st = newton_impl<float>(m, b, &o, nullptr, phi, &rep);
+    ok = (st == QCAD_OK || st == QCAD_ERR_NOT_CONVERGED) &&
+         std::isfinite(eval_residual(m, make_phys(m, b), phi, nullptr, 0, precision, nullptr).r2);
+  } catch (const Error& e) {
+    if (e.code != QCAD_ERR_INVALID_ARG) {
+      m->prof.on = prof;
+      throw;
+    }
+  }
+  m->prof.on = prof;
+  return ok;
 }
 
 qcad_status poisson_residual(qcad_mesh_s* m, const qcad_bias* b, const double* theta, const double* phi, double* R,

@@ -271,6 +271,8 @@ template <class T>
 void launch_cheb_step_lin(const Grid<T>& g, PcgVecs<T> vecs, PcgScalars* sc, int step, int last, LaunchCfg cfg,
                           cudaStream_t s);
 int lin_blocks_per_sm(int precision, int by, int rows);
+// The default shape of the plane-factorized kernels on a grid, as an explicit configuration.
+LaunchCfg default_lin_shape(int precision, int nxn, int nyn, int nzn, bool act);
 
 // Resident blocks per SM of the Jacobian apply of a precision (0 FP64, 1 FP32) and variant.
 int apply_blocks_per_sm(int precision, int by, int variant);
