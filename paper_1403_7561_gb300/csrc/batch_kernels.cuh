@@ -130,8 +130,10 @@ void launch_batch_residual_2pass(const BatchResEntry* tab, int n_inst, int qp_bl
   note_launch(), batch_clear_act_kernel<<<dim3(4, n_inst), 256, 0, s>>>(tab);
   note_launch(3);
   batch_residual_classify_kernel<<<qp_blocks, 256, 0, s>>>(tab, n_inst);
-  const int db = n_inst < 8 ? sm_count() : 2 * sm_count() * 8 / n_inst;  // density blocks per instance
-  batch_residual_density_kernel<<<dim3(db > 16 ? db : 16, n_inst), 256, 0, s>>>(tab);
+  // density blocks per instance: 16 per SM in all, as many as the density pass of one mesh (8 per SM) at
+  // most; the blocks stride over the lists, whose lengths only the device knows
+  const int all = 16 * sm_count() / n_inst, db = all < 16 ? 16 : all < 8 * sm_count() ? all : 8 * sm_count();
+  batch_residual_density_kernel<<<dim3(db, n_inst), 256, 0, s>>>(tab);
   batch_residual_node_kernel<<<node_blocks, 32 * NODE_WARPS, 0, s>>>(tab, n_inst);
 }
 
