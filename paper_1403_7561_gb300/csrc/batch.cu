@@ -156,7 +156,11 @@ qcad_status poisson_solve_batch_impl(int n, const qcad_mesh_t* ms, const qcad_bi
                                      double* const* phis, qcad_solve_report* reps);
 
 // z-chunk of the batched FP32 apply (plane-factorized, 8 warps, two rows per thread) for one
-// mesh: the fastest of a few lengths, timed on the mesh's own grid.
+// mesh: the fastest of a few lengths, timed on the mesh's own grid with response everywhere. With the map
+// of a solve the mesh alone runs 8 planes fastest up to 111 elements a side, while together with others,
+// whose blocks fill the SMs, it wants longer chunks: Jacobi batches of four meshes of 100 to 112 elements
+// 468 ms with 8 planes, 446 with 16, 442 with 32; of eight of 48 to 112 elements 410, 394, 394. The form
+// without a map picks 16 from 98 elements on and 8 below, the better ones of these.
 static int tune_batch_kchunk(qcad_mesh_s* m) {
   cudaStream_t s = m->stream;
   const long long n = m->n_nodes;
