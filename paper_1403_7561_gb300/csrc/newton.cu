@@ -616,7 +616,7 @@ qcad_status poisson_solve(qcad_mesh_s* m, const qcad_bias* b, const qcad_solver_
 // potential of a coarse Newton solve. False where there is none to time with: no valid bias, or a solve
 // that broke down.
 bool linearize_for_tuning(qcad_mesh_s* m, const qcad_bias* b, int precision) {
-  if (!b || m->has_robin) return false;
+  if (!b || (b->n_gates > 0 && !b->V_gate) || m->has_robin) return false;
   const bool prof = m->prof.on;
   m->prof.on = false;  // the profile counts the caller's work
   bool ok = false;
@@ -629,6 +629,7 @@ bool linearize_for_tuning(qcad_mesh_s* m, const qcad_bias* b, int precision) {
     o.cheb_degree = DEG_MG;
     o.newton_tol_R = o.newton_tol_dphi = 1e-3;  // what responds is settled long before the potential
     o.max_newton = 20;
+    o.max_krylov = 2000;
     qcad_solve_report rep{};
     const qcad_status st = newton_impl<float>(m, b, &o, nullptr, phi, &rep);
     ok = (st == QCAD_OK || st == QCAD_ERR_NOT_CONVERGED) &&

@@ -1,4 +1,6 @@
 """The launch autotuner times the operator that the solves at the given bias run."""
+import ctypes
+
 import pytest
 import torch
 
@@ -42,3 +44,15 @@ def test_solves_after_tuning(q, precision):
         phis.append(phi)
     for phi in phis[1:]:
         assert torch.max(torch.abs(phi - phis[0])).item() <= 1e-9
+
+
+def test_a_bias_that_cannot_be_solved_tunes_as_none(q):
+    # no voltages, no temperature, no bias at all: the shapes are timed with response everywhere
+    dev = W.five_gate_device(n=(37, 33, 21), T=4.0, with_subdomain=False)
+    m = q.qcad_mesh_create(dev)
+    no_voltages, no_temperature = q.make_bias(dev["bias"]), q.make_bias(dict(dev["bias"], T=0.0))
+    no_voltages.V_gate = ctypes.POINTER(ctypes.c_double)()
+    t = ctypes.c_float()
+    for b in (ctypes.byref(no_voltages), ctypes.byref(no_temperature), None):
+        assert q._lib.qcad_autotune(m.handle, b, 1, None, None, None, ctypes.byref(t)) == 0
+        assert t.value > 0
